@@ -12,9 +12,10 @@
 //          squared TSC window (sinc^3 per axis) and by the transform size;
 //   solve: TSC charge assignment (atomics) -> FFT -> product with each kernel
 //          component -> inverse FFT -> TSC interpolation; then a cell list
-//          (cells >= r_cut, stable per-cell order, particles copied in cell
-//          order) and the direct short-range sum with the minimum image along z.
-// FP64 throughout; cuFFT does the transforms.  One sample at a time.
+//          (cells >= r_cut/2 x r_cut/4, stable per-cell order, particles copied in
+//          cell order) and the direct short-range sum with the minimum image along z.
+// FP64 on the mesh (cuFFT does the transforms), float-float for the short-range pairs
+// (pdq_split.cuh).  One sample at a time.
 #include <cufft.h>
 #include <math.h>
 
@@ -23,6 +24,7 @@
 
 #include "pdq_common.cuh"
 #include "pdq_device.cuh"
+#include "pdq_split.cuh"
 
 struct pdq_p3m {
     int device;
@@ -43,9 +45,8 @@ struct pdq_p3m {
     int* cell_start;            // [ncells + 1]
     int* cell_fill;             // [ncells]
     int* cell_list;             // [max_n]
-    double4_32a* sorted64;          // [max_n] live particles in cell order: x, y, z, q
-    double2* lf_tab;                // [kTab + 1] K_L factor and its u-derivative at u = k (alpha r_cut)^2 / kTab
-    float4* sorted32;           // [max_n] the same positions in FP32 (distance pre-filter)
+    float4* sorted;             // [3][max_n] live particles in cell order, split: (x, y, z) hi and q hi, mid and q lo, lo
+    float4* lf_tab;             // [2][kTab] K_L factor by quartics on kTab intervals of u = (alpha r)^2 < (alpha r_cut)^2
     double* sums;               // [sums_cap][3], for the step driver
     int64_t sums_cap;
 };
@@ -56,12 +57,14 @@ namespace {
 struct P3MGeom {
     double R, L, h, hz, x0, alpha, rc, contact;
     int Mx, Nx, Nz, n_img, ncx, ncz;
-    const double2* lf_tab;
+    const float4* lf_tab;
+    SplitGrid grid;             // of the split coordinates
 };
 
-// The short-range pairs read the long-range factor from a cubic Hermite table in
-// u = (alpha r)^2 (relative interpolation error ~1e-13) instead of FP64 erf and exp.
-constexpr int kTab = 4096;
+// The short-range pairs read the long-range factor from quartics in u = (alpha r)^2, one per interval
+// of a table (through 5 Chebyshev nodes each: relative interpolation error ~2e-15 at alpha r_cut = 3.3),
+// instead of erf and exp.  1,024 intervals of 32 B fit shared memory beside the pair queues.
+constexpr int kTab = 1024;
 
 struct P3MPart {                // the particles of one sample, current half of the state
     const void* pos;
@@ -213,6 +216,10 @@ __global__ void k_p3m_interp(const P3MGeom G, const P3MPart S, const double* __r
     sums[3 * g + c] = s;
 }
 
+// Cells are at least r_cut / kReachXY wide across the pipe and r_cut / kReachZ along it, so a particle's
+// neighbours lie at most that many cells away.
+constexpr int kReachXY = 2, kReachZ = 4;
+
 __device__ __forceinline__ int cell_of(const P3MGeom& G, double x, double y, double z) {
     const double wxy = 2.0 * G.R / G.ncx, wz = G.L / G.ncz;
     int cx = (int)floor((x + G.R) / wxy), cy = (int)floor((y + G.R) / wxy), cz = (int)floor(z / wz);
@@ -230,17 +237,21 @@ __global__ void k_cell_count(const P3MGeom G, const P3MPart S, int* count) {
     atomicAdd(&count[cell_of(G, x, y, z)], 1);
 }
 
-// Exclusive scan of the cell counts (one CTA of 1024 threads, chunks in order).
+// Exclusive scan of the cell counts (one CTA of 1024 threads, 8 cells per thread, chunks in order).
 __global__ void __launch_bounds__(1024) k_cell_scan(const int* count, int64_t ncells, int* start) {
-    __shared__ int warp_sum[32];
-    __shared__ int carry;
+    constexpr int E = 8;
+    __shared__ int warp_sum[33];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) carry = 0;
-    __syncthreads();
-    for (int64_t c0 = 0; c0 < ncells; c0 += 1024) {
-        const int64_t c = c0 + tid;
-        const int v = c < ncells ? count[c] : 0;
-        int incl = v;
+    int carry = 0;
+    for (int64_t c0 = 0; c0 < ncells; c0 += 1024 * E) {
+        const int64_t c = c0 + (int64_t)tid * E;
+        int v[E], sum = 0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            v[e] = c + e < ncells ? count[c + e] : 0;
+            sum += v[e];
+        }
+        int incl = sum;
         for (int d = 1; d < 32; d <<= 1) {
             const int t = __shfl_up_sync(0xffffffffu, incl, d);
             if (lane >= d) incl += t;
@@ -248,17 +259,23 @@ __global__ void __launch_bounds__(1024) k_cell_scan(const int* count, int64_t nc
         if (lane == 31) warp_sum[warp] = incl;
         __syncthreads();
         if (warp == 0) {
-            int w = warp_sum[lane], wi = w;
+            const int w = warp_sum[lane];
+            int wi = w;
             for (int d = 1; d < 32; d <<= 1) {
                 const int t = __shfl_up_sync(0xffffffffu, wi, d);
                 if (lane >= d) wi += t;
             }
             warp_sum[lane] = wi - w;
+            if (lane == 31) warp_sum[32] = wi;
         }
         __syncthreads();
-        if (c < ncells) start[c] = carry + warp_sum[warp] + incl - v;
-        __syncthreads();
-        if (tid == 1023) carry += warp_sum[31] + incl;
+        int at = carry + warp_sum[warp] + incl - sum;
+        carry += warp_sum[32];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            if (c + e < ncells) start[c + e] = at;
+            at += v[e];
+        }
         __syncthreads();
     }
     if (tid == 0) start[ncells] = carry;
@@ -286,131 +303,237 @@ __global__ void k_cell_sort(const int* start, int64_t ncells, int* list) {
     }
 }
 
-// Live particles copied in cell order (FP64 and an FP32 copy of the positions).
-__global__ void k_cell_gather(const P3MPart S, const int* start, int64_t ncells, const int* list, double4_32a* s64,
-                              float4* s32) {
+// Live particles copied in cell order, their coordinates and charge split into floats.
+__global__ void k_cell_gather(const P3MGeom G, const P3MPart S, const int* start, int64_t ncells, const int* list,
+                              float4* sorted, int64_t stride) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= start[ncells]) return;
     double x, y, z, q;
     load_particle(S, S.o + list[t], x, y, z, q);
-    s64[t] = make_double4_32a(x, y, z, q);
-    s32[t] = make_float4((float)x, (float)y, (float)z, 0.f);
+    float4 h, m, l;
+    split3(G.grid, x, h.x, m.x, l.x);
+    split3(G.grid, y, h.y, m.y, l.y);
+    split3(G.grid, z, h.z, m.z, l.z);
+    h.w = (float)q;
+    m.w = (float)(q - (double)h.w);
+    l.w = 0.f;
+    sorted[t] = h;
+    sorted[stride + t] = m;
+    sorted[2 * stride + t] = l;
 }
 
-// K_L factor and d/du at u = (alpha r)^2, for the table: the series (2 alpha^3 c / 3)
-// (1 - 3u/5 + 3u^2/14) below u = 2.5e-3, the closed form above.
-__device__ __forceinline__ double2 long_factor_u(double u, double alpha) {
+// K_L factor at u = (alpha r)^2: c alpha^3 sum_m (-1)^m 2 u^m / (m! (2m + 3)) below u = 1 (where the
+// closed form cancels), the closed form above.
+__device__ __forceinline__ double long_factor_u(double u, double alpha) {
     const double c = 1.1283791670955126, a3 = alpha * alpha * alpha;
-    if (u < 2.5e-3) return make_double2((2.0 / 3.0) * c * a3 * (1.0 - 0.6 * u + (3.0 / 14.0) * u * u),
-                                        (2.0 / 3.0) * c * a3 * (-0.6 + (3.0 / 7.0) * u));
-    const double r = sqrt(u) / alpha, e = exp(-u), er = erf(sqrt(u));
-    const double f = er / (r * r * r) - c * alpha * e / (r * r);
-    const double dfdr = -3.0 * er / (r * r * r * r) + 3.0 * c * alpha * e / (r * r * r) + 2.0 * c * a3 * e / r;
-    return make_double2(f, dfdr / (2.0 * r * alpha * alpha));   // d/du = (d/dr) / (2 r alpha^2)
+    if (u < 1.0) {
+        double s = 0.0, t = 1.0;                    // t = (-u)^m / m!
+        for (int m = 0; m < 24; ++m) {
+            s += 2.0 * t / (2 * m + 3);
+            t *= -u / (m + 1);
+        }
+        return c * a3 * s;
+    }
+    const double x = sqrt(u);
+    return a3 * (erf(x) / (u * x) - c * exp(-u) / u);
 }
 
-__global__ void k_lf_table(double alpha, double umax, double2* tab) {
+// One thread per interval: the quartic in t = position inside the interval (0..1) through the five
+// Chebyshev nodes, by divided differences expanded to powers; the two leading coefficients as
+// float-floats.
+__global__ void k_lf_table(double alpha, double umax, float4* tab) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > kTab) return;
-    tab[k] = long_factor_u(umax * k / kTab, alpha);
+    if (k >= kTab) return;
+    double x[5], f[5];
+    for (int i = 0; i < 5; ++i) {
+        x[i] = 0.5 - 0.5 * cos(kPi * (2 * i + 1) / 10.0);
+        f[i] = long_factor_u(umax * (k + x[i]) / kTab, alpha);
+    }
+    for (int j = 1; j < 5; ++j)
+        for (int i = 4; i >= j; --i) f[i] = (f[i] - f[i - 1]) / (x[i] - x[i - j]);
+    double p[5] = {f[4], 0.0, 0.0, 0.0, 0.0};
+    for (int i = 3; i >= 0; --i) {                  // p <- p (t - x_i) + f_i
+        for (int j = 4; j > 0; --j) p[j] = p[j - 1] - x[i] * p[j];
+        p[0] = f[i] - x[i] * p[0];
+    }
+    const float c0 = (float)p[0], c1 = (float)p[1];
+    tab[k] = make_float4(c0, (float)(p[0] - (double)c0), c1, (float)(p[1] - (double)c1));
+    tab[kTab + k] = make_float4((float)p[2], (float)p[3], (float)p[4], 0.f);
 }
 
-__device__ __forceinline__ double long_factor_tab(const P3MGeom& G, double r2) {
-    const double umax = G.alpha * G.alpha * G.rc * G.rc, hu = umax / kTab;
-    const double x = G.alpha * G.alpha * r2 / hu;
-    int k = (int)x;
-    k = k < 0 ? 0 : (k >= kTab ? kTab - 1 : k);
-    const double t = x - k, t2 = t * t, t3 = t2 * t;
-    const double2 a = G.lf_tab[k], b = G.lf_tab[k + 1];
-    return (2.0 * t3 - 3.0 * t2 + 1.0) * a.x + (t3 - 2.0 * t2 + t) * hu * a.y + (-2.0 * t3 + 3.0 * t2) * b.x +
-           (t3 - t2) * hu * b.y;
-}
+// The particle-independent floats of the pair arithmetic.
+struct PPConst {
+    float Lh, Lm, Ll, invL;      // the period, split like a coordinate
+    float rch, rcl, dch, dcl;    // r_cut^2 and d_c^2
+    float kh, kl;                // table intervals per unit r^2
+};
 
-// One short-range pair: q_j (d / max(r, d_c)^3 - K_L(d)) when r < r_cut (FP64).
-__device__ __forceinline__ void pp_pair(const P3MGeom& G, const double4_32a& pi, const double4_32a& pj, double invL,
-                                        double rc2, double dc2, double& sx, double& sy, double& sz) {
-    const double dx = pi.x - pj.x, dy = pi.y - pj.y;
-    double dz = pi.z - pj.z;
-    dz -= G.L * rint(dz * invL);
-    const double r2 = dx * dx + dy * dy + dz * dz;
-    if (!(r2 < rc2)) return;
-    const double ic = rsqrt(fmax(r2, dc2));             // 1 / max(r, d_c)
-    const double f = pj.w * (ic * ic * ic - long_factor_tab(G, r2));
-    sx += f * dx; sy += f * dy; sz += f * dz;
+// One short-range pair: q_j (d / max(r, d_c)^3 - K_L(d)) when r < r_cut, in float-float (~145 FP32
+// operations); added to the float-float sums s, c.
+__device__ __forceinline__ void pp_pair(const PPConst& K, const float4* T, const float4 ih, const float4 im,
+                                        const float4 il, const float4 jh, const float4 jm, const float4 jl, float s[3],
+                                        float c[3]) {
+    float D[3], E[3], R, r;
+    split_diff(ih.x, im.x, il.x, jh.x, jm.x, jl.x, D[0], E[0]);
+    split_diff(ih.y, im.y, il.y, jh.y, jm.y, jl.y, D[1], E[1]);
+    const float dz = __fsub_rn(ih.z, jh.z), n = rintf(dz * K.invL);        // nearest image, n in {-1, 0, 1}
+    two_sum(__fmaf_rn(-n, K.Lh, dz), __fmaf_rn(-n, K.Lm, __fsub_rn(im.z, jm.z)), D[2], E[2]);
+    E[2] = __fadd_rn(E[2], __fmaf_rn(-n, K.Ll, __fsub_rn(il.z, jl.z)));
+    split_norm2(D, E, R, r);
+    if (!(__fadd_rn(__fsub_rn(R, K.rch), __fsub_rn(r, K.rcl)) < 0.f)) return;
+    // K_L factor: interval and position inside it, then the quartic with its last steps in float-float
+    float X, Xe;
+    split_mul(R, r, K.kh, K.kl, X, Xe);
+    int k = (int)X;
+    k = k < kTab ? k : kTab - 1;
+    const float th = __fsub_rn(X, (float)k);
+    const float4 t0 = T[k], t1 = T[kTab + k];
+    const float v = __fmaf_rn(th, __fmaf_rn(th, __fmaf_rn(th, t1.z, t1.y), t1.x), t0.w);    // c1 lo and the rest
+    const float m = __fmul_rn(th, t0.z);
+    float kl, ke;
+    fast_two_sum(t0.x, m, kl, ke);
+    ke = __fadd_rn(__fadd_rn(ke, t0.y),
+                   __fmaf_rn(th, v, __fmaf_rn(Xe, t0.z, __fmaf_rn(th, t0.z, -m))));
+    const bool clamp = __fadd_rn(__fsub_rn(R, K.dch), __fsub_rn(r, K.dcl)) < 0.f;
+    float w, we, g, ge;
+    split_inv_cube(clamp ? K.dch : R, clamp ? K.dcl : r, w, we);
+    two_sum(w, -kl, g, ge);
+    ge = __fadd_rn(ge, __fsub_rn(we, ke));
+    float f, fe;
+    split_mul(g, ge, jh.w, jm.w, f, fe);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        float p, e, u;
+        split_mul(f, fe, D[a], E[a], p, e);
+        two_sum(s[a], p, s[a], u);
+        c[a] = __fadd_rn(c[a], __fadd_rn(u, e));
+    }
 }
 
 // Short-range part: q_j (d / max(r, d_c)^3 - K_L(d)) over j != i closer than r_cut, added to sums.
-// One warp per particle i (cell order): the lanes screen 32 candidates of the 27 neighbour cells
-// at a time in FP32 (r^2 < (r_cut + 1e-3)^2 + 1e-3), the survivors go to a per-warp queue in
-// shared memory, and every 32 queued pairs are evaluated in FP64 with all lanes busy; the lanes'
-// partial sums are reduced in a fixed order.
+// One warp per particle i (cell order).  Cells are r_cut/2 wide across and r_cut/4 along the pipe
+// and a column's cells follow one another, so the candidates are one run of particles (two across the
+// period) in each of at most 25 columns; lane c looks column c's runs up, all at once.  The lanes then
+// screen 32 candidates at a time on the hi parts (r^2 < (r_cut + 1e-3)^2 + 1e-3), the next 32 in
+// flight, the survivors go to a per-warp queue in shared memory, and every 32 queued pairs are
+// evaluated with all lanes busy; the lanes' partial sums (about a dozen pairs each) are reduced in a
+// fixed order.
+// Bound by instruction issue (screening ~1,500 candidates and ~410 pairs of ~190 instructions per
+// particle).  One million particles, mesh 256^3: 7.5 ms; 42.4 ms in FP64 with the Hermite table in
+// global memory (FP64 pipe 87 % busy), 13.6 ms in float-float over the 27 cells of width r_cut.
 constexpr int kPPWarps = 8;
 __global__ void __launch_bounds__(32 * kPPWarps) k_p3m_pp(const P3MGeom G, const P3MPart S, const int* start,
                                                           int64_t ncells, const int* list,
-                                                          const double4_32a* __restrict__ s64,
-                                                          const float4* __restrict__ s32, double* sums) {
+                                                          const float4* __restrict__ sorted, int64_t stride,
+                                                          double* sums) {
+    __shared__ float4 T[2 * kTab];
     __shared__ int queue[kPPWarps][64];
+    for (int k = threadIdx.x; k < 2 * kTab; k += blockDim.x) T[k] = G.lf_tab[k];
+    __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int* qw = queue[w];
     const int n_live = start[ncells];
-    const double rc2 = G.rc * G.rc, dc2 = G.contact * G.contact, invL = 1.0 / G.L;
     const float rcf = (float)G.rc + 1e-3f, rc2f = rcf * rcf + 1e-3f, Lf = (float)G.L, invLf = 1.0f / Lf;
+    PPConst K;
+    {
+        // (the floor keeps d_c^-3 inside FP32's range; it is 1e-10 wall units)
+        const double rc2 = G.rc * G.rc, dc2 = fmax(G.contact * G.contact, 1e-20), kk = kTab / rc2;
+        split3(G.grid, G.L, K.Lh, K.Lm, K.Ll);
+        K.invL = invLf;
+        K.rch = (float)rc2; K.rcl = (float)(rc2 - (double)K.rch);
+        K.dch = (float)dc2; K.dcl = (float)(dc2 - (double)K.dch);
+        K.kh = (float)kk; K.kl = (float)(kk - (double)K.kh);
+    }
     const unsigned lt = (1u << lane) - 1u;
+    const float4 *sh = sorted, *sm = sorted + stride, *sl = sorted + 2 * stride;
+    const float wxy = (float)(2.0 * G.R / G.ncx), Rf = (float)G.R;
     for (int t = blockIdx.x * kPPWarps + w; t < n_live; t += gridDim.x * kPPWarps) {
-        const double4_32a pi = s64[t];
-        const float4 fi = s32[t];
-        const int ci = cell_of(G, pi.x, pi.y, pi.z);
-        const int cz = ci % G.ncz, cy = (ci / G.ncz) % G.ncx, cx = ci / (G.ncz * G.ncx);
-        double sx = 0.0, sy = 0.0, sz = 0.0;
-        int qn = 0;
-        const int nz = G.ncz >= 3 ? 3 : G.ncz;
-        for (int a = cx - 1; a <= cx + 1; ++a) {
-            if (a < 0 || a >= G.ncx) continue;
-            for (int b = cy - 1; b <= cy + 1; ++b) {
-                if (b < 0 || b >= G.ncx) continue;
-                for (int u = 0; u < nz; ++u) {
-                    int cc = G.ncz >= 3 ? cz - 1 + u : u;
-                    if (cc < 0) cc += G.ncz;
-                    if (cc >= G.ncz) cc -= G.ncz;
-                    const int cell = (a * G.ncx + b) * G.ncz + cc;
-                    const int pe = start[cell + 1];
-                    for (int p0 = start[cell]; p0 < pe; p0 += 32) {
-                        const int p = p0 + lane;
-                        bool pass = false;
-                        if (p < pe && p != t) {
-                            const float4 fj = s32[p];
-                            const float ex = fi.x - fj.x, ey = fi.y - fj.y;
-                            float ez = fi.z - fj.z;
-                            ez -= Lf * rintf(ez * invLf);
-                            pass = ex * ex + ey * ey + ez * ez < rc2f;
-                        }
-                        const unsigned m = __ballot_sync(0xffffffffu, pass);
-                        if (pass) qw[qn + __popc(m & lt)] = p;
-                        qn += __popc(m);
-                        __syncwarp();
-                        if (qn >= 32) {
-                            pp_pair(G, pi, s64[qw[lane]], invL, rc2, dc2, sx, sy, sz);
-                            __syncwarp();
-                            if (lane < qn - 32) qw[lane] = qw[32 + lane];
-                            qn -= 32;
-                            __syncwarp();
-                        }
+        const float4 ih = sh[t], im = sm[t], il = sl[t];
+        // column lane of the 5 x 5 around i: its runs [b0, e0) and, across the period, [b1, e1)
+        int b0 = 0, e0 = 0, b1 = 0, e1 = 0;
+        {
+            const int ci = cell_of(G, (double)ih.x + (double)im.x + (double)il.x,
+                                   (double)ih.y + (double)im.y + (double)il.y,
+                                   (double)ih.z + (double)im.z + (double)il.z);
+            const int cz = ci % G.ncz, cy = (ci / G.ncz) % G.ncx, cx = ci / (G.ncz * G.ncx);
+            constexpr int kCols = 2 * kReachXY + 1;
+            const int a = cx + lane / kCols - kReachXY, b = cy + lane % kCols - kReachXY;
+            if (lane < kCols * kCols && a >= 0 && a < G.ncx && b >= 0 && b < G.ncx) {
+                // distance across from i to the column (an edge column reaches outward without end)
+                const float xl = a == 0 ? -INFINITY : a * wxy - Rf, xh = a == G.ncx - 1 ? INFINITY : (a + 1) * wxy - Rf;
+                const float yl = b == 0 ? -INFINITY : b * wxy - Rf, yh = b == G.ncx - 1 ? INFINITY : (b + 1) * wxy - Rf;
+                const float ex = fmaxf(0.f, fmaxf(xl - ih.x, ih.x - xh)), ey = fmaxf(0.f, fmaxf(yl - ih.y, ih.y - yh));
+                if (ex * ex + ey * ey < rc2f) {
+                    const int* st = start + (a * G.ncx + b) * G.ncz;
+                    const int zl = cz - kReachZ, zh = cz + kReachZ + 1;          // cells [zl, zh)
+                    if (zh - zl >= G.ncz) { b0 = st[0]; e0 = st[G.ncz]; }
+                    else {
+                        b0 = st[zl > 0 ? zl : 0];
+                        e0 = st[zh < G.ncz ? zh : G.ncz];
+                        if (zl < 0) { b1 = st[G.ncz + zl]; e1 = st[G.ncz]; }
+                        else if (zh > G.ncz) { b1 = st[0]; e1 = st[zh - G.ncz]; }
                     }
                 }
             }
         }
-        if (lane < qn) pp_pair(G, pi, s64[qw[lane]], invL, rc2, dc2, sx, sy, sz);
+        float s[3] = {0.f, 0.f, 0.f}, c[3] = {0.f, 0.f, 0.f};
+        int qn = 0;
+        auto pair = [&](int p) { pp_pair(K, T, ih, im, il, sh[p], sm[p], sl[p], s, c); };
+        const float4 none = make_float4(1e15f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+            const int bb = half ? b1 : b0, ee = half ? e1 : e0;
+            unsigned cols = __ballot_sync(0xffffffffu, bb < ee);
+            int p = 0, pe = 0;
+            // the next 32 candidates: on in the run, or the first of the next column's
+            auto advance = [&]() -> bool {
+                p += 32;
+                if (p - lane < pe) return true;
+                if (!cols) return false;
+                const int src = __ffs(cols) - 1;
+                cols &= cols - 1;
+                p = __shfl_sync(0xffffffffu, bb, src) + lane;
+                pe = __shfl_sync(0xffffffffu, ee, src);
+                return true;
+            };
+            bool more = advance();
+            float4 fj = more && p < pe && p != t ? sh[p] : none;
+            while (more) {
+                const int pc = p;
+                const float4 fc = fj;
+                more = advance();
+                fj = more && p < pe && p != t ? sh[p] : none;
+                const float ex = ih.x - fc.x, ey = ih.y - fc.y;
+                float ez = ih.z - fc.z;
+                ez -= Lf * rintf(ez * invLf);
+                const bool pass = ex * ex + ey * ey + ez * ez < rc2f;
+                const unsigned m = __ballot_sync(0xffffffffu, pass);
+                if (pass) qw[qn + __popc(m & lt)] = pc;
+                qn += __popc(m);
+                __syncwarp();
+                if (qn >= 32) {
+                    pair(qw[lane]);
+                    __syncwarp();
+                    if (lane < qn - 32) qw[lane] = qw[32 + lane];
+                    qn -= 32;
+                    __syncwarp();
+                }
+            }
+        }
+        if (lane < qn) pair(qw[lane]);
         __syncwarp();
         for (int d = 16; d > 0; d >>= 1) {
-            sx += __shfl_xor_sync(0xffffffffu, sx, d);
-            sy += __shfl_xor_sync(0xffffffffu, sy, d);
-            sz += __shfl_xor_sync(0xffffffffu, sz, d);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const float os = __shfl_xor_sync(0xffffffffu, s[a], d), oc = __shfl_xor_sync(0xffffffffu, c[a], d);
+                float u;
+                two_sum(s[a], os, s[a], u);
+                c[a] = __fadd_rn(__fadd_rn(c[a], oc), u);
+            }
         }
         if (lane == 0) {
             const int64_t gi = S.o + list[t];
-            sums[3 * gi] += sx;
-            sums[3 * gi + 1] += sy;
-            sums[3 * gi + 2] += sz;
+            for (int a = 0; a < 3; ++a) sums[3 * gi + a] += (double)s[a] + (double)c[a];
         }
     }
 }
@@ -425,6 +548,7 @@ P3MGeom geom_of(const pdq_p3m* P, double contact) {
     G.contact = contact; G.Mx = P->Mx; G.Nx = P->Nx; G.Nz = P->Nz; G.n_img = P->n_img;
     G.ncx = P->ncx; G.ncz = P->ncz;
     G.lf_tab = P->lf_tab;
+    G.grid = split_grid(std::max(P->R, P->L));
     return G;
 }
 
@@ -434,7 +558,7 @@ void free_plan(pdq_p3m* P) {
     if (P->have_inv) cufftDestroy(P->inv);
     cudaFree(P->Gh); cudaFree(P->Q); cudaFree(P->Qh); cudaFree(P->Ah); cudaFree(P->A);
     cudaFree(P->cell_count); cudaFree(P->cell_start); cudaFree(P->cell_fill); cudaFree(P->cell_list);
-    cudaFree(P->sorted64); cudaFree(P->sorted32); cudaFree(P->lf_tab);
+    cudaFree(P->sorted); cudaFree(P->lf_tab);
     cudaFree(P->sums);
     delete P;
 }
@@ -469,8 +593,8 @@ extern "C" int pdq_p3m_create(const pdq_field* field, const pdq_p3m_desc* d, int
     if (!(P->rc < 0.5 * P->L)) { delete P; return PDQ_ERR_INVALID_ARG; }
     P->nreal = (size_t)P->Nx * P->Nx * P->Nz;
     P->ncplx = (size_t)P->Nx * P->Nx * (P->Nz / 2 + 1);
-    P->ncx = std::max(1, (int)floor(2.0 * P->R / P->rc));
-    P->ncz = std::max(1, (int)floor(P->L / P->rc));
+    P->ncx = std::max(1, (int)std::min(128.0, floor(2.0 * P->R * kReachXY / P->rc)));
+    P->ncz = std::max(1, (int)std::min(512.0, floor(P->L * kReachZ / P->rc)));
     P->ncells = (int64_t)P->ncx * P->ncx * P->ncz;
     cudaStream_t s = (cudaStream_t)stream;
     int rc = PDQ_OK;
@@ -487,9 +611,8 @@ extern "C" int pdq_p3m_create(const pdq_field* field, const pdq_p3m_desc* d, int
     alloc((void**)&P->cell_start, (P->ncells + 1) * sizeof(int));
     alloc((void**)&P->cell_fill, P->ncells * sizeof(int));
     alloc((void**)&P->cell_list, P->max_n * sizeof(int));
-    alloc((void**)&P->sorted64, P->max_n * sizeof(double4_32a));
-    alloc((void**)&P->sorted32, P->max_n * sizeof(float4));
-    alloc((void**)&P->lf_tab, (kTab + 1) * sizeof(double2));
+    alloc((void**)&P->sorted, 3 * P->max_n * sizeof(float4));
+    alloc((void**)&P->lf_tab, 2 * kTab * sizeof(float4));
     alloc((void**)&Gr, 3 * P->nreal * sizeof(double));
     if (rc == PDQ_OK) rc = cufft_status(cufftPlan3d(&P->fwd, P->Nx, P->Nx, P->Nz, CUFFT_D2Z));
     if (rc == PDQ_OK) P->have_fwd = true;
@@ -499,7 +622,7 @@ extern "C" int pdq_p3m_create(const pdq_field* field, const pdq_p3m_desc* d, int
     if (rc == PDQ_OK) {
         const P3MGeom G = geom_of(P, 0.0);
         k_p3m_kernel<<<grid_of(P->nreal, 256), 256, 0, s>>>(G, Gr, Gr + P->nreal, Gr + 2 * P->nreal);
-        k_lf_table<<<grid_of(kTab + 1, 256), 256, 0, s>>>(P->alpha, P->alpha * P->alpha * P->rc * P->rc, P->lf_tab);
+        k_lf_table<<<grid_of(kTab, 128), 128, 0, s>>>(P->alpha, P->alpha * P->alpha * P->rc * P->rc, P->lf_tab);
         for (int c = 0; c < 3 && rc == PDQ_OK; ++c)
             rc = cufft_status(cufftExecD2Z(P->fwd, Gr + c * P->nreal, P->Gh + c * P->ncplx));
         if (rc == PDQ_OK) k_p3m_deconv<<<grid_of(P->ncplx, 256), 256, 0, s>>>(G, P->Gh, (int64_t)P->ncplx);
@@ -571,9 +694,9 @@ extern "C" int pdq_p3m_coulomb(pdq_p3m* P, const pdq_phys* phys, const pdq_state
         k_cell_scan<<<1, 1024, 0, s>>>(P->cell_count, P->ncells, P->cell_start);
         k_cell_fill<<<gp, 256, 0, s>>>(G, S, P->cell_start, P->cell_fill, P->cell_list);
         k_cell_sort<<<grid_of(P->ncells, 128), 128, 0, s>>>(P->cell_start, P->ncells, P->cell_list);
-        k_cell_gather<<<gp, 256, 0, s>>>(S, P->cell_start, P->ncells, P->cell_list, P->sorted64, P->sorted32);
+        k_cell_gather<<<gp, 256, 0, s>>>(G, S, P->cell_start, P->ncells, P->cell_list, P->sorted, P->max_n);
         k_p3m_pp<<<(unsigned)std::min<int64_t>(grid_of(S.n, kPPWarps), 16 * 152), 32 * kPPWarps, 0, s>>>(
-            G, S, P->cell_start, P->ncells, P->cell_list, P->sorted64, P->sorted32, sums);
+            G, S, P->cell_start, P->ncells, P->cell_list, P->sorted, P->max_n, sums);
     }
     PDQ_CUDA(cudaGetLastError());
     return PDQ_OK;

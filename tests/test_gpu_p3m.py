@@ -126,6 +126,34 @@ def test_p3m_sums_mixed_state(pdq, setup):
     assert np.max(np.abs(got - want)) <= 1e-9 * _rms(want)
 
 
+@pytest.mark.parametrize("seam", [False, True])
+@pytest.mark.parametrize("at", ["contact", "table", "cut"])
+def test_p3m_short_range_pairs_at_their_edges(pdq, setup, at, seam):
+    # pairs alone in a sample: at and around the clamp d_c (a coincident pair too), on the edges of the
+    # long-range table's intervals, and just inside and outside r_cut; along x and across the period.
+    # Bar as above: the float-float pair (2^-46) and the table (2e-15) sit far below it, the mesh part
+    # differs by the ordering of the transforms
+    f, of, grid, plan, d, Gh = setup
+    dc = oracle.class_table(ST3)[:, 1].max()
+    r = {"contact": dc * np.array([0.0, 1e-3, 0.5, 1 - 1e-12, 1.0, 1 + 1e-12, 1.5]),
+         "table": plan.r_cut * np.sqrt(np.array([1, 2, 511, 1023]) / 1024.0 * (1 + 1e-15)),
+         "cut": plan.r_cut * np.array([1 - 1e-3, 1 - 1e-10, 1 + 1e-10, 1 + 1e-3])}[at]
+    n = len(r)
+    x, y, z = np.zeros(2 * n), np.full(2 * n, 17.25), np.full(2 * n, 0.03125)
+    if seam:      # the second particle a distance r below z = 0, wrapped
+        z[1::2] = np.mod(z[1::2] - r, 720.0)
+    else:
+        x[0::2], x[1::2] = 100.0, 100.0 - r
+    q = np.tile([0.7, -0.4], n)
+    ids = np.tile([0, 1], n).astype(np.int32)
+    st = _state(pdq, 0, [2] * n, (x, y, z, q, np.zeros((2 * n, 3)), np.full(2 * n, 2, np.int32), ids))
+    got = plan.coulomb(pdq.phys_default(), st).cpu().numpy()
+    want = _ref_sums(d, Gh, [2] * n, x, y, z, q)
+    assert np.all(np.isfinite(got))
+    scale = np.maximum(np.abs(want).reshape(n, 6).max(1), _rms(want) * 1e-3).repeat(2)[:, None]
+    assert np.max(np.abs(got - want) / scale) <= 1e-9
+
+
 @pytest.mark.parametrize("block", [64, 256])
 def test_p3m_step_matches_oracle(pdq, setup, block):
     # the P3M step = the oracle's step with the reference P3M sums of each step's start state
