@@ -60,6 +60,28 @@ __device__ __forceinline__ ZClass zclass(float alo, float ahi, float blo, float 
     return t;
 }
 
+// How a Newton-pair launch over S samples of `capacity` particles in all is cut, for CTAs of NT threads
+// of which `slots` run at once: U particles per thread and parts per tile.  A tile of a large batch is
+// taken whole with u_max (12) per thread.  When the heaviest item (a sample's first tile, ~NT U N pairs)
+// is not small against the work per slot, S N^2 / 2 / slots, the launch would end on a few CTAs or leave
+// SMs idle: the tile then narrows until its diagonal block, (NT U)^2 / 2 pairs on one CTA, is at most
+// a slot's share, and its later particles are cut into parts so that each slot gets kNewtonItems of the
+// heaviest kind.  (Narrow tiles share a step's shared loads and shuffles among fewer packed pairs, so
+// wide ones are kept as long as they fit.)
+struct NewtonCut { int U, parts; };
+constexpr double kNewtonItems = 4.0;
+inline NewtonCut newton_cut(int64_t capacity, int64_t S, int NT, int64_t slots, int u_max) {
+    const double n = (double)capacity / (double)(S > 0 ? S : 1);          // mean particles per sample
+    const double share = (double)capacity * n / (double)slots;            // twice a slot's pairs
+    NewtonCut c{u_max, 1};
+    if (share >= 2.0 * kNewtonItems * NT * u_max * n) return c;
+    while (c.U > 4 && (double)(NT * c.U) * (NT * c.U) > share) c.U -= 4;
+    const double want = 2.0 * kNewtonItems * NT * c.U * n / (share > 0.0 ? share : 1.0);
+    const double tiles = floor(n / NT) + 1.0;                              // j-tiles of a mean sample
+    c.parts = 1 + (int)fmax(1.0, fmin(ceil(want), tiles));
+    return c;
+}
+
 // Coulomb sums of one i-tile: particles [base, base + NT*U) of a sample ending at `end`, paired
 // with every particle of the sample from `base` on, added into acc (x, y, z; w untouched).
 // Warp w holds the i-particles [32 U w, 32 U (w + 1)) of the tile (lane l: 32 k + l, k < U), a
@@ -81,12 +103,14 @@ __device__ __forceinline__ ZClass zclass(float alo, float ahi, float blo, float 
 //   - The later particles: Newton pairs by j-tiles of NT staged by the whole CTA; the per-warp
 //     j-side sums of a tile are added in shared memory and leave with one float4 atomic per j.
 // The earlier particles of the sample reach this tile as the j side of earlier tiles.
+// With CUT the tile's work is cut over `parts` > 1 CTAs: part 0 does the diagonal block, part
+// p >= 1 the p-th of parts - 1 equal runs of j-tiles of the later particles (newton_parts says when).
 // load(g) gives particle g as (x, y, z, q).  Padding particles sit far off the axis
 // (x = +-1e15) with zero charge, so they add nothing.  All threads of the CTA take part; the
 // shared arrays are the calling kernel's (one set per kernel instantiation).
-template <int NT, int U, class Load>
+template <int NT, int U, bool CUT = false, class Load>
 __device__ __forceinline__ void newton_tile(const Load& load, int64_t base, int64_t end, float Lf, float invL,
-                                            float c2, float4* __restrict__ acc) {
+                                            float c2, float4* __restrict__ acc, int part = 0, int parts = 1) {
     constexpr int W = NT / 32, H = U / 2;
     static_assert(U % 4 == 0 && NT % 32 == 0, "packed pairs over whole warps, an even number of them");
     // the staged j particles pre-duplicated, (x,x,y,y) in sxy, (z,z,q,q) in szq and (z-L,z-L,q,q) in
@@ -110,7 +134,16 @@ __device__ __forceinline__ void newton_tile(const Load& load, int64_t base, int6
     const float kPadI = 1e15f, kPadJ = -1e15f;
     const int n = (int)(end - base);                 // particles of the sample from base on
     const int nd = n < NT * U ? n : NT * U;          // the diagonal block
-    for (int t = tid; t < 3 * NT * U; t += NT) (&s_dj[0][0])[t] = 0.f;
+    const bool diag = !CUT || part == 0;
+    int jb = nd, je = n;                             // the later particles of this part
+    if constexpr (CUT) {
+        const int per = ((n - nd + NT - 1) / NT + parts - 2) / (parts - 1) * NT;
+        jb = diag ? n : nd + (part - 1) * per;
+        je = diag || jb + per > n ? n : jb + per;
+        if (!diag && jb >= je) return;               // uniform across the CTA
+    }
+    if (diag)
+        for (int t = tid; t < 3 * NT * U; t += NT) (&s_dj[0][0])[t] = 0.f;
     f2 X[H], Y[H], Z[H], NQ[H], AX[H], AY[H], AZ[H];
     float ilo = INFINITY, ihi = -INFINITY;
 #pragma unroll
@@ -188,7 +221,7 @@ __device__ __forceinline__ void newton_tile(const Load& load, int64_t base, int6
     // B_{w+W/2} with all its packed pairs, warp w >= W/2 the 2H groups of B_{w-W/2} with its
     // packed pairs h >= H/2 (the last H groups of B_w).  Every warp issues the same number of pair
     // evaluations; within a pass all its packed pairs take part.
-    {
+    if (diag) {
         constexpr int DN = (W - 1) / 2, NP0 = 2 * H, NP1 = NP0 + 2 * H * DN;
         constexpr int NPW = NP1 + ((W % 2 == 0) ? 2 * H : 0);
         const int ngd = (nd + 31) >> 5;                                   // 32-groups with particles
@@ -283,10 +316,10 @@ __device__ __forceinline__ void newton_tile(const Load& load, int64_t base, int6
 
     // ---- Newton pairs with the later particles, by j-tiles of NT (the next tile's particle in
     // flight during a tile) ----
-    float4 pj = nd + tid < n ? load(base + nd + tid) : make_float4(kPadJ, 0.f, 0.f, 0.f);
-    for (int j0 = nd; j0 < n; j0 += NT) {
+    float4 pj = jb + tid < je ? load(base + jb + tid) : make_float4(kPadJ, 0.f, 0.f, 0.f);
+    for (int j0 = jb; j0 < je; j0 += NT) {
         const int j = j0 + tid;
-        float jlo = j < n ? pj.z : INFINITY, jhi = j < n ? pj.z : -INFINITY;
+        float jlo = j < je ? pj.z : INFINITY, jhi = j < je ? pj.z : -INFINITY;
         for (int d = 16; d > 0; d >>= 1) {
             jlo = fminf(jlo, __shfl_xor_sync(0xffffffffu, jlo, d));
             jhi = fmaxf(jhi, __shfl_xor_sync(0xffffffffu, jhi, d));
@@ -303,7 +336,7 @@ __device__ __forceinline__ void newton_tile(const Load& load, int64_t base, int6
             szm[e] = vzm; szm[e + 32] = vzm;
         }
         __syncthreads();
-        const float4 pnext = j + NT < n ? load(base + j + NT) : make_float4(kPadJ, 0.f, 0.f, 0.f);
+        const float4 pnext = j + NT < je ? load(base + j + NT) : make_float4(kPadJ, 0.f, 0.f, 0.f);
 #pragma unroll 1
         for (int g = 0; g < W; ++g) {
             f2 JX, JY, JZ;
@@ -314,7 +347,7 @@ __device__ __forceinline__ void newton_tile(const Load& load, int64_t base, int6
             f2_unpack(JZ, l0, l1); s_jacc[warp][2][g * 32 + lane] = l0 + l1;
         }
         __syncthreads();
-        if (j < n) {
+        if (j < je) {
             float sx = 0.f, sy = 0.f, sz = 0.f;
 #pragma unroll
             for (int w = 0; w < W; ++w) { sx += s_jacc[w][0][tid]; sy += s_jacc[w][1][tid]; sz += s_jacc[w][2][tid]; }
@@ -329,8 +362,12 @@ __device__ __forceinline__ void newton_tile(const Load& load, int64_t base, int6
         f2_unpack(AY[h], a0[1], a1[1]);
         f2_unpack(AZ[h], a0[2], a1[2]);
         const int g0 = warp * (32 * U) + (2 * h) * 32 + lane, g1 = g0 + 32;
-        if (g0 < n) atomicAdd(&acc[base + g0], make_float4(a0[0] + s_dj[0][g0], a0[1] + s_dj[1][g0], a0[2] + s_dj[2][g0], 0.f));
-        if (g1 < n) atomicAdd(&acc[base + g1], make_float4(a1[0] + s_dj[0][g1], a1[1] + s_dj[1][g1], a1[2] + s_dj[2][g1], 0.f));
+        if (diag) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) { a0[k] += s_dj[k][g0]; a1[k] += s_dj[k][g1]; }
+        }
+        if (g0 < n) atomicAdd(&acc[base + g0], make_float4(a0[0], a0[1], a0[2], 0.f));
+        if (g1 < n) atomicAdd(&acc[base + g1], make_float4(a1[0], a1[1], a1[2], 0.f));
     }
 }
 

@@ -193,6 +193,8 @@ struct StepArgs {
     // k_pairs_sym64 and passed to the given-sums step as ext
     float4* acc4;
     double* acc64;
+    // MIXED pair variant 3: particles per thread of k_pairs_sym and CTAs per tile (newton_cut)
+    int newton_u, newton_parts;
     // host only: upper bound on the work items of a launch (the persistent grid is capped by it,
     // so that few items spread one per CTA over the SMs instead of piling onto the first CTAs)
     int64_t max_items;
@@ -996,10 +998,11 @@ __global__ void __launch_bounds__(NT, ((V == 4 || V == 6) && P == PDQ_MIXED) ? 6
 // over a queue measured ~5 more register moves per packed pair evaluation in the hot loop.
 // Each CTA sums its tile's pairs with newton_tile (Newton pairs between the warps' blocks of the
 // tile and with every later particle of the sample; one-sided only within a warp's block).
+// Small batches: gridDim.y parts per tile, part 0 the diagonal block (see newton_cut).
 // Register budget: 3 CTAs of 128 threads per SM (168 registers) for 12 particles per thread (8 per
 // thread ran 1 % faster at 4 CTAs and 128 registers than at 3), 6 CTAs of 64.
-template <int NT, int U>
-__global__ void __launch_bounds__(NT, NT == 128 ? 3 : 6) k_pairs_sym(const StepArgs A) {
+template <int NT, int U, bool CUT>
+__global__ void __launch_bounds__(NT, (U == 12 ? 3 : U == 8 ? 4 : 5) * (128 / NT)) k_pairs_sym(const StepArgs A) {
     const int item = blockIdx.x;
     if (item >= A.ctl[CTL_NITEMS]) return;
     const float4* __restrict__ pos_in = (const float4*)A.pos_in;
@@ -1008,8 +1011,10 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 3 : 6) k_pairs_sym(const StepA
     const int64_t o = A.offset[it.x];
     const int64_t end = o + A.count[it.x];
     const int64_t base = o + (int64_t)it.y * (NT * U);
-    newton_tile<NT, U>(load, base, end, (float)A.K.L, (float)A.K.invL, (float)A.K.contact2f, A.acc4);
+    newton_tile<NT, U, CUT>(load, base, end, (float)A.K.L, (float)A.K.invL, (float)A.K.contact2f, A.acc4, blockIdx.y,
+                            gridDim.y);
 }
+
 
 // FP64 Newton pair: coulomb_pair_x2_sym for one i-particle in double (minimum image by the
 // 1.5 * 2^52 rounding constant, as the one-sided FP64 pair).
@@ -1474,17 +1479,6 @@ static int tile_threads(const pdq_state* st, const pdq_step_cfg* cfg) {
 static bool newton_pairs(const pdq_state* st, const pdq_step_cfg* cfg) {
     return cfg && cfg->variant == 3 && (!(cfg->forces & PDQ_F_CONTACT) || st->precision == PDQ_MIXED);
 }
-// particles per thread: FP64 1 (2 for its Newton-pair kernel); MIXED 4 (two packed pairs), 8 for
-// pair variant 2, 12 for pair variant 3 (8 with contact forces: their update runs 4 per thread
-// over 2 NT threads); 12 gave 1.2 % over 8 (six packed calls share each step's shared loads and
-// shuffles) at 3 CTAs of 128 threads per SM
-static int tile_ilp(const pdq_state* st, const pdq_step_cfg* cfg = nullptr) {
-    if (st->precision == PDQ_FP64) return newton_pairs(st, cfg) ? 2 : 1;
-    if (newton_pairs(st, cfg)) return (cfg->forces & PDQ_F_CONTACT) ? 8 : 12;
-    if (cfg && (cfg->forces & PDQ_F_CONTACT)) return 4;      // contact runs: variant 0 layout
-    return (cfg && cfg->variant == 2) ? 8 : 4;
-}
-
 static int sm_count() {
     static int n = 0;
     if (!n) {
@@ -1494,6 +1488,22 @@ static int sm_count() {
         if (n <= 0) n = 1;
     }
     return n;
+}
+
+// The cut of a MIXED Newton-pair launch (3 CTAs of 128 threads, or 6 of 64, run per SM).
+static NewtonCut mixed_cut(const pdq_state* st, const pdq_step_cfg* cfg) {
+    const int NT = tile_threads(st, cfg), u_max = (cfg->forces & PDQ_F_CONTACT) ? 8 : 12;
+    return newton_cut(st->capacity, st->n_samples, NT, (int64_t)sm_count() * (3 * 128 / NT > 0 ? 3 * 128 / NT : 1), u_max);
+}
+// particles per thread: FP64 1 (2 for its Newton-pair kernel); MIXED 4 (two packed pairs), 8 for
+// pair variant 2, for pair variant 3 as newton_cut says: 12 in large batches (8 with contact forces:
+// their update runs 4 per thread over 2 NT threads); 12 gave 1.2 % over 8 (six packed calls share each
+// step's shared loads and shuffles) at 3 CTAs of 128 threads per SM
+static int tile_ilp(const pdq_state* st, const pdq_step_cfg* cfg = nullptr) {
+    if (st->precision == PDQ_FP64) return newton_pairs(st, cfg) ? 2 : 1;
+    if (newton_pairs(st, cfg)) return mixed_cut(st, cfg).U;
+    if (cfg && (cfg->forces & PDQ_F_CONTACT)) return 4;      // contact runs: variant 0 layout
+    return (cfg && cfg->variant == 2) ? 8 : 4;
 }
 
 template <int P, int NT, int U, int V>
@@ -1509,9 +1519,7 @@ static int launch_step(const StepArgs& A, cudaStream_t s) {
     return PDQ_OK;
 }
 
-// Pair variant 3: the Newton-pair sums (NT threads, 12 particles per thread) into A.acc4, then
-// the given-sums step over the same tiles (2 NT threads, 6 particles per thread; with contact forces
-// the sums take 8 per thread and the contact variant 4 per thread over 2 NT threads).
+// Pair variant 3 in FP64: the Newton-pair sums into A.acc64, then the given-sums step.
 template <int NT>
 static int launch_newton64(const StepArgs& A, cudaStream_t s) {
     static int per_sm = 0;
@@ -1529,21 +1537,24 @@ static int launch_newton64(const StepArgs& A, cudaStream_t s) {
     B.ext = A.acc64;
     return launch_step<PDQ_FP64, 2 * NT, 1, 5>(B, s);
 }
-// MIXED contact runs under pair variant 3: the Newton-pair sums, then the contact variant of the
-// step that takes them from A.acc4 (V = 6) over the same tiles.
-template <int NT>
-static int launch_newton_contact(const StepArgs& A, cudaStream_t s) {
+// MIXED: the Newton-pair sums into A.acc4, then the step that takes them over the same tiles (2 NT
+// threads, half as many particles per thread): the given-sums update, or with contact forces the
+// contact variant (V = 6).
+template <int NT, int U, bool CONTACT>
+static int launch_newton_u(const StepArgs& A, cudaStream_t s) {
     PDQ_CUDA(cudaMemsetAsync(A.acc4, 0, sizeof(float4) * (size_t)(A.cap > 0 ? A.cap : 1), s));
-    if (A.K.forces & PDQ_F_COULOMB)      // the sums enter the update only with the Coulomb force on
-        k_pairs_sym<NT, 8><<<(unsigned)std::max<int64_t>(1, A.max_items), NT, 0, s>>>(A);
-    return launch_step<PDQ_MIXED, 2 * NT, 4, 6>(A, s);
+    if (A.K.forces & PDQ_F_COULOMB) {    // the sums enter the update only with the Coulomb force on
+        const dim3 grid((unsigned)std::max<int64_t>(1, A.max_items), (unsigned)A.newton_parts);
+        if (A.newton_parts > 1) k_pairs_sym<NT, U, true><<<grid, NT, 0, s>>>(A);
+        else k_pairs_sym<NT, U, false><<<grid, NT, 0, s>>>(A);
+    }
+    return launch_step<PDQ_MIXED, 2 * NT, U / 2, CONTACT ? 6 : 5>(A, s);
 }
 template <int NT>
-static int launch_newton(const StepArgs& A, cudaStream_t s) {
-    PDQ_CUDA(cudaMemsetAsync(A.acc4, 0, sizeof(float4) * (size_t)(A.cap > 0 ? A.cap : 1), s));
-    if (A.K.forces & PDQ_F_COULOMB)      // the sums enter the update only with the Coulomb force on
-        k_pairs_sym<NT, 12><<<(unsigned)std::max<int64_t>(1, A.max_items), NT, 0, s>>>(A);
-    return launch_step<PDQ_MIXED, 2 * NT, 6, 5>(A, s);
+static int launch_newton(const StepArgs& A, bool contact, cudaStream_t s) {
+    if (contact) return A.newton_u == 8 ? launch_newton_u<NT, 8, true>(A, s) : launch_newton_u<NT, 4, true>(A, s);
+    if (A.newton_u == 12) return launch_newton_u<NT, 12, false>(A, s);
+    return A.newton_u == 8 ? launch_newton_u<NT, 8, false>(A, s) : launch_newton_u<NT, 4, false>(A, s);
 }
 
 // variant: MIXED pair math, 0 = all packed f32x2, 1 = packed with scalar accumulation,
@@ -1553,8 +1564,8 @@ static int launch_newton(const StepArgs& A, cudaStream_t s) {
 // Coulomb sums (A.ext, P3M): V = 5, no pair loop.
 static int dispatch_step(int prec, int NT, int variant, bool contact, const StepArgs& A, cudaStream_t s) {
     if (A.acc4) {
-        if (NT == 64) return contact ? launch_newton_contact<64>(A, s) : launch_newton<64>(A, s);
-        if (NT == 128) return contact ? launch_newton_contact<128>(A, s) : launch_newton<128>(A, s);
+        if (NT == 64) return launch_newton<64>(A, contact, s);
+        if (NT == 128) return launch_newton<128>(A, contact, s);
         return PDQ_ERR_INVALID_ARG;
     }
     if (A.acc64) {
@@ -1807,12 +1818,23 @@ int step_impl(const pdq_field* field, const pdq_phys* phys, pdq_state* st, const
         return PDQ_ERR_INVALID_ARG;
     if (ext && (contact || cfg->use_graph)) return PDQ_ERR_INVALID_ARG;
     const int NT = tile_threads(st, cfg);
-    const int U = ext ? (st->precision == PDQ_FP64 ? 1 : 4) : tile_ilp(st, cfg);   // given sums: 4 per thread
+    int U = ext ? (st->precision == PDQ_FP64 ? 1 : 4) : tile_ilp(st, cfg);   // given sums: 4 per thread
+    NewtonCut cut{U, 1};
     if (NT != 64 && NT != 128 && NT != 256 && !(NT == 32 && st->precision == PDQ_FP64)) return PDQ_ERR_INVALID_ARG;
     const bool newton = !ext && newton_pairs(st, cfg);
     if (newton && NT != 64 && NT != 128) return PDQ_ERR_INVALID_ARG;   // its update step runs 2 NT threads
     size_t items_bytes, need, cnt_off = 0, part_off = 0, acc_off = 0;
     workspace_layout(st, NT * U, &items_bytes, &need, &cnt_off, &part_off, contact, &acc_off, newton);
+    if (newton && st->precision == PDQ_MIXED) {
+        cut = mixed_cut(st, cfg);
+        // a workspace that only fits the item table of whole, wide tiles takes those
+        const int wide = contact ? 8 : 12;
+        if (workspace_bytes < need && U < wide) {
+            U = wide;
+            cut = NewtonCut{wide, 1};
+            workspace_layout(st, NT * U, &items_bytes, &need, &cnt_off, &part_off, contact, &acc_off, newton);
+        }
+    }
     if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255)) return PDQ_ERR_WORKSPACE;
     const int JS = newton ? newton_chunks(st, NT * U) : j_split(st, NT * U, contact || ext);
     if (n_steps == 0) return PDQ_OK;
@@ -1837,6 +1859,8 @@ int step_impl(const pdq_field* field, const pdq_phys* phys, pdq_state* st, const
     A.n_dep = (unsigned long long*)tally->n_dep; A.n_alive = (unsigned long long*)tally->n_alive;
     A.jsplit = JS;
     A.cap = st->capacity;
+    A.newton_u = cut.U;
+    A.newton_parts = cut.parts;
     A.ext = ext;
     if (newton && st->precision == PDQ_MIXED) A.acc4 = (float4*)((char*)workspace + acc_off);
     if (newton && st->precision == PDQ_FP64) A.acc64 = (double*)((char*)workspace + acc_off);

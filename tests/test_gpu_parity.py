@@ -309,6 +309,17 @@ def test_fp64_lognormal_charge_parity(pdq, fields):
     _compare_by_id(st, ost, np.r_[0, np.cumsum(counts)], 1e-9, 1e-9)
 
 
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("counts", [[1], [513, 4096, 0], [1500] * 5, [129] * 40, [9000, 30]])
+def test_mixed_newton_pairs_cut_tiles(pdq, fields, counts, block):
+    # small batches: narrow tiles whose later particles are cut over several work items (one part, parts
+    # without particles, a partial last j-tile); three steps, the MIXED bars of this file
+    prm = np.tile(PRM3, (len(counts) // 3 + 1, 1))[:len(counts)]
+    st, tally, ost, nd, na = _run_both(pdq, fields, 1, counts, ST3, prm, 3, {"variant": 3}, block=block)
+    assert _compare_by_id(st, ost, np.r_[0, np.cumsum(counts)], 2e-6, 2e-5, max_flip=0.005) > 0
+
+
+
 @pytest.mark.parametrize("variant,block", [(0, 0), (3, 64), (3, 128)])
 def test_mixed_parity(pdq, fields, variant, block):
     # FP32 pair sum / interpolation / velocities, FP64 wall-normal position; variant 3 evaluates
