@@ -32,13 +32,14 @@ struct pdq_p3m {
     int M, Mx, Nx, Nz, n_img;
     int64_t max_n;
     size_t nreal, ncplx;
-    cufftHandle fwd, inv;
-    bool have_fwd, have_inv;
+    size_t nhalf;               // real nodes of the Mx planes the charges reach
+    cufftHandle fwd, lines, inv;     // planes (y, z) real to complex, lines along x, planes back
+    bool have_fwd, have_lines, have_inv;
     cufftDoubleComplex* Gh;     // [3][ncplx] influence function
-    double* Q;                  // [nreal] charges
+    double* Q;                  // [nhalf] charges
     cufftDoubleComplex* Qh;     // [ncplx]
     cufftDoubleComplex* Ah;     // [ncplx]
-    double* A;                  // [nreal]
+    double* A;                  // [3][nhalf] the field's components
     int ncx, ncz;
     int64_t ncells;
     int* cell_count;            // [ncells]
@@ -192,8 +193,9 @@ __global__ void k_p3m_mul(const cufftDoubleComplex* __restrict__ Qh, const cufft
     Ah[idx] = make_cuDoubleComplex(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// Long-range sum, component c, interpolated with the assignment weights (written, not added).
-__global__ void k_p3m_interp(const P3MGeom G, const P3MPart S, const double* __restrict__ A, int c, double* sums) {
+// Long-range sums interpolated with the assignment weights (written, not added).
+__global__ void k_p3m_interp(const P3MGeom G, const P3MPart S, const double* __restrict__ A, int64_t nhalf,
+                             double* sums) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= S.n) return;
     const int64_t g = S.o + k;
@@ -203,17 +205,17 @@ __global__ void k_p3m_interp(const P3MGeom G, const P3MPart S, const double* __r
     const int ix = tsc((x - G.x0) / G.h, 1, G.Mx - 2, wx);
     const int iy = tsc((y - G.x0) / G.h, 1, G.Mx - 2, wy);
     const int iz = tsc(z / G.hz, -1 << 30, 1 << 30, wz);
-    double s = 0.0;
+    double s[3] = {0.0, 0.0, 0.0};
     for (int a = 0; a < 3; ++a)
         for (int b = 0; b < 3; ++b) {
             const int64_t rowb = ((int64_t)(ix + a - 1) * G.Nx + (iy + b - 1)) * G.Nz;
             for (int cc = 0; cc < 3; ++cc) {
                 int zz = (iz + cc - 1) % G.Nz;
                 if (zz < 0) zz += G.Nz;
-                s += A[rowb + zz] * wx[a] * wy[b] * wz[cc];
+                for (int c = 0; c < 3; ++c) s[c] += A[c * nhalf + rowb + zz] * wx[a] * wy[b] * wz[cc];
             }
         }
-    sums[3 * g + c] = s;
+    for (int c = 0; c < 3; ++c) sums[3 * g + c] = s[c];
 }
 
 // Cells are at least r_cut / kReachXY wide across the pipe and r_cut / kReachZ along it, so a particle's
@@ -555,6 +557,7 @@ P3MGeom geom_of(const pdq_p3m* P, double contact) {
 void free_plan(pdq_p3m* P) {
     if (!P) return;
     if (P->have_fwd) cufftDestroy(P->fwd);
+    if (P->have_lines) cufftDestroy(P->lines);
     if (P->have_inv) cufftDestroy(P->inv);
     cudaFree(P->Gh); cudaFree(P->Q); cudaFree(P->Qh); cudaFree(P->Ah); cudaFree(P->A);
     cudaFree(P->cell_count); cudaFree(P->cell_start); cudaFree(P->cell_fill); cudaFree(P->cell_list);
@@ -592,6 +595,7 @@ extern "C" int pdq_p3m_create(const pdq_field* field, const pdq_p3m_desc* d, int
     P->max_n = max_particles;
     if (!(P->rc < 0.5 * P->L)) { delete P; return PDQ_ERR_INVALID_ARG; }
     P->nreal = (size_t)P->Nx * P->Nx * P->Nz;
+    P->nhalf = (size_t)P->Mx * P->Nx * P->Nz;
     P->ncplx = (size_t)P->Nx * P->Nx * (P->Nz / 2 + 1);
     P->ncx = std::max(1, (int)std::min(128.0, floor(2.0 * P->R * kReachXY / P->rc)));
     P->ncz = std::max(1, (int)std::min(512.0, floor(P->L * kReachZ / P->rc)));
@@ -603,10 +607,10 @@ extern "C" int pdq_p3m_create(const pdq_field* field, const pdq_p3m_desc* d, int
         if (rc == PDQ_OK && cudaMalloc(p, bytes) != cudaSuccess) rc = PDQ_ERR_OOM;
     };
     alloc((void**)&P->Gh, 3 * P->ncplx * sizeof(cufftDoubleComplex));
-    alloc((void**)&P->Q, P->nreal * sizeof(double));
+    alloc((void**)&P->Q, P->nhalf * sizeof(double));
     alloc((void**)&P->Qh, P->ncplx * sizeof(cufftDoubleComplex));
     alloc((void**)&P->Ah, P->ncplx * sizeof(cufftDoubleComplex));
-    alloc((void**)&P->A, P->nreal * sizeof(double));
+    alloc((void**)&P->A, 3 * P->nhalf * sizeof(double));
     alloc((void**)&P->cell_count, P->ncells * sizeof(int));
     alloc((void**)&P->cell_start, (P->ncells + 1) * sizeof(int));
     alloc((void**)&P->cell_fill, P->ncells * sizeof(int));
@@ -614,20 +618,33 @@ extern "C" int pdq_p3m_create(const pdq_field* field, const pdq_p3m_desc* d, int
     alloc((void**)&P->sorted, 3 * P->max_n * sizeof(float4));
     alloc((void**)&P->lf_tab, 2 * kTab * sizeof(float4));
     alloc((void**)&Gr, 3 * P->nreal * sizeof(double));
-    if (rc == PDQ_OK) rc = cufft_status(cufftPlan3d(&P->fwd, P->Nx, P->Nx, P->Nz, CUFFT_D2Z));
+    // The charges reach only Mx of the Nx planes across (the rest is the zero padding of the open
+    // convolution) and the field is read on the same Mx: the (y, z) transforms run on those planes alone,
+    // the x transforms on all lines.  256^3: 1.75 -> 1.1 ms forward and 1.77 -> 1.1 ms back per component
+    // against whole 3-D transforms.
+    int n2[2] = {P->Nx, P->Nz}, real2[2] = {P->Nx, P->Nz}, cplx2[2] = {P->Nx, P->Nz / 2 + 1}, n1[1] = {P->Nx};
+    const int plane = P->Nx * (P->Nz / 2 + 1);
+    if (rc == PDQ_OK) rc = cufft_status(cufftPlanMany(&P->fwd, 2, n2, real2, 1, P->Nx * P->Nz, cplx2, 1, plane, CUFFT_D2Z, P->Mx));
     if (rc == PDQ_OK) P->have_fwd = true;
-    if (rc == PDQ_OK) rc = cufft_status(cufftPlan3d(&P->inv, P->Nx, P->Nx, P->Nz, CUFFT_Z2D));
+    if (rc == PDQ_OK) rc = cufft_status(cufftPlanMany(&P->lines, 1, n1, n1, plane, 1, n1, plane, 1, CUFFT_Z2Z, plane));
+    if (rc == PDQ_OK) P->have_lines = true;
+    if (rc == PDQ_OK) rc = cufft_status(cufftPlanMany(&P->inv, 2, n2, cplx2, 1, plane, real2, 1, P->Nx * P->Nz, CUFFT_Z2D, P->Mx));
     if (rc == PDQ_OK) P->have_inv = true;
-    if (rc == PDQ_OK) rc = cufft_status(cufftSetStream(P->fwd, s));
+    cufftHandle whole = 0;
+    bool have_whole = false;
+    if (rc == PDQ_OK) rc = cufft_status(cufftPlan3d(&whole, P->Nx, P->Nx, P->Nz, CUFFT_D2Z));
+    if (rc == PDQ_OK) have_whole = true;
+    if (rc == PDQ_OK) rc = cufft_status(cufftSetStream(whole, s));
     if (rc == PDQ_OK) {
         const P3MGeom G = geom_of(P, 0.0);
         k_p3m_kernel<<<grid_of(P->nreal, 256), 256, 0, s>>>(G, Gr, Gr + P->nreal, Gr + 2 * P->nreal);
         k_lf_table<<<grid_of(kTab, 128), 128, 0, s>>>(P->alpha, P->alpha * P->alpha * P->rc * P->rc, P->lf_tab);
         for (int c = 0; c < 3 && rc == PDQ_OK; ++c)
-            rc = cufft_status(cufftExecD2Z(P->fwd, Gr + c * P->nreal, P->Gh + c * P->ncplx));
+            rc = cufft_status(cufftExecD2Z(whole, Gr + c * P->nreal, P->Gh + c * P->ncplx));
         if (rc == PDQ_OK) k_p3m_deconv<<<grid_of(P->ncplx, 256), 256, 0, s>>>(G, P->Gh, (int64_t)P->ncplx);
         if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) rc = PDQ_ERR_CUDA;
     }
+    if (have_whole) cufftDestroy(whole);
     cudaFree(Gr);
     if (rc != PDQ_OK) { free_plan(P); return rc; }
     *out = P;
@@ -668,6 +685,7 @@ extern "C" int pdq_p3m_coulomb(pdq_p3m* P, const pdq_phys* phys, const pdq_state
         if (cnt[k] < 0 || cnt[k] > P->max_n) return PDQ_ERR_INVALID_ARG;
     PDQ_CUDA(cudaMemsetAsync(sums, 0, (size_t)st->capacity * 3 * sizeof(double), s));
     PDQ_CUDA(cufftSetStream(P->fwd, s) == CUFFT_SUCCESS ? cudaSuccess : cudaErrorUnknown);
+    PDQ_CUDA(cufftSetStream(P->lines, s) == CUFFT_SUCCESS ? cudaSuccess : cudaErrorUnknown);
     PDQ_CUDA(cufftSetStream(P->inv, s) == CUFFT_SUCCESS ? cudaSuccess : cudaErrorUnknown);
     const int h = st->cur;
     for (int k = 0; k < st->n_samples; ++k) {
@@ -677,16 +695,22 @@ extern "C" int pdq_p3m_coulomb(pdq_p3m* P, const pdq_phys* phys, const pdq_state
         S.o = off[k]; S.n = cnt[k]; S.precision = st->precision;
         const unsigned gp = grid_of(S.n, 256);
         // long range: assign, transform, multiply, transform back, interpolate
-        PDQ_CUDA(cudaMemsetAsync(P->Q, 0, P->nreal * sizeof(double), s));
+        PDQ_CUDA(cudaMemsetAsync(P->Q, 0, P->nhalf * sizeof(double), s));
         k_p3m_assign<<<gp, 256, 0, s>>>(G, S, P->Q);
         rc = cufft_status(cufftExecD2Z(P->fwd, P->Q, P->Qh));
         if (rc) return rc;
+        const size_t filled = (size_t)P->Mx * P->Nx * (P->Nz / 2 + 1);
+        PDQ_CUDA(cudaMemsetAsync(P->Qh + filled, 0, (P->ncplx - filled) * sizeof(cufftDoubleComplex), s));
+        rc = cufft_status(cufftExecZ2Z(P->lines, P->Qh, P->Qh, CUFFT_FORWARD));
+        if (rc) return rc;
         for (int c = 0; c < 3; ++c) {
             k_p3m_mul<<<grid_of(P->ncplx, 256), 256, 0, s>>>(P->Qh, P->Gh + c * P->ncplx, P->Ah, (int64_t)P->ncplx);
-            rc = cufft_status(cufftExecZ2D(P->inv, P->Ah, P->A));
+            rc = cufft_status(cufftExecZ2Z(P->lines, P->Ah, P->Ah, CUFFT_INVERSE));
             if (rc) return rc;
-            k_p3m_interp<<<gp, 256, 0, s>>>(G, S, P->A, c, sums);
+            rc = cufft_status(cufftExecZ2D(P->inv, P->Ah, P->A + c * P->nhalf));
+            if (rc) return rc;
         }
+        k_p3m_interp<<<gp, 256, 0, s>>>(G, S, P->A, (int64_t)P->nhalf, sums);
         // short range: cell list, then the direct sum
         PDQ_CUDA(cudaMemsetAsync(P->cell_count, 0, P->ncells * sizeof(int), s));
         PDQ_CUDA(cudaMemsetAsync(P->cell_fill, 0, P->ncells * sizeof(int), s));
