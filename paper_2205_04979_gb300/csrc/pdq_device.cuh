@@ -140,6 +140,19 @@ __device__ __forceinline__ float rsqrt_ftz(float x) {
 }
 __device__ __forceinline__ double rsqrt_ftz(double x) { return rsqrt(x); }
 
+// r2^(-3/2) in FP64 for a normal r2 > 0: the hardware's FP64 estimate y of r2^(-1/2) (~2^-20) and the
+// binomial series of (1 - d)^(-3/2) in d = 1 - r2 y^2, to d^3: 7 FP64 operations, against ~10 for the
+// library's reciprocal square root (with its branch for special values) and the two products.
+__device__ __forceinline__ double inv_cube64(double r2) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
+    const double t = y * y;
+    const double d = __fma_rn(-r2, t, 1.0);
+    const double c = d * __fma_rn(d, __fma_rn(d, 2.1875, 1.875), 1.5);
+    const double y3 = y * t;
+    return __fma_rn(y3, c, y3);
+}
+
 __device__ __forceinline__ void coulomb_pair(float xi, float yi, float zi, const float4 pj, float L, float invL,
                                              float c2, float& ax, float& ay, float& az) {
     const float dx = xi - pj.x, dy = yi - pj.y;
@@ -160,8 +173,7 @@ __device__ __forceinline__ void coulomb_pair(double xi, double yi, double zi, co
     const double t = __dadd_rn(__fma_rn(dz, invL, 6755399441055744.0), -6755399441055744.0);
     dz = __fma_rn(-L, t, dz);
     const double r2 = fmax(__fma_rn(dx, dx, __fma_rn(dy, dy, dz * dz)), c2);
-    const double ri = rsqrt(r2);
-    const double s = pj.w * ri * (ri * ri);
+    const double s = pj.w * inv_cube64(r2);
     ax = __fma_rn(s, dx, ax);
     ay = __fma_rn(s, dy, ay);
     az = __fma_rn(s, dz, az);
@@ -208,6 +220,7 @@ __device__ __forceinline__ void f2_unpack(f2 v, float& a, float& b) { asm("mov.b
 __device__ __forceinline__ f2 f2_sub(f2 a, f2 b) { f2 d; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
 __device__ __forceinline__ f2 f2_add(f2 a, f2 b) { f2 d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
 __device__ __forceinline__ f2 f2_mul(f2 a, f2 b) { f2 d; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
+__device__ __forceinline__ f2 f2_dup(float a) { return f2_pack(a, a); }
 __device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
     f2 d;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));

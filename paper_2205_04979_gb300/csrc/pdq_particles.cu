@@ -22,6 +22,7 @@
 #include "pdq_common.cuh"
 #include "pdq_device.cuh"
 #include "pdq_newton.cuh"
+#include "pdq_split.cuh"
 
 namespace pdq {
 
@@ -195,6 +196,7 @@ struct StepArgs {
     double* acc64;
     // MIXED pair variant 3: particles per thread of k_pairs_sym and CTAs per tile (newton_cut)
     int newton_u, newton_parts;
+    SplitGrid grid;      // FP64 pair variant 3: of the split coordinates (k_pairs_split64)
     // host only: upper bound on the work items of a launch (the persistent grid is capped by it,
     // so that few items spread one per CTA over the SMs instead of piling onto the first CTAs)
     int64_t max_items;
@@ -514,8 +516,7 @@ __device__ __forceinline__ void coulomb_pair_direct64(double xi, double yi, doub
     const double dx = xi - pj.x, dy = yi - pj.y, dz = zi - pj.z;
     double r2 = __fma_rn(dx, dx, __fma_rn(dy, dy, dz * dz));
     if constexpr (CLAMP) r2 = fmax(r2, c2);
-    const double ri = rsqrt(r2);
-    const double s = pj.w * ri * (ri * ri);
+    const double s = pj.w * inv_cube64(r2);
     ax = __fma_rn(s, dx, ax);
     ay = __fma_rn(s, dy, ay);
     az = __fma_rn(s, dz, az);
@@ -534,8 +535,7 @@ __device__ __forceinline__ void coulomb_pair_track(double xi, double yi, double 
     const double r2u = __fma_rn(dx, dx, __fma_rn(dy, dy, dz * dz));
     mnh = min(mnh, __double2hiint(r2u));
     const double r2 = fmax(r2u, c2);
-    const double ri = rsqrt(r2);
-    const double s = pj.w * ri * (ri * ri);
+    const double s = pj.w * inv_cube64(r2);
     ax = __fma_rn(s, dx, ax);
     ay = __fma_rn(s, dy, ay);
     az = __fma_rn(s, dz, az);
@@ -1015,6 +1015,9 @@ __global__ void __launch_bounds__(NT, (U == 12 ? 3 : U == 8 ? 4 : 5) * (128 / NT
                             gridDim.y);
 }
 
+// Samples of at least this many particles take k_pairs_split64 instead of k_pairs_sym64 (pair variant
+// 3 in FP64).
+constexpr int kSplitMin = 8192;
 
 // FP64 Newton pair: coulomb_pair_x2_sym for one i-particle in double (minimum image by the
 // 1.5 * 2^52 rounding constant, as the one-sided FP64 pair).
@@ -1030,8 +1033,7 @@ __device__ __forceinline__ void coulomb_pair_sym64(double xi, double yi, double 
     }
     double r2 = __fma_rn(dx, dx, __fma_rn(dy, dy, dz * dz));
     if constexpr (CLAMP) r2 = fmax(r2, c2);
-    const double ri = rsqrt(r2);
-    const double ri3 = ri * (ri * ri);
+    const double ri3 = inv_cube64(r2);
     const double si = zqj.y * ri3, sj = nqi * ri3;
     ax = __fma_rn(si, dx, ax);
     ay = __fma_rn(si, dy, ay);
@@ -1071,6 +1073,10 @@ __global__ void __launch_bounds__(NT) k_pairs_sym64(const StepArgs A) {
         const int2 it = A.items[item];
         const int64_t o = A.offset[it.x];
         const int64_t end = o + A.count[it.x];
+        if (end - o >= kSplitMin) {      // k_pairs_split64's
+            __syncthreads();
+            continue;
+        }
         const int tile = it.y / JS, jc = it.y - tile * JS;
         const int64_t base = o + (int64_t)tile * (NT * U);
         const int64_t dend = base + NT * U < end ? base + NT * U : end;
@@ -1227,6 +1233,200 @@ __global__ void __launch_bounds__(NT) k_pairs_sym64(const StepArgs A) {
             A.ctl[CTL_QUEUE2] = 0;
             A.ctl[CTL_DONE2] = 0;
             __threadfence();
+        }
+    }
+}
+
+// FP64 Coulomb sums of large samples, one-sided, with the far pairs on the FP32 pipe: a j group whose
+// z distance from the warp's i-particles exceeds twice the sample's mean spacing is summed in float-float
+// (pdq_split.cuh, ~2^-46 per pair, three-float accumulators), the near groups in FP64.  A far pair's
+// term is small against the sum, so its rounding is too: over samples of 8,192 to 100,000 particles
+// the sums are no further from the exact ones than k_pairs_sym64's.  Below kSplitMin the near share
+// grows and that no longer holds.  The item table is k_pairs_sym64's (tiles of 2 NT particles, JS
+// chunks of the sample's j range); each CTA adds its item's sums to A.acc64 by atomics.
+// Bound by the FP32 FMA pipe (~135 operations per ordered pair, packed for two i).  100,000 particles,
+// 64 threads: 56 ms per step, 192 ms in k_pairs_sym64 (FP64 pipe 90 % busy); error of the sums against
+// extended precision, in units of 2^-53 of their 2-norm: 3.8 (6.3 before), at 8,192 particles 5.8 (5.7).
+// Three-float accumulators that are flushed once per j-tile instead of once per group left 7 and 14 units, without
+// the second word of the sums 24 and 38.
+template <int NT>
+__global__ void __launch_bounds__(NT, 384 / NT) k_pairs_split64(const StepArgs A) {
+    constexpr int W = NT / 32;
+    __shared__ __align__(16) double2 s_xy[NT], s_zq[NT];
+    __shared__ __align__(16) ulonglong2 s_f[6][NT];      // each float twice: x y, z q (hi), x y, z q (mid), x y, z - (lo)
+    __shared__ double2 s_zr[W];
+    const int item = blockIdx.x;
+    if (item >= A.ctl[CTL_NITEMS]) return;
+    const StepConst& K = A.K;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int2 it = A.items[item];
+    const int64_t o = A.offset[it.x], end = o + A.count[it.x], n = end - o;
+    if (n < kSplitMin) return;
+    const int JS = A.jsplit, tile = it.y / JS, jc = it.y - tile * JS;
+    const int64_t base = o + (int64_t)tile * (2 * NT), ch = ((n + JS - 1) / JS + NT - 1) / NT * NT;
+    const int64_t jb = o + jc * ch, je = jb + ch < end ? jb + ch : end;
+    if (jb >= je) return;
+    const double4_32a* __restrict__ pos_in = (const double4_32a*)A.pos_in;
+    const double L = K.L, invL = K.invL, c2 = K.contact2, halfL = 0.5 * L;
+    const double dcz = sqrt(c2) + 1e-9;        // contact distance + rounding margin
+    const double far = fmax(dcz, 2.0 * cbrt(kPi * K.R * K.R * L / (double)n));
+    // this lane's two i-particles, a contiguous run of 64 per warp
+    double xi[2], yi[2], zi[2], sum[3][2];
+    double ilo = INFINITY, ihi = -INFINITY;
+    f2 H[3], M[3], T[3], S[3], C[3], CC[3];
+    {
+        float h[2][3], m[2][3], l[2][3];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int64_t g = base + warp * 64 + u * 32 + lane;
+            const double4_32a p = pos_in[g < end ? g : end - 1];      // past the end: a copy, not stored
+            xi[u] = p.x; yi[u] = p.y; zi[u] = p.z;
+            ilo = fmin(ilo, p.z);
+            ihi = fmax(ihi, p.z);
+            sum[0][u] = sum[1][u] = sum[2][u] = 0.0;
+            split3(A.grid, p.x, h[u][0], m[u][0], l[u][0]);
+            split3(A.grid, p.y, h[u][1], m[u][1], l[u][1]);
+            split3(A.grid, p.z, h[u][2], m[u][2], l[u][2]);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            H[k] = f2_pack(h[0][k], h[1][k]); M[k] = f2_pack(m[0][k], m[1][k]); T[k] = f2_pack(l[0][k], l[1][k]);
+            S[k] = C[k] = CC[k] = 0ull;
+        }
+    }
+    for (int d = 16; d > 0; d >>= 1) {
+        ilo = fmin(ilo, __shfl_xor_sync(0xffffffffu, ilo, d));
+        ihi = fmax(ihi, __shfl_xor_sync(0xffffffffu, ihi, d));
+    }
+    float Lh, Lm, Ll;
+    split3(A.grid, L, Lh, Lm, Ll);
+    const float hLh = (float)halfL, hLl = (float)(halfL - (double)hLh);
+    for (int64_t j0 = jb; j0 < je; j0 += NT) {
+        const int64_t j = j0 + tid;
+        double4_32a p = make_double4_32a(xi[0], yi[0], zi[0], 0.0);      // past the end: no charge
+        if (j < je) p = pos_in[j];
+        double lo = j < je ? p.z : INFINITY, hi = j < je ? p.z : -INFINITY;
+        for (int d = 16; d > 0; d >>= 1) {
+            lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, d));
+            hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, d));
+        }
+        if (lane == 0) s_zr[warp] = make_double2(lo, hi);
+        {
+            float h[3], m[3], l[3];
+            split3(A.grid, p.x, h[0], m[0], l[0]);
+            split3(A.grid, p.y, h[1], m[1], l[1]);
+            split3(A.grid, p.z, h[2], m[2], l[2]);
+            const float qh = (float)p.w, ql = (float)(p.w - (double)qh);
+            s_xy[tid] = make_double2(p.x, p.y);
+            s_zq[tid] = make_double2(p.z, p.w);
+            s_f[0][tid] = make_ulonglong2(f2_dup(h[0]), f2_dup(h[1]));
+            s_f[1][tid] = make_ulonglong2(f2_dup(h[2]), f2_dup(qh));
+            s_f[2][tid] = make_ulonglong2(f2_dup(m[0]), f2_dup(m[1]));
+            s_f[3][tid] = make_ulonglong2(f2_dup(m[2]), f2_dup(ql));
+            s_f[4][tid] = make_ulonglong2(f2_dup(l[0]), f2_dup(l[1]));
+            s_f[5][tid] = make_ulonglong2(f2_dup(l[2]), 0ull);
+        }
+        __syncthreads();
+        double t[3][2] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};      // this j-tile's (a long chain of adds rounds more)
+#pragma unroll 1
+        for (int g = 0; g < W; ++g) {
+            const int ng = (int)(je - j0 - 32 * g < 32 ? je - j0 - 32 * g : 32);
+            if (ng <= 0) break;                        // uniform across the CTA
+            // z_i - z_j over the group lies in [dlo, dhi]
+            const double dlo = ilo - s_zr[g].y, dhi = ihi - s_zr[g].x;
+            const bool is_far = (dlo > far && dhi < L - far) || (dhi < -far && dlo > far - L);
+            double shift = 0.0;
+            bool direct = true;
+            if (dlo > -halfL && dhi < halfL) shift = 0.0;
+            else if (dlo > halfL && dhi < 3.0 * halfL) shift = L;
+            else if (dhi < -halfL && dlo > -3.0 * halfL) shift = -L;
+            else direct = false;
+            if (is_far) {
+                auto far_sum = [&](auto minimg) {
+                    // the period's parts, signed by the group's shift
+                    const float sg = (float)(shift * invL);
+                    const f2 zh = f2_sub(H[2], f2_dup(sg * Lh)), zm = f2_sub(M[2], f2_dup(sg * Lm));
+                    const f2 zl = f2_sub(T[2], f2_dup(sg * Ll));
+#pragma unroll 1
+                    for (int k = 32 * g; k < 32 * g + ng; ++k) {
+                        const ulonglong2 f0 = s_f[0][k], f1 = s_f[1][k], f2_ = s_f[2][k], f3 = s_f[3][k];
+                        const ulonglong2 f4 = s_f[4][k], f5 = s_f[5][k];
+                        f2 D[3], E[3], w, v, P, Q;
+                        split_diff(H[0], M[0], T[0], f0.x, f2_.x, f4.x, D[0], E[0]);
+                        split_diff(H[1], M[1], T[1], f0.y, f2_.y, f4.y, D[1], E[1]);
+                        if constexpr (decltype(minimg)::value) {
+                            // nearest image pair by pair: the group's z distances all have the sign of dlo,
+                            // so L goes off where |z_i - z_j| (all its bits) exceeds L/2
+                            const f2 dh = f2_sub(H[2], f1.x), dm = f2_sub(M[2], f3.x), dl = f2_sub(T[2], f5.x);
+                            two_sum(dh, dm, D[2], E[2]);
+                            E[2] = f2_add(E[2], dl);
+                            const float sg = dlo > 0.0 ? 1.f : -1.f;
+                            float ta, tb;
+                            f2_unpack(f2_add(f2_fma(D[2], f2_dup(sg), f2_dup(-hLh)), f2_fma(E[2], f2_dup(sg), f2_dup(-hLl))),
+                                      ta, tb);
+                            const f2 nn = f2_pack(ta > 0.f ? -sg : 0.f, tb > 0.f ? -sg : 0.f);
+                            two_sum(f2_fma(nn, f2_dup(Lh), dh), f2_fma(nn, f2_dup(Lm), dm), D[2], E[2]);
+                            E[2] = f2_add(E[2], f2_fma(nn, f2_dup(Ll), dl));
+                        } else {
+                            const f2 dh = f2_sub(zh, f1.x), dm = f2_sub(zm, f3.x);
+                            two_sum(dh, dm, D[2], E[2]);
+                            E[2] = f2_add(E[2], f2_sub(zl, f5.x));
+                        }
+                        split_inv_cube_norm(D, E, w, v);
+                        split_mul(w, v, f1.y, f3.y, P, Q);
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            f2 F, Fe, e0, e1;
+                            split_mul(P, Q, D[c], E[c], F, Fe);
+                            two_sum(S[c], F, S[c], e0);
+                            two_sum(C[c], e0, C[c], e1);
+                            CC[c] = f2_add(CC[c], f2_add(Fe, e1));
+                        }
+                    }
+                };
+                if (direct) far_sum(std::false_type{});
+                else far_sum(std::true_type{});
+                // the low words leave once per group, before their sum's own rounding counts
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    float r0, r1;
+                    f2_unpack(CC[c], r0, r1);
+                    t[c][0] += (double)r0;
+                    t[c][1] += (double)r1;
+                    CC[c] = 0ull;
+                }
+            } else if (direct) {
+                const double z0 = zi[0] - shift, z1 = zi[1] - shift;
+#pragma unroll 2
+                for (int k = 32 * g; k < 32 * g + ng; ++k) {
+                    const double2 a = s_xy[k], b = s_zq[k];
+                    const double4_32a pj = make_double4_32a(a.x, a.y, b.x, b.y);
+                    coulomb_pair_direct64<true>(xi[0], yi[0], z0, pj, c2, t[0][0], t[1][0], t[2][0]);
+                    coulomb_pair_direct64<true>(xi[1], yi[1], z1, pj, c2, t[0][1], t[1][1], t[2][1]);
+                }
+            } else {
+#pragma unroll 2
+                for (int k = 32 * g; k < 32 * g + ng; ++k) {
+                    const double2 a = s_xy[k], b = s_zq[k];
+                    const double4_32a pj = make_double4_32a(a.x, a.y, b.x, b.y);
+                    coulomb_pair(xi[0], yi[0], zi[0], pj, L, invL, c2, t[0][0], t[1][0], t[2][0]);
+                    coulomb_pair(xi[1], yi[1], zi[1], pj, L, invL, c2, t[0][1], t[1][1], t[2][1]);
+                }
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) { sum[c][0] += t[c][0]; sum[c][1] += t[c][1]; }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        float s[2], e[2];
+        f2_unpack(S[c], s[0], s[1]);
+        f2_unpack(C[c], e[0], e[1]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int64_t g = base + warp * 64 + u * 32 + lane;
+            if (g < end) atomicAdd(&A.acc64[3 * g + c], sum[c][u] + ((double)s[u] + (double)e[u]));
         }
     }
 }
@@ -1532,6 +1732,8 @@ static int launch_newton64(const StepArgs& A, cudaStream_t s) {
     if (A.K.forces & PDQ_F_COULOMB) {    // the sums enter the update only with the Coulomb force on
         k_pairs_sym64<NT, 2><<<(unsigned)std::max<int64_t>(1, std::min(full, A.max_items > 0 ? A.max_items : full)),
                                NT, 0, s>>>(A);
+        if (A.cap >= kSplitMin)
+            k_pairs_split64<NT><<<(unsigned)std::max<int64_t>(1, A.max_items), NT, 0, s>>>(A);
     }
     StepArgs B = A;
     B.ext = A.acc64;
@@ -1638,12 +1840,19 @@ static int j_split(const pdq_state* st, int TI, bool contact = false) {
     return js < 1 ? 1 : (int)js;
 }
 
-// FP64 Newton pairs: j-chunks per tile so that the triangular work of few large samples spreads
-// evenly (about 8 i-tiles of j per chunk, at most 64 chunks).
-static int newton_chunks(const pdq_state* st, int TI) {
+// FP64 pair variant 3: j-chunks per tile (at most 64).  `coarse`: about 8 i-tiles of j per chunk, so that
+// the triangular work of few large samples spreads evenly.  Otherwise at least as many as give each SM
+// 48 items (6 CTAs of 64 threads run there at once), of one j-tile or more: 20,000 particles had 20
+// chunks and left the last SMs 40 % of the time alone.
+static int newton_chunks(const pdq_state* st, int TI, bool coarse) {
     if (st->precision != PDQ_FP64) return 1;
     const int64_t cap = st->capacity > 0 ? st->capacity : 1;
     int64_t js = (cap + 8 * (int64_t)TI - 1) / (8 * (int64_t)TI);
+    if (!coarse) {
+        const int64_t tiles = (cap + TI - 1) / TI, n = (cap + st->n_samples - 1) / st->n_samples;
+        const int64_t want = (48 * (int64_t)sm_count() + tiles - 1) / tiles, most = (n + TI / 2 - 1) / (TI / 2);
+        js = std::max(js, std::min(want, most));
+    }
     if (js > 64) js = 64;
     return js < 1 ? 1 : (int)js;
 }
@@ -1653,8 +1862,8 @@ static int newton_chunks(const pdq_state* st, int TI) {
 // pair variant 3: the sums, float4 [capacity] (MIXED) or double [capacity][3] (FP64).
 static void workspace_layout(const pdq_state* st, int TI, size_t* items_bytes, size_t* total,
                              size_t* cnt_off = nullptr, size_t* part_off = nullptr, bool contact = false,
-                             size_t* acc_off = nullptr, bool newton = false) {
-    const int JS = newton ? newton_chunks(st, TI) : j_split(st, TI, contact);
+                             size_t* acc_off = nullptr, bool newton = false, bool coarse = false) {
+    const int JS = newton ? newton_chunks(st, TI, coarse) : j_split(st, TI, contact);
     const int64_t max_tiles = st->capacity / TI + st->n_samples + 1;
     *items_bytes = align256(sizeof(int2) * (size_t)max_tiles * JS);
     *total = *items_bytes + align256(sizeof(int32_t) * (size_t)st->n_samples);
@@ -1835,8 +2044,13 @@ int step_impl(const pdq_field* field, const pdq_phys* phys, pdq_state* st, const
             workspace_layout(st, NT * U, &items_bytes, &need, &cnt_off, &part_off, contact, &acc_off, newton);
         }
     }
+    bool coarse = false;
+    if (newton && st->precision == PDQ_FP64 && workspace_bytes < need) {      // likewise for fewer chunks
+        coarse = true;
+        workspace_layout(st, NT * U, &items_bytes, &need, &cnt_off, &part_off, contact, &acc_off, newton, coarse);
+    }
     if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255)) return PDQ_ERR_WORKSPACE;
-    const int JS = newton ? newton_chunks(st, NT * U) : j_split(st, NT * U, contact || ext);
+    const int JS = newton ? newton_chunks(st, NT * U, coarse) : j_split(st, NT * U, contact || ext);
     if (n_steps == 0) return PDQ_OK;
     StepArgs A;
     memset(&A, 0, sizeof(A));
@@ -1861,6 +2075,7 @@ int step_impl(const pdq_field* field, const pdq_phys* phys, pdq_state* st, const
     A.cap = st->capacity;
     A.newton_u = cut.U;
     A.newton_parts = cut.parts;
+    A.grid = split_grid(std::max(A.K.R, A.K.L));
     A.ext = ext;
     if (newton && st->precision == PDQ_MIXED) A.acc4 = (float4*)((char*)workspace + acc_off);
     if (newton && st->precision == PDQ_FP64) A.acc64 = (double*)((char*)workspace + acc_off);

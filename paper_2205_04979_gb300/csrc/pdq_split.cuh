@@ -90,4 +90,48 @@ __device__ __forceinline__ void split_mul(float a, float b, float c, float d, fl
     e = __fmaf_rn(a, d, __fmaf_rn(b, c, __fmaf_rn(b, d, __fmaf_rn(a, c, -p))));
 }
 
+// The same on two pairs at a time (f32x2), for one j against two i-particles.
+__device__ __forceinline__ f2 f2_neg(f2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ void two_sum(f2 a, f2 b, f2& s, f2& e) {
+    const f2 t = f2_add(a, b), bb = f2_sub(t, a);
+    e = f2_add(f2_sub(a, f2_sub(t, bb)), f2_sub(b, bb));
+    s = t;
+}
+__device__ __forceinline__ void split_diff(f2 ah, f2 am, f2 al, f2 bh, f2 bm, f2 bl, f2& D, f2& E) {
+    const f2 dh = f2_sub(ah, bh), dm = f2_sub(am, bm);
+    D = f2_add(dh, dm);
+    E = f2_add(f2_sub(dm, f2_sub(D, dh)), f2_sub(al, bl));
+}
+__device__ __forceinline__ void split_mul(f2 a, f2 b, f2 c, f2 d, f2& p, f2& e) {
+    p = f2_mul(a, c);
+    e = f2_fma(a, d, f2_fma(b, c, f2_fma(b, d, f2_fma(a, c, f2_neg(p)))));
+}
+// (w, v) = (D + E)^2 summed over the components, to the power -3/2.
+__device__ __forceinline__ void split_inv_cube_norm(const f2 D[3], const f2 E[3], f2& w, f2& v) {
+    f2 p[3], e[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        p[k] = f2_mul(D[k], D[k]);
+        e[k] = f2_fma(D[k], f2_add(E[k], E[k]), f2_fma(E[k], E[k], f2_fma(D[k], D[k], f2_neg(p[k]))));
+    }
+    f2 s, t1, t2, R;
+    two_sum(p[0], p[1], s, t1);
+    two_sum(s, p[2], R, t2);
+    const f2 r = f2_add(f2_add(f2_add(e[0], e[1]), f2_add(e[2], t1)), t2);
+    float Ra, Rb;
+    f2_unpack(R, Ra, Rb);
+    const f2 y = f2_pack(rsqrt_ftz(Ra), rsqrt_ftz(Rb));
+    const f2 q = f2_mul(y, y), qe = f2_fma(y, y, f2_neg(q));
+    const f2 m = f2_mul(R, q);
+    // 1 - (R + r) y^2 = a - u
+    const f2 a = f2_sub(f2_dup(1.0f), m);
+    const f2 u = f2_fma(r, q, f2_fma(R, qe, f2_fma(R, q, f2_neg(m))));
+    const f2 ab = f2_sub(a, u);
+    const f2 ch = f2_mul(f2_dup(1.5f), a);
+    const f2 cl = f2_fma(f2_dup(1.875f), f2_mul(ab, ab), f2_mul(f2_dup(-1.5f), u));
+    const f2 c = f2_mul(y, q), ce = f2_fma(y, qe, f2_fma(y, q, f2_neg(c)));
+    w = f2_fma(ch, c, c);
+    v = f2_add(f2_fma(ch, c, f2_sub(c, w)), f2_fma(c, cl, f2_fma(ce, f2_add(ch, cl), ce)));
+}
+
 }  // namespace pdq

@@ -246,6 +246,41 @@ def test_fp64_newton_pairs_chunked_single_sample(pdq, fields):
     assert np.array_equal(tally.n_dep.cpu().numpy(), nd) and np.array_equal(tally.n_alive.cpu().numpy(), na)
 
 
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("counts", [[8191], [8192], [8321, 40]])
+def test_fp64_newton_pairs_large_samples(pdq, fields, counts, block):
+    # samples of 8,192 particles and more sum their far pairs in float-float; one step against the
+    # oracle, and the Coulomb sums alone (a step of that force from rest) against extended precision on
+    # 64 particles.  Bar of the sums: terms rounded at 2^-46 add up at random to 2^-46 sqrt(sum f^2), at
+    # this density ~0.1 of the sum: ~7 units of 2^-53; the FP64 adds give as much again.  24 units.
+    off = np.r_[0, np.cumsum(counts)]
+    st, tally, ost, nd, na = _run_both(pdq, fields, 0, counts, ST3, PRM3[:len(counts)], 1, {"variant": 3}, block=block)
+    assert _compare_by_id(st, ost, off, 1e-12, 1e-12) > 0
+    assert np.array_equal(tally.n_dep.cpu().numpy(), nd) and np.array_equal(tally.n_alive.cpu().numpy(), na)
+    phys, st, prm, ost, off = _setup(pdq, fields, 0, counts[:1], ST3, PRM3[:1], sigma=0.5)
+    cfg = pdq.step_cfg(1.0, forces=pdq.F_COULOMB, gravity=(0, 0, 0), block=block, variant=3)
+    pdq.step_particles(fields[0], phys, st, prm, cfg, 1, pdq.Tally(1, 3), pdq.workspace(st, cfg))
+    v = np.zeros((counts[0], 3))
+    v[st.tag.cpu().numpy()[:, 0]] = st.current()[1].cpu().numpy()[:, :3]
+    ld = np.longdouble
+    X, q = np.stack([ost.x, ost.y, ost.z], 1).astype(ld), ost.q.astype(ld)
+    table = oracle.class_table(ST3)
+    dc2 = ld(table[:, 1].max()) ** 2
+    err = ref = 0.0
+    for c in range(3):
+        idx = np.random.default_rng(c).choice(np.flatnonzero(ost.cls == c), 22, replace=False)
+        want = []
+        for i in idx:
+            d = X[i] - X
+            d[:, 2] -= 720 * np.rint(d[:, 2] / 720)
+            r2 = np.maximum((d * d).sum(1), dc2)
+            want.append(q[i] * (q[:, None] * d / (r2 * np.sqrt(r2))[:, None]).sum(0))
+        want = np.array(want)
+        k = (want * v[idx]).sum() / (want * want).sum()       # the class's coefficient, with its rounding
+        err, ref = err + (((v[idx] - k * want) / k) ** 2).sum(), ref + (want * want).sum()
+    assert np.sqrt(float(err / ref)) <= 24 * 2.0 ** -53
+
+
 @pytest.mark.parametrize("variant", [0, 3])
 def test_fp64_rebound_parity(pdq, fields, variant):
     # Rebounding particles bounce inside the stiff vdW zone (accelerations ~1e4 wall units),
