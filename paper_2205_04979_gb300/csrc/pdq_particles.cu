@@ -1431,6 +1431,158 @@ __global__ void __launch_bounds__(NT, 384 / NT) k_pairs_split64(const StepArgs A
     }
 }
 
+// FP64 one-sided runs of few particles (pair variant 0, 32 threads, one j-chunk per tile: JS 32 >= capacity):
+// the sums by pairs of 32-particle tiles, one CTA each, every pair evaluated once for both tiles (tile I
+// with tiles I + d mod T, d = 0 .. T/2, so that hardly a CTA of the grid is idle; with I <= J the CTAs
+// that left at once made the SMs' shares uneven, 43 us for 1,000 particles instead of 33; the one-sided
+// loop with its chunk counters took ~50 of the step's 75 us, now 58 with the update's 24): lane l holds i = l of tile I and meets j = (l + k) mod 32 of tile J at step k, whose running sum
+// moves on to lane l - 1.  Warp w takes the steps [8 w, 8 w + 8): a warp alone issues an FP64 instruction
+// every ~94 clocks, a scheduler's FP64 unit takes one every 64.  The warps' sums are added in order; tile I's
+// go to chunk J of the partial sums and tile J's to chunk I, each slot written once, so the result does not
+// depend on the schedule.
+constexpr int kTileWarps = 4;
+__global__ void __launch_bounds__(32 * kTileWarps) k_pairs_tiles64(const StepArgs A) {
+    constexpr int kSteps = 32 / kTileWarps;
+    __shared__ __align__(16) double2 s_xy[32], s_zq[32];
+    __shared__ double s_sum[kTileWarps][6][32];
+    const int JS = A.jsplit, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t item = (int64_t)blockIdx.x * JS;
+    if (item >= A.ctl[CTL_NITEMS]) return;
+    const StepConst& K = A.K;
+    const int2 it = A.items[item];
+    const int I = it.y / JS, d = blockIdx.y;
+    const int64_t o = A.offset[it.x];
+    const int n = A.count[it.x], T = (n + 31) / 32;
+    if (2 * d > T || (2 * d == T && 2 * I >= T)) return;
+    const int J = I + d < T ? I + d : I + d - T;
+    const double4_32a* __restrict__ pos_in = (const double4_32a*)A.pos_in;
+    const double L = K.L, invL = K.invL, c2 = K.contact2;
+    const int gi = 32 * I + lane, gj = 32 * J + lane;
+    double4_32a p = make_double4_32a(1e15, 0.0, 0.0, 0.0), q = make_double4_32a(-1e15, 0.0, 0.0, 0.0);
+    if (gi < n) p = pos_in[o + gi];
+    if (gj < n) q = pos_in[o + gj];
+    if (warp == 0) {
+        s_xy[lane] = make_double2(q.x, q.y);
+        s_zq[lane] = make_double2(q.z, q.w);
+    }
+    __syncthreads();
+    double ax = 0.0, ay = 0.0, az = 0.0, jx = 0.0, jy = 0.0, jz = 0.0;
+    if (I == J) {       // every pair from both sides (the self pair: d = 0 adds nothing)
+#pragma unroll 4
+        for (int k = kSteps * warp; k < kSteps * (warp + 1); ++k) {
+            const double2 a = s_xy[k], b = s_zq[k];
+            coulomb_pair(p.x, p.y, p.z, make_double4_32a(a.x, a.y, b.x, b.y), L, invL, c2, ax, ay, az);
+        }
+    } else {
+        // as in the other pair kernels, by the tiles' z ranges (in FP32, rounded outward): a uniform shift
+        // for the nearest image inside one period window, no clamp for z-separated tiles
+        float ilo = gi < n ? __double2float_rd(p.z) : INFINITY, ihi = gi < n ? __double2float_ru(p.z) : -INFINITY;
+        float jlo = gj < n ? __double2float_rd(q.z) : INFINITY, jhi = gj < n ? __double2float_ru(q.z) : -INFINITY;
+        for (int d = 16; d > 0; d >>= 1) {
+            ilo = fminf(ilo, __shfl_xor_sync(0xffffffffu, ilo, d));
+            ihi = fmaxf(ihi, __shfl_xor_sync(0xffffffffu, ihi, d));
+            jlo = fminf(jlo, __shfl_xor_sync(0xffffffffu, jlo, d));
+            jhi = fmaxf(jhi, __shfl_xor_sync(0xffffffffu, jhi, d));
+        }
+        const double dlo = (double)ilo - (double)jhi, dhi = (double)ihi - (double)jlo, halfL = 0.5 * L;
+        const double dcz = (double)(sqrtf(K.contact2f) + 1e-2f);
+        double shift = 0.0;
+        bool direct = true;
+        if (dlo > -halfL && dhi < halfL) shift = 0.0;
+        else if (dlo > halfL && dhi < 3.0 * halfL) shift = L;
+        else if (dhi < -halfL && dlo > -3.0 * halfL) shift = -L;
+        else direct = false;
+        const bool apart = dlo - shift > dcz || dhi - shift < -dcz;
+        const double nq = -p.w;
+        auto group = [&](auto minimg, auto clamp, double zi) {
+#pragma unroll 4
+            for (int k = kSteps * warp; k < kSteps * (warp + 1); ++k) {
+                const int jj = (lane + k) & 31;
+                const double2 a = s_xy[jj], b = s_zq[jj];
+                coulomb_pair_sym64<decltype(minimg)::value, decltype(clamp)::value>(p.x, p.y, zi, nq, a, b, L, invL, c2, ax,
+                                                                                    ay, az, jx, jy, jz);
+                jx = __shfl_sync(0xffffffffu, jx, (lane + 1) & 31);
+                jy = __shfl_sync(0xffffffffu, jy, (lane + 1) & 31);
+                jz = __shfl_sync(0xffffffffu, jz, (lane + 1) & 31);
+            }
+        };
+        if (!direct) group(std::true_type{}, std::true_type{}, p.z);
+        else if (apart) group(std::false_type{}, std::false_type{}, p.z - shift);
+        else group(std::false_type{}, std::true_type{}, p.z - shift);
+        const int home = (lane + kSteps * (warp + 1)) & 31;      // the j whose sum arrived here
+        s_sum[warp][3][home] = jx; s_sum[warp][4][home] = jy; s_sum[warp][5][home] = jz;
+    }
+    s_sum[warp][0][lane] = ax; s_sum[warp][1][lane] = ay; s_sum[warp][2][lane] = az;
+    __syncthreads();
+    for (int c = warp; c < 6; c += kTileWarps) {
+        if (c >= 3 && I == J) continue;
+        double v = s_sum[0][c][lane];
+        for (int w = 1; w < kTileWarps; ++w) v += s_sum[w][c][lane];
+        const int chunk = c < 3 ? J : I, at = c < 3 ? gi : gj;
+        if (at < n) A.part[(int64_t)(chunk * 3 + c % 3) * A.cap + o + at] = v;
+    }
+}
+
+// The update of such a run: kTilePart particles per warp, whose partial sums 32 / kTilePart lanes each add
+// up (runs of chunks in order, then the runs in order), and one lane each advances them.  A warp's FP64
+// instruction occupies its scheduler's FP64 unit by the lane, so a few particles on every scheduler
+// finish sooner than 32 on a few.
+constexpr int kTilePart = 8;
+__global__ void __launch_bounds__(32) k_update_tiles64(const StepArgs A) {
+    constexpr int R = 32 / kTilePart;
+    const StepConst& K = A.K;
+    const int lane = threadIdx.x, r = lane / kTilePart, JS = A.jsplit, C = K.n_classes;
+    const int64_t step = A.ctl[CTL_STEP], item = blockIdx.x / R;
+    if (item * JS < A.ctl[CTL_NITEMS]) {
+        const int2 it = A.items[item * JS];
+        const int s = it.x;
+        const int64_t o = A.offset[s], end = o + A.count[s];
+        const int64_t g = o + (int64_t)(it.y / JS) * 32 + (blockIdx.x % R) * kTilePart + lane % kTilePart;
+        double sx = 0.0, sy = 0.0, sz = 0.0;
+        if ((K.forces & PDQ_F_COULOMB) && g < end) {
+            const int T = (int)((end - o + 31) / 32), per = (T + R - 1) / R;
+            const int c1 = (r + 1) * per < T ? (r + 1) * per : T;
+#pragma unroll 4
+            for (int c = r * per; c < c1; ++c) {
+                const double* part = A.part + (int64_t)(c * 3) * A.cap + g;
+                sx += part[0]; sy += part[A.cap]; sz += part[2 * A.cap];
+            }
+        }
+        for (int q = 1; q < R; ++q) {
+            const double x = __shfl_sync(0xffffffffu, sx, lane % kTilePart + q * kTilePart);
+            const double y = __shfl_sync(0xffffffffu, sy, lane % kTilePart + q * kTilePart);
+            const double z = __shfl_sync(0xffffffffu, sz, lane % kTilePart + q * kTilePart);
+            if (r == 0) { sx += x; sy += y; sz += z; }
+        }
+        int cls = -1;
+        bool was_alive = false, dep = false;
+        if (r == 0 && g < end) local_update<PDQ_FP64>(A, g, sx, sy, sz, A.params[s], cls, was_alive, dep);
+        __syncwarp();
+        if (step >= K.window_start) {
+            const unsigned live = __ballot_sync(0xffffffffu, was_alive), dm = __ballot_sync(0xffffffffu, dep);
+            if (live) {
+                for (int c = 0; c < C; ++c) {
+                    const unsigned m = __ballot_sync(0xffffffffu, cls == c);
+                    const unsigned na = __popc(m & live), nd = __popc(m & dm);
+                    if (lane == 0) {
+                        if (na) atomicAdd(&A.n_alive[(int64_t)s * C + c], (unsigned long long)na);
+                        if (nd) atomicAdd(&A.n_dep[(int64_t)s * C + c], (unsigned long long)nd);
+                    }
+                }
+            }
+        }
+    }
+    if (lane == 0) {
+        __threadfence();
+        const unsigned long long prev = atomicAdd((unsigned long long*)&A.ctl[CTL_DONE], 1ull);
+        if (prev == gridDim.x - 1) {   // last CTA: advance the step
+            A.ctl[CTL_DONE] = 0;
+            A.ctl[CTL_STEP] = step + 1;
+            __threadfence();
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Work items: samples ordered by live count (largest first), JS items per i-tile
 // (one per j-chunk; JS = 1 unless the FP64 j-split is on), item.y = tile * JS + chunk.
@@ -1802,6 +1954,11 @@ static int dispatch_step(int prec, int NT, int variant, bool contact, const Step
         return PDQ_ERR_INVALID_ARG;
     }
     if (prec == PDQ_FP64) {
+        if (NT == 32 && A.jsplit > 1 && (int64_t)A.jsplit * 32 >= A.cap) {
+            if (A.K.forces & PDQ_F_COULOMB) k_pairs_tiles64<<<dim3((unsigned)(A.max_items / A.jsplit), (unsigned)(A.jsplit / 2 + 1)), 32 * kTileWarps, 0, s>>>(A);
+            k_update_tiles64<<<(unsigned)(A.max_items / A.jsplit * (32 / kTilePart)), 32, 0, s>>>(A);
+            return PDQ_OK;
+        }
         if (NT == 32) return launch_step<PDQ_FP64, 32, 1, 0>(A, s);
         if (NT == 64) return launch_step<PDQ_FP64, 64, 1, 0>(A, s);
         if (NT == 128) return launch_step<PDQ_FP64, 128, 1, 0>(A, s);
@@ -1829,9 +1986,11 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 // particles there are; when the i-tiles alone give fewer, each tile's pair sum is
 // spread over JS work items (j-chunks of at least one j-tile).  MIXED never splits
 // (its batches have thousands of tiles); neither do contact runs.
-static int j_split(const pdq_state* st, int TI, bool contact = false) {
+static int j_split(const pdq_state* st, int TI, bool contact = false, bool coarse = false) {
     if (st->precision != PDQ_FP64 || contact) return 1;
     const int64_t cap = st->capacity > 0 ? st->capacity : 1;
+    // up to 2,048 particles at 32 threads: one tile per chunk, summed by tile pairs (k_pairs_tiles64)
+    if (TI == 32 && cap <= 2048 && !coarse) return (int)((cap + 31) / 32);
     const int64_t tile_warps = (cap + TI - 1) / TI * ((TI + 31) / 32);
     int64_t js = (1024 + tile_warps - 1) / tile_warps;
     const int64_t max_js = (cap + TI - 1) / TI;       // chunks are whole j-tiles of TI particles
@@ -1863,7 +2022,7 @@ static int newton_chunks(const pdq_state* st, int TI, bool coarse) {
 static void workspace_layout(const pdq_state* st, int TI, size_t* items_bytes, size_t* total,
                              size_t* cnt_off = nullptr, size_t* part_off = nullptr, bool contact = false,
                              size_t* acc_off = nullptr, bool newton = false, bool coarse = false) {
-    const int JS = newton ? newton_chunks(st, TI, coarse) : j_split(st, TI, contact);
+    const int JS = newton ? newton_chunks(st, TI, coarse) : j_split(st, TI, contact, coarse);
     const int64_t max_tiles = st->capacity / TI + st->n_samples + 1;
     *items_bytes = align256(sizeof(int2) * (size_t)max_tiles * JS);
     *total = *items_bytes + align256(sizeof(int32_t) * (size_t)st->n_samples);
@@ -2045,12 +2204,12 @@ int step_impl(const pdq_field* field, const pdq_phys* phys, pdq_state* st, const
         }
     }
     bool coarse = false;
-    if (newton && st->precision == PDQ_FP64 && workspace_bytes < need) {      // likewise for fewer chunks
+    if (!ext && st->precision == PDQ_FP64 && workspace_bytes < need) {      // likewise for fewer chunks
         coarse = true;
         workspace_layout(st, NT * U, &items_bytes, &need, &cnt_off, &part_off, contact, &acc_off, newton, coarse);
     }
     if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255)) return PDQ_ERR_WORKSPACE;
-    const int JS = newton ? newton_chunks(st, NT * U, coarse) : j_split(st, NT * U, contact || ext);
+    const int JS = newton ? newton_chunks(st, NT * U, coarse) : j_split(st, NT * U, contact || ext, coarse);
     if (n_steps == 0) return PDQ_OK;
     StepArgs A;
     memset(&A, 0, sizeof(A));

@@ -281,6 +281,26 @@ def test_fp64_newton_pairs_large_samples(pdq, fields, counts, block):
     assert np.sqrt(float(err / ref)) <= 24 * 2.0 ** -53
 
 
+@pytest.mark.parametrize("counts", [[1], [31], [32, 0, 33], [700, 5, 129], [2048], [2049]])
+def test_fp64_tile_pairs_of_small_samples(pdq, fields, counts):
+    # 32 threads and up to 2,048 particles: sums by pairs of 32-particle tiles (one tile, a partial one, an even
+    # and an odd number, several samples), and the first size past it; one step at the one-step bar, 12 with
+    # compaction at the bar of 50, and the same bits on a second run
+    prm, off = PRM3[:len(counts)], np.r_[0, np.cumsum(counts)]
+    st, tally, ost, nd, na = _run_both(pdq, fields, 0, counts, ST3, prm, 1, {}, block=32)
+    assert _compare_by_id(st, ost, off, 1e-12, 1e-12) > 0
+    assert np.array_equal(tally.n_dep.cpu().numpy(), nd) and np.array_equal(tally.n_alive.cpu().numpy(), na)
+    runs = [_run_both(pdq, fields, 0, counts, ST3, prm, 12, {"compact_every": 5}, block=32) for _ in range(2)]
+    st, tally, ost, nd, na = runs[0]
+    assert _compare_by_id(st, ost, off, 1e-9, 1e-9) > 0
+    assert np.array_equal(tally.n_dep.cpu().numpy(), nd) and np.array_equal(tally.n_alive.cpu().numpy(), na)
+    n = st.count.cpu().numpy()
+    offs = st.offset.cpu().numpy()
+    for a, b in zip(runs[0][0].current()[:2], runs[1][0].current()[:2]):
+        for k in range(len(counts)):
+            assert torch.equal(a[offs[k]:offs[k] + n[k]], b[offs[k]:offs[k] + n[k]])
+
+
 @pytest.mark.parametrize("variant", [0, 3])
 def test_fp64_rebound_parity(pdq, fields, variant):
     # Rebounding particles bounce inside the stiff vdW zone (accelerations ~1e4 wall units),
