@@ -475,7 +475,7 @@ template <int P, int NT, bool SUMS = false>
 __global__ void __launch_bounds__(NT) k_adj_forward(const AdjArgs A) {
     typedef typename Real<P>::T T;
     typedef typename Real<P>::T4 T4;
-    constexpr int U = adj_ilp<P>();          // particles per thread (ILP over the shared j-tile)
+    constexpr int U = SUMS ? 1 : adj_ilp<P>();   // particles per thread (ILP over the shared j-tile)
     __shared__ __align__(32) unsigned char smem_raw[NT * 32];
     T4* sj = reinterpret_cast<T4*>(smem_raw);
     const int s = blockIdx.y, tid = threadIdx.x;
@@ -1258,6 +1258,7 @@ static int adjoint_impl(const pdq_field* field, const pdq_phys* phys, const pdq_
     if (newton && (nmax + 4 * NTN - 1) / (4 * NTN) > 65535) return PDQ_ERR_UNSUPPORTED;
     constexpr int US = 12;   // forward sums: 12 particles per thread (as the step's Newton kernel)
     const dim3 grid_sums((unsigned)A.S, (unsigned)((nmax + US * NTN - 1) / (US * NTN)));
+    const dim3 grid_local((unsigned)((nmax + NT - 1) / NT), (unsigned)A.S);     // given sums: one particle per thread
     const dim3 grid_vjp((unsigned)A.S, (unsigned)((nmax + 4 * NTN - 1) / (4 * NTN)));
     // one forward step; `recompute`: a step of the reverse sweep's segment recompute, which takes
     // the stored sums when there are any
@@ -1270,7 +1271,7 @@ static int adjoint_impl(const pdq_field* field, const pdq_phys* phys, const pdq_
                 if (e != cudaSuccess) return e;
                 k_adj_sums_sym<NTN, US><<<grid_sums, NTN, 0, s>>>(A);
             }
-            k_adj_forward<PDQ_MIXED, NT, true><<<grid, NT, 0, s>>>(A);
+            k_adj_forward<PDQ_MIXED, NT, true><<<grid_local, NT, 0, s>>>(A);
             A.acc4 = acc_scratch;
         } else if (mixed) {
             k_adj_forward<PDQ_MIXED, NT><<<grid, NT, 0, s>>>(A);
@@ -1305,6 +1306,13 @@ static int adjoint_impl(const pdq_field* field, const pdq_phys* phys, const pdq_
         return copy_state(from, ck[k]);
     };
     const int nsc = A.S * A.C;
+    // The segment slots hold segment `held` (-1: none): the forward sweep leaves the last one there, so the
+    // reverse sweep does not recompute it.  A reverse-only call knows by a mark in the scratch cotangents,
+    // which every sweep that overwrites the slots clears.  (20 steps, K = 10, 16 x 2,048 particles: a quarter
+    // of the pair sums of forward + reverse; all of the recompute when K covers the run.)
+    const int64_t n_last = (Ly.n_ck - 1) * K;
+    const int64_t held_mark[4] = {0x706471736567746cLL, n_steps, K, N};
+    int64_t held = -1;
     if (forward) {
         // seed (or load) into segment slot 0, save as checkpoint 0
         A.out = seg[0];
@@ -1321,12 +1329,21 @@ static int adjoint_impl(const pdq_field* field, const pdq_phys* phys, const pdq_
         PDQ_CUDA(cudaMemsetAsync(A.num, 0, sc, s));
         PDQ_CUDA(cudaMemsetAsync(A.den, 0, sc, s));
         PDQ_CUDA(checkpoint(0, seg[0]));
-        // forward sweep: ping-pong between segment slots 0 and 1, checkpoint every K steps
+        // forward sweep: ping-pong between segment slots 0 and 1, checkpoint every K steps; the last
+        // segment goes through all the slots, as the reverse sweep wants it
         if (store) PDQ_CUDA(cudaMemcpyAsync(marker, mark, sizeof(mark), cudaMemcpyHostToDevice, s));
-        for (int64_t n = 0; n < n_steps; ++n) {
+        for (int64_t n = 0; n < n_last; ++n) {
             PDQ_CUDA(fwd(seg[n & 1], seg[(n + 1) & 1], n, 1, false));
-            if ((n + 1) % K == 0 && (n + 1) < n_steps) PDQ_CUDA(checkpoint((n + 1) / K, seg[(n + 1) & 1]));
+            if ((n + 1) % K == 0) PDQ_CUDA(checkpoint((n + 1) / K, seg[(n + 1) & 1]));
         }
+        if (n_last & 1) PDQ_CUDA(copy_state(seg[0], seg[1]));
+        for (int64_t t = 0; n_last + t < n_steps; ++t) PDQ_CUDA(fwd(seg[t], seg[t + 1], n_last + t, 1, false));
+        held = Ly.n_ck - 1;
+        // a later reverse call finds the segment there unless this call's sweep overwrites it
+        if (n_vec == 0 || Ly.n_ck == 1)
+            PDQ_CUDA(cudaMemcpyAsync(scratch[0], held_mark, sizeof(held_mark), cudaMemcpyHostToDevice, s));
+        else
+            PDQ_CUDA(cudaMemsetAsync(scratch[0], 0, sizeof(held_mark), s));
         k_adj_finish<<<(nsc + 255) / 256, 256, 0, s>>>(A.num, A.den, nullptr, nsc, A.K.R, A.K.dt, J, nullptr,
                                                        nullptr);
         PDQ_CUDA(cudaGetLastError());
@@ -1337,6 +1354,13 @@ static int adjoint_impl(const pdq_field* field, const pdq_phys* phys, const pdq_
         PDQ_CUDA(cudaMemcpyAsync(got, marker, sizeof(got), cudaMemcpyDeviceToHost, s));
         PDQ_CUDA(cudaStreamSynchronize(s));
         if (memcmp(got, mark, sizeof(got)) != 0) return PDQ_ERR_INVALID_ARG;
+    }
+    if (!forward) {
+        int64_t got[4];
+        PDQ_CUDA(cudaMemcpyAsync(got, scratch[0], sizeof(got), cudaMemcpyDeviceToHost, s));
+        PDQ_CUDA(cudaStreamSynchronize(s));
+        if (memcmp(got, held_mark, sizeof(got)) == 0) held = Ly.n_ck - 1;
+        if (Ly.n_ck > 1) PDQ_CUDA(cudaMemsetAsync(scratch[0], 0, sizeof(got), s));
     }
     // backward sweeps, one per cotangent vector
     for (int v = 0; v < n_vec; ++v) {
@@ -1350,8 +1374,11 @@ static int adjoint_impl(const pdq_field* field, const pdq_phys* phys, const pdq_
             const int64_t len = std::min<int64_t>(K, n_steps - n0);
             A.qhat = ck_qh[kseg];
             A.cls = ck_cl[kseg];
-            PDQ_CUDA(copy_state(seg[0], ck[kseg]));
-            for (int64_t t = 0; t < len; ++t) PDQ_CUDA(fwd(seg[t], seg[t + 1], n0 + t, 0, true));
+            if (held != kseg) {
+                PDQ_CUDA(copy_state(seg[0], ck[kseg]));
+                for (int64_t t = 0; t < len; ++t) PDQ_CUDA(fwd(seg[t], seg[t + 1], n0 + t, 0, true));
+                held = kseg;
+            }
             for (int64_t t = len - 1; t >= 0; --t) {
                 A.in = seg[t];
                 A.step = n0 + t;

@@ -364,6 +364,36 @@ def test_adjoint_reverse_alone_matches_the_combined_call(pdq):
     assert torch.allclose(p2, p3, rtol=1e-12, atol=1e-14 * float(p1.abs().max()))
 
 
+@pytest.mark.parametrize("steps,K", [(12, 12), (12, 5), (12, 6), (12, 1), (7, 20)])
+def test_adjoint_reverse_takes_the_last_segment_it_finds(pdq, steps, K):
+    # one segment, a short and a full last one, single steps, K beyond the run: a reverse call right after
+    # the forward sweep (segment found in the workspace), one after that (overwritten, unless it is the
+    # only one), and one after a combined call in the same workspace, against separate combined runs
+    c = CASES["A"]
+    field = pdq.Field(pdq.field_desc(**GRID), 0)
+    phys = pdq.phys_default()
+    batch = pdq.Batch(0, COUNTS, c["st"])
+    cfg = pdq.step_cfg(c["dt"], window_start=c["win"], gravity=c["gravity"])
+    prm = pdq.params_tensor(PARAMS)
+    one = _onehot()
+
+    def combined(ws=None):
+        return pdq.adjoint_run_seeded(field, phys, batch, prm, cfg, steps, K, c["eps"], SEED, gbar=one, ws=ws)[1]
+
+    def close(a, b):
+        return torch.allclose(a, b, rtol=1e-12, atol=1e-14 * float(b.abs().max()))
+    # the recomputed segment is the forward sweep's: only the order of double atomics differs
+    want = pdq.adjoint_run_seeded(field, phys, batch, prm, cfg, steps, 3, c["eps"], SEED, gbar=one)[1]
+    ws = pdq.adjoint_workspace(batch.b, steps, K)
+    pdq.adjoint_run_seeded(field, phys, batch, prm, cfg, steps, K, c["eps"], SEED, ws=ws)
+    for _ in range(2):
+        got = pdq.adjoint_reverse(field, phys, batch.b, prm, cfg, steps, K, c["eps"], one, ws)
+        assert torch.allclose(got, want, rtol=1e-9, atol=1e-12 * float(want.abs().max()))
+    first = combined(ws)
+    assert close(first, got) and close(combined(), got)
+    assert close(pdq.adjoint_reverse(field, phys, batch.b, prm, cfg, steps, K, c["eps"], one, ws), got)
+
+
 def test_adjoint_from_state_rejects_zero_charge_scale(pdq):
     c = CASES["A"]
     field = pdq.Field(pdq.field_desc(**GRID), 0)
