@@ -34,12 +34,12 @@
 #include <math.h>
 #include <string.h>
 
-#include "pdq_common.cuh"
+#include "pdq_device.cuh"
 
 namespace pdq {
 
 constexpr double kBoltzmann = 1.380649e-23;   // J/K
-constexpr int kLfThreads = 256;
+constexpr int kLfThreads = 256, kLfThreads64 = 256;   // threads per CTA of the FP32 and the FP64 march
 
 struct LfClass {
     double tau;       // tau_p+ = tau_1+
@@ -103,107 +103,223 @@ struct __align__(16) LfCell {
     T dw, de, dv, a;
 };
 
-// exp(x) - 1 over x, for the FP32 march (x <= 0): Taylor polynomial below
-// |x| = 0.5 (terms to x^8/9!, truncation < 1e-9 relative), the approximate
-// exponential beyond (E - 1 then stays below -0.39, so its relative rounding
-// does not grow).  Returns phi and E = 1 + x phi.
-__device__ __forceinline__ float lf_phi(float x, float* E) {
-    if (x > -0.5f) {
-        float p = 2.7557319e-6f;                  // 1/9!
-        p = fmaf(p, x, 2.4801587e-5f);            // 1/8!
-        p = fmaf(p, x, 1.9841270e-4f);            // 1/7!
-        p = fmaf(p, x, 1.3888889e-3f);            // 1/6!
-        p = fmaf(p, x, 8.3333333e-3f);            // 1/5!
-        p = fmaf(p, x, 4.1666667e-2f);            // 1/4!
-        p = fmaf(p, x, 1.6666667e-1f);            // 1/3!
-        p = fmaf(p, x, 0.5f);                     // 1/2!
-        p = fmaf(p, x, 1.0f);
-        *E = fmaf(x, p, 1.0f);
-        return p;
+// The class's cell table into shared memory, each node evaluated once: chunks of blockDim nodes staged
+// in s_node (the last one carried over), a cell from each neighbouring pair.
+template <typename T>
+__device__ __forceinline__ void lf_table(const LfArgs& A, const LfClass& K, LfCell<T>* cell, T* t_h, LfNode* s_node,
+                                         double* s_sigma) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    for (int c0 = 0; c0 < A.n_y; c0 += nt) {
+        const int k = c0 + tid;                        // node k; cell k - 1 lies between nodes k - 1 and k
+        if (k < A.n_y) s_node[tid + 1] = lf_node(A, K, k);
+        __syncthreads();
+        if (k < A.n_y && k > 0) {
+            const LfNode lo = s_node[tid], hi = s_node[tid + 1];
+            const double dy = hi.y - lo.y;
+            LfCell<T> e;
+            e.dw = (T)(hi.w - lo.w);
+            e.de = (T)(hi.inv_y - lo.inv_y);
+            e.dv = (T)(hi.psi - lo.psi);
+            e.a = (T)(dy / K.tau);
+            cell[k - 1] = e;
+            t_h[k - 1] = (T)(dy / (0.5 * (lo.D + hi.D)));
+        }
+        if (k == 0) *s_sigma = sqrt(K.resp * lf_var_at(A, s_node[1].y) + K.thermal);
+        __syncthreads();
+        if (tid == 0) s_node[0] = s_node[nt];
+        __syncthreads();
     }
-    const float e = __expf(x);
-    *E = e;
-    return __fdividef(e - 1.0f, x);
 }
 
-// T = double: the march in FP64.  T = float (PDQ_MIXED): the cell table and the
-// march in FP32 (root by x rsqrt(x) and an approximate division, the cell's
-// exponential by lf_phi; Q summed with Kahan compensation), the wall
-// condition and the final ratio in FP64.  Each CTA builds its class's table
-// once and walks blocks of 256 samples blockIdx.x, blockIdx.x + gridDim.x, ...
-template <typename T>
-__global__ void __launch_bounds__(kLfThreads) k_lf_vdep(const LfArgs A) {
+// kinetic wall condition: one-way flux of a Gaussian velocity (mean V_w, sd sigma), FP64
+__device__ __forceinline__ double lf_result(double v_w, double sg, double P, double Q) {
+    const double u = -v_w;
+    const double M = u / (1.4142135623730951 * sg);
+    const double Kw = -(0.5 * u * (1.0 + erf(M)) + sg * exp(-M * M) * 0.3989422804014327);
+    return -Kw / (P - Kw * Q);
+}
+
+// The march in FP64, one sample per thread.  Bound by the FP64 pipe, so the library's square root,
+// divisions and expm1 give way to the hardware's 2^-20 estimates with one cubic correction each (a + s
+// and x are sums of squares: no special values), and (e^x - 1)/x to its Taylor polynomial below |x| = 1/2
+// (degree 6 below 2^-6, where half of the cells lie, else 13; truncation < 2^-56).  65,536 samples x 10
+// classes: 127 ms (155 ms with the library's functions); error against 64 bits 9.3e-16 (9.6e-16).
+// x = a^2 + 2c > 0:
+__device__ __forceinline__ double lf_sqrt(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double t = x * y, e = __fma_rn(-t, y, 1.0);
+    return __fma_rn(t, e * __fma_rn(e, 0.375, 0.5), t);
+}
+__device__ __forceinline__ double lf_div(double n, double d) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    const double e = __fma_rn(-d, r, 1.0);
+    r = __fma_rn(r, __fma_rn(e, e, e), r);
+    const double q = n * r;
+    return __fma_rn(__fma_rn(-d, q, n), r, q);
+}
+__device__ __forceinline__ double lf_phi64(double x, double* E) {
+    if (x > -0.5) {
+        double p = 1.0 / 5040.0;
+        if (x <= -0.015625) {
+            p = 1.0 / 87178291200.0;                              // 1/14!
+            p = __fma_rn(p, x, 1.0 / 6227020800.0);
+            p = __fma_rn(p, x, 1.0 / 479001600.0);
+            p = __fma_rn(p, x, 1.0 / 39916800.0);
+            p = __fma_rn(p, x, 1.0 / 3628800.0);
+            p = __fma_rn(p, x, 1.0 / 362880.0);
+            p = __fma_rn(p, x, 1.0 / 40320.0);
+            p = __fma_rn(p, x, 1.0 / 5040.0);
+        }
+        p = __fma_rn(p, x, 1.0 / 720.0);
+        p = __fma_rn(p, x, 1.0 / 120.0);
+        p = __fma_rn(p, x, 1.0 / 24.0);
+        p = __fma_rn(p, x, 1.0 / 6.0);
+        p = __fma_rn(p, x, 0.5);
+        p = __fma_rn(p, x, 1.0);
+        *E = __fma_rn(x, p, 1.0);
+        return p;
+    }
+    const double em = exp(x) - 1.0;
+    *E = 1.0 + em;
+    return lf_div(em, x);
+}
+
+constexpr int kLfStride = 32;   // cells between two looks at P
+
+__global__ void __launch_bounds__(kLfThreads64) k_lf_vdep64(const LfArgs A) {
     extern __shared__ __align__(16) unsigned char lf_smem[];
     const int c = blockIdx.y;
     const LfClass K = A.cls[c];
     const int ncell = A.n_y - 1;
-    LfCell<T>* cell = reinterpret_cast<LfCell<T>*>(lf_smem);
-    T* t_h = reinterpret_cast<T*>(cell + ncell);
+    LfCell<double>* cell = reinterpret_cast<LfCell<double>*>(lf_smem);
+    double* t_h = reinterpret_cast<double*>(cell + ncell);
+    __shared__ LfNode s_node[kLfThreads64 + 1];
     __shared__ double s_sigma;
-    for (int k = threadIdx.x; k < ncell; k += blockDim.x) {
-        const LfNode lo = lf_node(A, K, k), hi = lf_node(A, K, k + 1);
-        const double dy = hi.y - lo.y;
-        LfCell<T> e;
-        e.dw = (T)(hi.w - lo.w);
-        e.de = (T)(hi.inv_y - lo.inv_y);
-        e.dv = (T)(hi.psi - lo.psi);
-        e.a = (T)(dy / K.tau);
-        cell[k] = e;
-        t_h[k] = (T)(dy / (0.5 * (lo.D + hi.D)));
-        if (k == 0) s_sigma = sqrt(K.resp * lf_var_at(A, lo.y) + K.thermal);
-    }
-    __syncthreads();
+    lf_table(A, K, cell, t_h, s_node, &s_sigma);
     const double sg = s_sigma;
-    const int64_t nblk = (A.S + kLfThreads - 1) / kLfThreads;
+    const int64_t nblk = (A.S + kLfThreads64 - 1) / kLfThreads64;
     for (int64_t b = blockIdx.x; b < nblk; b += gridDim.x) {
-        const int64_t s = b * kLfThreads + threadIdx.x;
-        if (s >= A.S) continue;
-        const double xi = A.params[s].xi, zeta = A.params[s].zeta;
-        const T ae = (T)(-K.ce * xi * xi), av = (T)(-K.cv * zeta);
-        const T half = (T)0.5, two = (T)2, zero = (T)0, one = (T)1;
-        T v_out = zero;   // V at node k + 1 (the axis: 0)
-        T P = one, Q = zero, Qc = zero;
-        for (int k = ncell - 1; k >= 0; --k) {
-            const LfCell<T> e = cell[k];
-            const T h = t_h[k];
-            // momentum: implicit drag, root <= 0 of V^2/2 - a V = c
-            const T c2 = half * v_out * v_out + e.dw + (ae * e.de + av * e.dv);
-            T v_in = zero;
-            T G, E;
-            if constexpr (sizeof(T) == sizeof(double)) {
-                if (c2 > zero) v_in = -two * c2 / (e.a + sqrt(fma(e.a, e.a, two * c2)));
-                // continuity: exact cell solution with the cell-mean V and D
-                const T vm = half * (v_in + v_out);
-                const T am = vm * h;
-                G = h;
-                E = one;
-                if (am != zero) {
-                    const T em = expm1(am);
-                    G = em / vm;
-                    E = one + em;
-                }
-                Q = fma(P, G, Q);
+        const int64_t s = b * kLfThreads64 + threadIdx.x;
+        const pdq_sample_params sp = A.params[s < A.S ? s : A.S - 1];      // past the end: a copy, not stored
+        const double ae = -K.ce * sp.xi * sp.xi, av = -K.cv * sp.zeta;
+        double v = 0.0, P = 1.0, Q = 0.0;   // v at node k + 1 (the axis: 0)
+        // momentum: implicit drag, root <= 0 of V^2/2 - a V = c
+        auto momentum = [&](const LfCell<double>& e) {
+            const double c2 = __fma_rn(0.5 * v, v, e.dw) + __fma_rn(ae, e.de, av * e.dv);
+            return c2 > 0.0 ? lf_div(-2.0 * c2, e.a + lf_sqrt(__fma_rn(e.a, e.a, 2.0 * c2))) : 0.0;
+        };
+        for (int k1 = ncell; k1 > 0;) {
+            const int k0 = k1 > kLfStride ? k1 - kLfStride : 0;
+            if (__all_sync(0xffffffffu, P == 0.0)) {
+                // the flux solution is complete (P and every further P G vanish): momentum alone
+                for (int k = k1 - 1; k >= k0; --k) v = momentum(cell[k]);
             } else {
-                if (c2 > zero) {
-                    const float x = fmaf(e.a, e.a, two * c2);
-                    v_in = __fdividef(-two * c2, e.a + x * rsqrtf(x));
+                for (int k = k1 - 1; k >= k0; --k) {
+                    const double h = t_h[k], vi = momentum(cell[k]);
+                    // continuity: exact cell solution with the cell-mean V and D
+                    double E;
+                    const double phi = lf_phi64((0.5 * (vi + v)) * h, &E);
+                    Q = __fma_rn(P, h * phi, Q);
+                    P *= E;
+                    v = vi;
                 }
-                const float am = half * (v_in + v_out) * h;   // <= 0
-                G = h * lf_phi(am, &E);
-                const T yq = fma(P, G, -Qc);
-                const T tq = Q + yq;
-                Qc = (tq - Q) - yq;
-                Q = tq;
             }
-            P *= E;
-            v_out = v_in;
+            k1 = k0;
         }
-        // kinetic wall condition: one-way flux of a Gaussian velocity (mean V_w, sd sigma), FP64
-        const double u = -(double)v_out;
-        const double M = u / (1.4142135623730951 * sg);
-        const double Kw = -(0.5 * u * (1.0 + erf(M)) + sg * exp(-M * M) * 0.3989422804014327);
-        const double Qd = (double)Q - (double)Qc;
-        A.vdep[s * A.C + c] = -Kw / ((double)P - Kw * Qd);
+        if (s < A.S) A.vdep[s * A.C + c] = lf_result(v, sg, P, Q);
+    }
+}
+
+// The march in FP32 (PDQ_MIXED), two samples per thread as packed f32x2: the cell table and the march
+// in FP32 (root by x rsqrt(x) and an approximate division; Q summed with Kahan compensation), the wall
+// condition and the final ratio in FP64.  Per item and cell 26 FMA-pipe operations issue as 13 packed
+// instructions, beside two table loads per pair of items and the scalar square roots and divisions.
+// (e^x - 1)/x is its Taylor polynomial below |x| = 0.5 (terms to x^8/9!, truncation < 1e-9 relative), the
+// approximate exponential beyond (E - 1 then stays below -0.39, so its relative rounding does not grow).
+// 262,144 samples x 10 classes: 8.0 ms, bit for bit the results of the scalar march (10.1 ms, bound by issue).
+__global__ void __launch_bounds__(kLfThreads) k_lf_vdep32(const LfArgs A) {
+    extern __shared__ __align__(16) unsigned char lf_smem[];
+    const int c = blockIdx.y;
+    const LfClass K = A.cls[c];
+    const int ncell = A.n_y - 1;
+    LfCell<float>* cell = reinterpret_cast<LfCell<float>*>(lf_smem);
+    float* t_h = reinterpret_cast<float*>(cell + ncell);
+    __shared__ LfNode s_node[kLfThreads + 1];
+    __shared__ double s_sigma;
+    lf_table(A, K, cell, t_h, s_node, &s_sigma);
+    const double sg = s_sigma;
+    constexpr int kPer = 2 * kLfThreads;
+    const int64_t nblk = (A.S + kPer - 1) / kPer;
+    const f2 half = f2_pack(0.5f, 0.5f);
+    for (int64_t b = blockIdx.x; b < nblk; b += gridDim.x) {
+        const int64_t s0 = b * kPer + threadIdx.x, s1 = s0 + kLfThreads;
+        const pdq_sample_params p0 = A.params[s0 < A.S ? s0 : A.S - 1], p1 = A.params[s1 < A.S ? s1 : A.S - 1];
+        const f2 ae = f2_pack((float)(-K.ce * p0.xi * p0.xi), (float)(-K.ce * p1.xi * p1.xi));
+        const f2 av = f2_pack((float)(-K.cv * p0.zeta), (float)(-K.cv * p1.zeta));
+        f2 V = 0ull, P = f2_pack(1.f, 1.f), Q = 0ull, NC = 0ull;      // NC: minus the compensation of Q
+        // momentum: implicit drag, root <= 0 of V^2/2 - a V = c
+        auto momentum = [&](const LfCell<float>& e) -> f2 {
+            const f2 a = f2_pack(e.a, e.a);
+            const f2 c2 = f2_add(f2_fma(f2_mul(half, V), V, f2_pack(e.dw, e.dw)),
+                                 f2_fma(ae, f2_pack(e.de, e.de), f2_mul(av, f2_pack(e.dv, e.dv))));
+            const f2 cc = f2_add(c2, c2), x = f2_fma(a, a, cc);
+            float ca, cb, xa, xb, da, db;
+            f2_unpack(cc, ca, cb);
+            f2_unpack(x, xa, xb);
+            f2_unpack(f2_fma(x, f2_pack(rsqrtf(xa), rsqrtf(xb)), a), da, db);
+            return f2_pack(ca > 0.f ? __fdividef(-ca, da) : 0.f, cb > 0.f ? __fdividef(-cb, db) : 0.f);
+        };
+        for (int k1 = ncell; k1 > 0;) {
+            const int k0 = k1 > kLfStride ? k1 - kLfStride : 0;
+            float Pa, Pb;
+            f2_unpack(P, Pa, Pb);
+            if (__all_sync(0xffffffffu, Pa == 0.f && Pb == 0.f)) {
+                // the flux solution is complete (P and every further P G vanish): momentum alone
+                for (int k = k1 - 1; k >= k0; --k) V = momentum(cell[k]);
+            } else {
+                for (int k = k1 - 1; k >= k0; --k) {
+                    const f2 h = f2_pack(t_h[k], t_h[k]), Vi = momentum(cell[k]);
+                    // continuity: exact cell solution with the cell-mean V and D
+                    const f2 am = f2_mul(f2_mul(half, f2_add(Vi, V)), h);      // <= 0
+                    f2 p = f2_dup(2.7557319e-6f);                              // 1/9!
+                    p = f2_fma(p, am, f2_dup(2.4801587e-5f));
+                    p = f2_fma(p, am, f2_dup(1.9841270e-4f));
+                    p = f2_fma(p, am, f2_dup(1.3888889e-3f));
+                    p = f2_fma(p, am, f2_dup(8.3333333e-3f));
+                    p = f2_fma(p, am, f2_dup(4.1666667e-2f));
+                    p = f2_fma(p, am, f2_dup(1.6666667e-1f));
+                    p = f2_fma(p, am, f2_dup(0.5f));
+                    p = f2_fma(p, am, f2_dup(1.0f));
+                    f2 E = f2_fma(am, p, f2_dup(1.0f));
+                    float ma, mb;
+                    f2_unpack(am, ma, mb);
+                    if (!(ma > -0.5f && mb > -0.5f)) {
+                        float ea, eb, pa, pb;
+                        f2_unpack(E, ea, eb);
+                        f2_unpack(p, pa, pb);
+                        if (!(ma > -0.5f)) { ea = __expf(ma); pa = __fdividef(ea - 1.0f, ma); }
+                        if (!(mb > -0.5f)) { eb = __expf(mb); pb = __fdividef(eb - 1.0f, mb); }
+                        E = f2_pack(ea, eb);
+                        p = f2_pack(pa, pb);
+                    }
+                    const f2 y = f2_fma(P, f2_mul(h, p), NC), t = f2_add(Q, y);
+                    NC = f2_sub(y, f2_sub(t, Q));
+                    Q = t;
+                    P = f2_mul(P, E);
+                    V = Vi;
+                }
+            }
+            k1 = k0;
+        }
+        float va, vb, Pa, Pb, Qa, Qb, na, nb;
+        f2_unpack(V, va, vb);
+        f2_unpack(P, Pa, Pb);
+        f2_unpack(Q, Qa, Qb);
+        f2_unpack(NC, na, nb);
+        if (s0 < A.S) A.vdep[s0 * A.C + c] = lf_result((double)va, sg, (double)Pa, (double)Qa + (double)na);
+        if (s1 < A.S) A.vdep[s1 * A.C + c] = lf_result((double)vb, sg, (double)Pb, (double)Qb + (double)nb);
     }
 }
 
@@ -267,21 +383,20 @@ static size_t lf_shared_bytes(int32_t n_y, size_t elem) { return (size_t)5 * (si
 
 // One wave: as many CTAs per class as fit on the GPU at once (its SMs times the
 // resident CTAs per SM, divided among the classes), each building its class's
-// table once and walking ceil(blocks / CTAs) sample blocks.
-template <typename T>
-static int launch_lf(const LfArgs& A, pdq_stream_t stream) {
-    const size_t smem = lf_shared_bytes(A.n_y, sizeof(T));
-    PDQ_CUDA(cudaFuncSetAttribute(k_lf_vdep<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+// table once and walking its share of the blocks of `per` samples.
+static int launch_lf(void (*kernel)(LfArgs), int threads, int per, size_t elem, const LfArgs& A, pdq_stream_t stream) {
+    const size_t smem = lf_shared_bytes(A.n_y, elem);
+    PDQ_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int dev = 0, sms = 0, per_sm = 0;
     PDQ_CUDA(cudaGetDevice(&dev));
     PDQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    PDQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lf_vdep<T>, kLfThreads, smem));
-    const int64_t nblk = (A.S + kLfThreads - 1) / kLfThreads;
+    PDQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
+    const int64_t nblk = (A.S + per - 1) / per;
     int64_t gx = (int64_t)(sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1) / A.C;
     if (gx < 1) gx = 1;
     if (gx > nblk) gx = nblk;
     const dim3 grid((unsigned)gx, (unsigned)A.C);
-    k_lf_vdep<T><<<grid, kLfThreads, smem, (cudaStream_t)stream>>>(A);
+    kernel<<<grid, threads, smem, (cudaStream_t)stream>>>(A);
     PDQ_CUDA(cudaGetLastError());
     return PDQ_OK;
 }
@@ -338,6 +453,6 @@ extern "C" int pdq_lf_vdep(const pdq_field* field, const pdq_phys* phys, const p
     A.var = var;
     A.params = params;
     A.vdep = vdep;
-    if (lf->precision == PDQ_FP64) return launch_lf<double>(A, stream);
-    return launch_lf<float>(A, stream);
+    if (lf->precision == PDQ_FP64) return launch_lf(k_lf_vdep64, kLfThreads64, kLfThreads64, sizeof(double), A, stream);
+    return launch_lf(k_lf_vdep32, kLfThreads, 2 * kLfThreads, sizeof(float), A, stream);
 }

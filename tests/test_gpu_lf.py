@@ -238,3 +238,19 @@ def test_two_model_study_with_the_eulerian_model(pdq):
     else:
         assert 2 <= r2["m"][0] <= r2["m"][1] and np.all(np.isfinite(r2["mean"]))
         assert -1.0 <= r2["pilot"]["rho"][0] <= 1.0 and np.all(r2["pilot"]["w_ms_per_sample"] > 0)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("S,n_y", [(1, 33), (255, 34), (257, 65), (511, 3), (513, 97), (769, 700)])
+def test_vdep_at_the_edges_of_blocks_and_cell_runs(pdq, fields, S, n_y, precision):
+    # sample counts around a CTA's 256 (FP64) and 512 samples (FP32, two per thread); cells around the runs
+    # of 32 between two looks at the flux solution; large classes, whose flux solution ends well off the
+    # wall, beside the smallest, whose never does.  The bars of this file.
+    f, of, var_o = fields[(64, 32, 64)]
+    st = [0.01, 1.0, 100.0]
+    prm = _params(S, S)
+    var = pdq.lf_fluid_variance(f)
+    got = pdq.lf_vdep(f, pdq.phys_default(), pdq.lf_desc(n_y=n_y, precision=precision), var, st,
+                      pdq.params_tensor(prm)).cpu().numpy()
+    ref = lfo.lf_vdep(oracle.phys(), st, prm, var_o, of.r_plus, of.beta, lfo.lf_params(n_y=n_y))
+    assert np.max(np.abs(got / ref - 1)) < (RTOL if precision == 0 else RTOL_MIXED)
