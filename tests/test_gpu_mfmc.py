@@ -73,6 +73,24 @@ def test_bootstrap_intervals_match_oracle(pdq):
     assert np.all(lo <= hi)
 
 
+@pytest.mark.parametrize("C,d", [(1, 1), (31, 2), (32, 3), (33, 4), (70, 5)])
+def test_sums_over_blocks_of_outputs(pdq, C, d):
+    # outputs around the 32 of a block, every compiled number of inputs and a general one, three models
+    # with prefixes of 2 groups, of one more than a cluster's rows, and equal ones; bars as above
+    rng = np.random.default_rng(C)
+    m, alpha, B, seed = [2, 33, 33], [1.0, 0.9, 0.4], 5, 7
+    base = rng.standard_normal((40, d + 2, C)) + 3.0
+    ys = [base[:2], base[:33] + 0.3 * rng.standard_normal((33, d + 2, C)), base + 0.5 * rng.standard_normal(base.shape)]
+    out = pdq.mfmc_sobol([torch.tensor(y, device="cuda") for y in ys], m, alpha, n_boot=B, seed=seed)
+    sm, st, mean, var = mfmc.mfmc_sobol([y[:n] for y, n in zip(ys, m)], m, alpha)
+    assert np.allclose(out["mean"], mean, rtol=1e-12) and np.allclose(out["var"], var, rtol=1e-10)
+    assert np.allclose(out["s_main"], sm, rtol=1e-9, atol=1e-11)
+    assert np.allclose(out["s_total"], st, rtol=1e-9, atol=1e-11)
+    ci_m, ci_t = mfmc.bootstrap_ci([y[:n] for y, n in zip(ys, m)], m, alpha, lambda b: oracle.boot_indices(seed, b, m), B)
+    assert np.allclose(out["s_main_ci"], ci_m, rtol=1e-8, atol=1e-10)
+    assert np.allclose(out["s_total_ci"], ci_t, rtol=1e-8, atol=1e-10)
+
+
 def test_dgsm_bounds_match_oracle(pdq):
     rng = np.random.default_rng(14)
     X = rng.uniform(-np.pi, np.pi, (5000, 3))
