@@ -39,7 +39,7 @@
 namespace pdq {
 
 constexpr double kBoltzmann = 1.380649e-23;   // J/K
-constexpr int kLfThreads = 256, kLfThreads64 = 256;   // threads per CTA of the FP32 and the FP64 march
+constexpr int kLfThreads = 512, kLfThreads64 = 256;   // threads per CTA of the FP32 and the FP64 march
 
 struct LfClass {
     double tau;       // tau_p+ = tau_1+
@@ -96,12 +96,14 @@ __device__ __forceinline__ LfNode lf_node(const LfArgs& A, const LfClass& K, int
 }
 
 // One cell of the class table: differences of R v_f'^2 and of the two potential
-// shapes across the cell and dy/tau (16 B in FP32, one shared-memory load; the
-// cell's dy/D_m sits in a second array).
+// shapes across the cell and dy/tau (the cell's dy/D_m sits in a second array).  T:
+// double, or f2 with the FP32 value in both halves, as the packed march reads it.
 template <typename T>
 struct __align__(16) LfCell {
     T dw, de, dv, a;
 };
+__device__ __forceinline__ void lf_put(double& t, double v) { t = v; }
+__device__ __forceinline__ void lf_put(f2& t, double v) { t = f2_dup((float)v); }
 
 // The class's cell table into shared memory, each node evaluated once: chunks of blockDim nodes staged
 // in s_node (the last one carried over), a cell from each neighbouring pair.
@@ -117,12 +119,12 @@ __device__ __forceinline__ void lf_table(const LfArgs& A, const LfClass& K, LfCe
             const LfNode lo = s_node[tid], hi = s_node[tid + 1];
             const double dy = hi.y - lo.y;
             LfCell<T> e;
-            e.dw = (T)(hi.w - lo.w);
-            e.de = (T)(hi.inv_y - lo.inv_y);
-            e.dv = (T)(hi.psi - lo.psi);
-            e.a = (T)(dy / K.tau);
+            lf_put(e.dw, hi.w - lo.w);
+            lf_put(e.de, hi.inv_y - lo.inv_y);
+            lf_put(e.dv, hi.psi - lo.psi);
+            lf_put(e.a, dy / K.tau);
             cell[k - 1] = e;
-            t_h[k - 1] = (T)(dy / (0.5 * (lo.D + hi.D)));
+            lf_put(t_h[k - 1], dy / (0.5 * (lo.D + hi.D)));
         }
         if (k == 0) *s_sigma = sqrt(K.resp * lf_var_at(A, s_node[1].y) + K.thermal);
         __syncthreads();
@@ -143,7 +145,8 @@ __device__ __forceinline__ double lf_result(double v_w, double sg, double P, dou
 // divisions and expm1 give way to the hardware's 2^-20 estimates with one cubic correction each (a + s
 // and x are sums of squares: no special values), and (e^x - 1)/x to its Taylor polynomial below |x| = 1/2
 // (degree 6 below 2^-6, where half of the cells lie, else 13; truncation < 2^-56).  65,536 samples x 10
-// classes: 127 ms (155 ms with the library's functions); error against 64 bits 9.3e-16 (9.6e-16).
+// classes: 121 ms (157 ms with the library's functions; 127 ms with the samples dealt out by whole CTAs);
+// error against 64 bits 9.4e-16 (1.1e-15).
 // x = a^2 + 2c > 0:
 __device__ __forceinline__ double lf_sqrt(double x) {
     double y;
@@ -199,9 +202,12 @@ __global__ void __launch_bounds__(kLfThreads64) k_lf_vdep64(const LfArgs A) {
     __shared__ double s_sigma;
     lf_table(A, K, cell, t_h, s_node, &s_sigma);
     const double sg = s_sigma;
-    const int64_t nblk = (A.S + kLfThreads64 - 1) / kLfThreads64;
-    for (int64_t b = blockIdx.x; b < nblk; b += gridDim.x) {
-        const int64_t s = b * kLfThreads64 + threadIdx.x;
+    // the class's samples by runs of 32, dealt out over the CTAs first and the warps then, so that the last,
+    // partial round leaves every SM the same work
+    const int64_t nrun = (A.S + 31) / 32;
+    for (int64_t b = (threadIdx.x >> 5) * (int64_t)gridDim.x + blockIdx.x; b < nrun;
+         b += (int64_t)(kLfThreads64 / 32) * gridDim.x) {
+        const int64_t s = b * 32 + (threadIdx.x & 31);
         const pdq_sample_params sp = A.params[s < A.S ? s : A.S - 1];      // past the end: a copy, not stored
         const double ae = -K.ce * sp.xi * sp.xi, av = -K.cv * sp.zeta;
         double v = 0.0, P = 1.0, Q = 0.0;   // v at node k + 1 (the axis: 0)
@@ -232,44 +238,50 @@ __global__ void __launch_bounds__(kLfThreads64) k_lf_vdep64(const LfArgs A) {
     }
 }
 
+// The approximate division without its fix-up for denormal divisors.
+__device__ __forceinline__ float lf_div_ftz(float a, float b) {
+    float q;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(q) : "f"(a), "f"(b));
+    return q;
+}
+
 // The march in FP32 (PDQ_MIXED), two samples per thread as packed f32x2: the cell table and the march
 // in FP32 (root by x rsqrt(x) and an approximate division; Q summed with Kahan compensation), the wall
 // condition and the final ratio in FP64.  Per item and cell 26 FMA-pipe operations issue as 13 packed
 // instructions, beside two table loads per pair of items and the scalar square roots and divisions.
 // (e^x - 1)/x is its Taylor polynomial below |x| = 0.5 (terms to x^8/9!, truncation < 1e-9 relative), the
 // approximate exponential beyond (E - 1 then stays below -0.39, so its relative rounding does not grow).
-// 262,144 samples x 10 classes: 8.0 ms, bit for bit the results of the scalar march (10.1 ms, bound by issue).
+// 262,144 samples x 10 classes: 6.25 ms, bit for bit the results of the scalar march (10.1 ms, bound by
+// issue); 8.0 ms with the table in single floats, 256-thread CTAs and the denormal fix-ups.
 __global__ void __launch_bounds__(kLfThreads) k_lf_vdep32(const LfArgs A) {
     extern __shared__ __align__(16) unsigned char lf_smem[];
     const int c = blockIdx.y;
     const LfClass K = A.cls[c];
     const int ncell = A.n_y - 1;
-    LfCell<float>* cell = reinterpret_cast<LfCell<float>*>(lf_smem);
-    float* t_h = reinterpret_cast<float*>(cell + ncell);
+    LfCell<f2>* cell = reinterpret_cast<LfCell<f2>*>(lf_smem);
+    f2* t_h = reinterpret_cast<f2*>(cell + ncell);
     __shared__ LfNode s_node[kLfThreads + 1];
     __shared__ double s_sigma;
     lf_table(A, K, cell, t_h, s_node, &s_sigma);
     const double sg = s_sigma;
-    constexpr int kPer = 2 * kLfThreads;
-    const int64_t nblk = (A.S + kPer - 1) / kPer;
+    const int64_t nrun = (A.S + 63) / 64;         // runs of 64 samples, dealt out as in the FP64 march
     const f2 half = f2_pack(0.5f, 0.5f);
-    for (int64_t b = blockIdx.x; b < nblk; b += gridDim.x) {
-        const int64_t s0 = b * kPer + threadIdx.x, s1 = s0 + kLfThreads;
+    for (int64_t b = (threadIdx.x >> 5) * (int64_t)gridDim.x + blockIdx.x; b < nrun;
+         b += (int64_t)(kLfThreads / 32) * gridDim.x) {
+        const int64_t s0 = b * 64 + (threadIdx.x & 31), s1 = s0 + 32;
         const pdq_sample_params p0 = A.params[s0 < A.S ? s0 : A.S - 1], p1 = A.params[s1 < A.S ? s1 : A.S - 1];
         const f2 ae = f2_pack((float)(-K.ce * p0.xi * p0.xi), (float)(-K.ce * p1.xi * p1.xi));
         const f2 av = f2_pack((float)(-K.cv * p0.zeta), (float)(-K.cv * p1.zeta));
         f2 V = 0ull, P = f2_pack(1.f, 1.f), Q = 0ull, NC = 0ull;      // NC: minus the compensation of Q
         // momentum: implicit drag, root <= 0 of V^2/2 - a V = c
-        auto momentum = [&](const LfCell<float>& e) -> f2 {
-            const f2 a = f2_pack(e.a, e.a);
-            const f2 c2 = f2_add(f2_fma(f2_mul(half, V), V, f2_pack(e.dw, e.dw)),
-                                 f2_fma(ae, f2_pack(e.de, e.de), f2_mul(av, f2_pack(e.dv, e.dv))));
-            const f2 cc = f2_add(c2, c2), x = f2_fma(a, a, cc);
+        auto momentum = [&](const LfCell<f2>& e) -> f2 {
+            const f2 c2 = f2_add(f2_fma(f2_mul(half, V), V, e.dw), f2_fma(ae, e.de, f2_mul(av, e.dv)));
+            const f2 cc = f2_add(c2, c2), x = f2_fma(e.a, e.a, cc);
             float ca, cb, xa, xb, da, db;
             f2_unpack(cc, ca, cb);
             f2_unpack(x, xa, xb);
-            f2_unpack(f2_fma(x, f2_pack(rsqrtf(xa), rsqrtf(xb)), a), da, db);
-            return f2_pack(ca > 0.f ? __fdividef(-ca, da) : 0.f, cb > 0.f ? __fdividef(-cb, db) : 0.f);
+            f2_unpack(f2_fma(x, f2_pack(rsqrt_ftz(xa), rsqrt_ftz(xb)), e.a), da, db);
+            return f2_pack(ca > 0.f ? lf_div_ftz(-ca, da) : 0.f, cb > 0.f ? lf_div_ftz(-cb, db) : 0.f);
         };
         for (int k1 = ncell; k1 > 0;) {
             const int k0 = k1 > kLfStride ? k1 - kLfStride : 0;
@@ -280,7 +292,7 @@ __global__ void __launch_bounds__(kLfThreads) k_lf_vdep32(const LfArgs A) {
                 for (int k = k1 - 1; k >= k0; --k) V = momentum(cell[k]);
             } else {
                 for (int k = k1 - 1; k >= k0; --k) {
-                    const f2 h = f2_pack(t_h[k], t_h[k]), Vi = momentum(cell[k]);
+                    const f2 h = t_h[k], Vi = momentum(cell[k]);
                     // continuity: exact cell solution with the cell-mean V and D
                     const f2 am = f2_mul(f2_mul(half, f2_add(Vi, V)), h);      // <= 0
                     f2 p = f2_dup(2.7557319e-6f);                              // 1/9!
@@ -299,8 +311,8 @@ __global__ void __launch_bounds__(kLfThreads) k_lf_vdep32(const LfArgs A) {
                         float ea, eb, pa, pb;
                         f2_unpack(E, ea, eb);
                         f2_unpack(p, pa, pb);
-                        if (!(ma > -0.5f)) { ea = __expf(ma); pa = __fdividef(ea - 1.0f, ma); }
-                        if (!(mb > -0.5f)) { eb = __expf(mb); pb = __fdividef(eb - 1.0f, mb); }
+                        if (!(ma > -0.5f)) { ea = __expf(ma); pa = lf_div_ftz(ea - 1.0f, ma); }
+                        if (!(mb > -0.5f)) { eb = __expf(mb); pb = lf_div_ftz(eb - 1.0f, mb); }
                         E = f2_pack(ea, eb);
                         p = f2_pack(pa, pb);
                     }
@@ -383,7 +395,8 @@ static size_t lf_shared_bytes(int32_t n_y, size_t elem) { return (size_t)5 * (si
 
 // One wave: as many CTAs per class as fit on the GPU at once (its SMs times the
 // resident CTAs per SM, divided among the classes), each building its class's
-// table once and walking its share of the blocks of `per` samples.
+// table once and walking its share of the runs of `per` samples (a warp's).  Few
+// samples spread a run to a CTA over as many SMs.
 static int launch_lf(void (*kernel)(LfArgs), int threads, int per, size_t elem, const LfArgs& A, pdq_stream_t stream) {
     const size_t smem = lf_shared_bytes(A.n_y, elem);
     PDQ_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -453,6 +466,6 @@ extern "C" int pdq_lf_vdep(const pdq_field* field, const pdq_phys* phys, const p
     A.var = var;
     A.params = params;
     A.vdep = vdep;
-    if (lf->precision == PDQ_FP64) return launch_lf(k_lf_vdep64, kLfThreads64, kLfThreads64, sizeof(double), A, stream);
-    return launch_lf(k_lf_vdep32, kLfThreads, 2 * kLfThreads, sizeof(float), A, stream);
+    if (lf->precision == PDQ_FP64) return launch_lf(k_lf_vdep64, kLfThreads64, 32, sizeof(double), A, stream);
+    return launch_lf(k_lf_vdep32, kLfThreads, 64, sizeof(f2), A, stream);
 }
