@@ -46,7 +46,8 @@ struct pdq_p3m {
     int* cell_start;            // [ncells + 1]
     int* cell_fill;             // [ncells]
     int* cell_list;             // [max_n]
-    float4* sorted;             // [3][max_n] live particles in cell order, split: (x, y, z) hi and q hi, mid and q lo, lo
+    float4* sorted;             // [3][max_n] live particles in cell order, split: x, y, z hi and q hi; mid and q lo;
+                                // lo and the cell's index
     float4* lf_tab;             // [2][kTab] K_L factor by quartics on kTab intervals of u = (alpha r)^2 < (alpha r_cut)^2
     double* sums;               // [sums_cap][3], for the step driver
     int64_t sums_cap;
@@ -318,7 +319,7 @@ __global__ void k_cell_gather(const P3MGeom G, const P3MPart S, const int* start
     split3(G.grid, z, h.z, m.z, l.z);
     h.w = (float)q;
     m.w = (float)(q - (double)h.w);
-    l.w = 0.f;
+    l.w = __int_as_float(cell_of(G, x, y, z));
     sorted[t] = h;
     sorted[stride + t] = m;
     sorted[2 * stride + t] = l;
@@ -421,7 +422,8 @@ __device__ __forceinline__ void pp_pair(const PPConst& K, const float4* T, const
 // evaluated with all lanes busy; the lanes' partial sums (about a dozen pairs each) are reduced in a
 // fixed order.
 // Bound by instruction issue (screening ~1,500 candidates and ~410 pairs of ~190 instructions per
-// particle).  One million particles, mesh 256^3: 7.5 ms; 42.4 ms in FP64 with the Hermite table in
+// particle).  One million particles, mesh 256^3: 6.8 ms (7.5 ms with the cell index recomputed in FP64 by
+// every lane); 42.4 ms in FP64 with the Hermite table in
 // global memory (FP64 pipe 87 % busy), 13.6 ms in float-float over the 27 cells of width r_cut.
 constexpr int kPPWarps = 8;
 __global__ void __launch_bounds__(32 * kPPWarps) k_p3m_pp(const P3MGeom G, const P3MPart S, const int* start,
@@ -454,9 +456,7 @@ __global__ void __launch_bounds__(32 * kPPWarps) k_p3m_pp(const P3MGeom G, const
         // column lane of the 5 x 5 around i: its runs [b0, e0) and, across the period, [b1, e1)
         int b0 = 0, e0 = 0, b1 = 0, e1 = 0;
         {
-            const int ci = cell_of(G, (double)ih.x + (double)im.x + (double)il.x,
-                                   (double)ih.y + (double)im.y + (double)il.y,
-                                   (double)ih.z + (double)im.z + (double)il.z);
+            const int ci = __float_as_int(il.w);
             const int cz = ci % G.ncz, cy = (ci / G.ncz) % G.ncx, cx = ci / (G.ncz * G.ncx);
             constexpr int kCols = 2 * kReachXY + 1;
             const int a = cx + lane / kCols - kReachXY, b = cy + lane % kCols - kReachXY;
@@ -533,9 +533,9 @@ __global__ void __launch_bounds__(32 * kPPWarps) k_p3m_pp(const P3MGeom G, const
                 c[a] = __fadd_rn(__fadd_rn(c[a], oc), u);
             }
         }
-        if (lane == 0) {
-            const int64_t gi = S.o + list[t];
-            for (int a = 0; a < 3; ++a) sums[3 * gi + a] += (double)s[a] + (double)c[a];
+        if (lane < 3) {      // lane a adds component a
+            const float sa = lane == 0 ? s[0] : lane == 1 ? s[1] : s[2], ca = lane == 0 ? c[0] : lane == 1 ? c[1] : c[2];
+            sums[3 * (S.o + list[t]) + lane] += (double)sa + (double)ca;
         }
     }
 }
