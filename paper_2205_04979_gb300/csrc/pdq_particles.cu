@@ -467,13 +467,21 @@ __device__ __forceinline__ float near_bound(const StepConst& K, const float* s_v
 
 // Contact accelerations of this thread's particles from the j-tile starting at j0, added to
 // its own slots of s_ct[3][U][NT].
-template <int P, int NT, int U>
+// A thread's u-th particle of an item: strided over the tile, or for V = 6 a contiguous run of 32 U per warp
+// (narrow in z, so that most j groups are out of the warp's reach).
+template <int NT, int U, int V>
+__device__ __forceinline__ int tile_slot(int u) {
+    const int tid = threadIdx.x;
+    return V == 6 ? (tid >> 5) * (32 * U) + u * 32 + (tid & 31) : u * NT + tid;
+}
+
+template <int P, int NT, int U, int V>
 __device__ __forceinline__ void contact_rows(const StepArgs& A, int64_t base, int64_t end, int64_t j0, double zeta,
                                              double* s_ct) {
     const int tid = threadIdx.x;
     const int64_t je = j0 + NT < end ? j0 + NT : end;
     for (int u = 0; u < U; ++u) {
-        const int64_t g = base + u * NT + tid;
+        const int64_t g = base + tile_slot<NT, U, V>(u);
         if (g >= end) continue;
         double c3[3] = {0.0, 0.0, 0.0};
         contact_tile<P>(A, g, j0, je, zeta, c3);
@@ -485,12 +493,12 @@ __device__ __forceinline__ void contact_rows(const StepArgs& A, int64_t base, in
 
 // End of a j-tile in the contact variant: the closing barrier also ORs the threads' near-pair
 // flags; a flagged tile is appended to the CTA's list (contact_rows runs when the list is full).
-template <int P, int NT, int U, int NF>
+template <int P, int NT, int U, int V, int NF>
 __device__ __forceinline__ void flag_tile(const StepArgs& A, bool near, int64_t j0, int& nflag, long long* s_flag,
                                           int64_t base, int64_t end, double zeta, double* s_ct) {
     if (!__syncthreads_or(near)) return;
     if (nflag == NF) {
-        for (int f = 0; f < NF; ++f) contact_rows<P, NT, U>(A, base, end, s_flag[f], zeta, s_ct);
+        for (int f = 0; f < NF; ++f) contact_rows<P, NT, U, V>(A, base, end, s_flag[f], zeta, s_ct);
         nflag = 0;
         __syncthreads();           // every thread has read the list before it is overwritten
     }
@@ -499,12 +507,12 @@ __device__ __forceinline__ void flag_tile(const StepArgs& A, bool near, int64_t 
 }
 
 // Contact accelerations from every flagged j-tile of the item.
-template <int P, int NT, int U>
+template <int P, int NT, int U, int V>
 __device__ __forceinline__ void flush_flags(const StepArgs& A, int nflag, const long long* s_flag, int64_t base,
                                             int64_t end, double zeta, double* s_ct) {
     if (!nflag) return;
     __syncthreads();               // the last entry is visible
-    for (int f = 0; f < nflag; ++f) contact_rows<P, NT, U>(A, base, end, s_flag[f], zeta, s_ct);
+    for (int f = 0; f < nflag; ++f) contact_rows<P, NT, U, V>(A, base, end, s_flag[f], zeta, s_ct);
     __syncthreads();               // the list is free for the next item
 }
 
@@ -615,7 +623,7 @@ __global__ void __launch_bounds__(NT, ((V == 4 || V == 6) && P == PDQ_MIXED) ? 6
         T xi[U], yi[U], zi[U], ax[U], ay[U], az[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int64_t g = base + u * NT + tid;
+            const int64_t g = base + tile_slot<NT, U, V>(u);
             if (g < end) { const T4 p = pos_in[g]; xi[u] = p.x; yi[u] = p.y; zi[u] = p.z; }
             else { xi[u] = (T)0; yi[u] = (T)0; zi[u] = (T)0; }
             ax[u] = ay[u] = az[u] = (T)0;
@@ -627,7 +635,7 @@ __global__ void __launch_bounds__(NT, ((V == 4 || V == 6) && P == PDQ_MIXED) ? 6
             float vmax = 0.f;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const int64_t g = base + u * NT + tid;
+                const int64_t g = base + tile_slot<NT, U, V>(u);
                 s_ct[(0 * U + u) * NT + tid] = 0.0;
                 s_ct[(1 * U + u) * NT + tid] = 0.0;
                 s_ct[(2 * U + u) * NT + tid] = 0.0;
@@ -643,7 +651,7 @@ __global__ void __launch_bounds__(NT, ((V == 4 || V == 6) && P == PDQ_MIXED) ? 6
         if constexpr (V == 5) {      // Coulomb sums given (P3M, or the Newton-pair kernel): no pair loop
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const int64_t g = base + u * NT + tid;
+                const int64_t g = base + tile_slot<NT, U, V>(u);
                 if (g < end) {
                     if (A.acc4) { const float4 a = A.acc4[g]; ax[u] = (T)a.x; ay[u] = (T)a.y; az[u] = (T)a.z; }
                     else { ax[u] = (T)A.ext[3 * g]; ay[u] = (T)A.ext[3 * g + 1]; az[u] = (T)A.ext[3 * g + 2]; }
@@ -669,7 +677,7 @@ __global__ void __launch_bounds__(NT, ((V == 4 || V == 6) && P == PDQ_MIXED) ? 6
                 float ilo = INFINITY, ihi = -INFINITY;
 #pragma unroll
                 for (int u = 0; u < U; ++u)
-                    if (base + u * NT + tid < end) { ilo = fminf(ilo, (float)zi[u]); ihi = fmaxf(ihi, (float)zi[u]); }
+                    if (base + tile_slot<NT, U, V>(u) < end) { ilo = fminf(ilo, (float)zi[u]); ihi = fmaxf(ihi, (float)zi[u]); }
                 for (int d = 16; d > 0; d >>= 1) {
                     ilo = fminf(ilo, __shfl_xor_sync(0xffffffffu, ilo, d));
                     ihi = fmaxf(ihi, __shfl_xor_sync(0xffffffffu, ihi, d));
@@ -716,26 +724,33 @@ __global__ void __launch_bounds__(NT, ((V == 4 || V == 6) && P == PDQ_MIXED) ? 6
                         // pair within reach of the contact range, and only for the nearest r^2
                         const bool far = direct && ((dlo - shift > thr) || (dhi - shift < -thr));
                         if (!far) {
-                            if (direct) {
-                                const f2 sh = f2_pack(shift, shift);
+                            // group by group for the warp's own, narrower z range
+#pragma unroll 1
+                            for (int g = 0; g < NT / 32; ++g) {
+                                const ZClass zc = zclass(ilo, ihi, s_zr[g].x, s_zr[g].y, Lf, thr);
+                                if (zc.apart) continue;
+                                const f2 sh = f2_pack(zc.shift, zc.shift);
                                 f2 Zs[H];
 #pragma unroll
                                 for (int h = 0; h < H; ++h) Zs[h] = f2_sub(Z[h], sh);
+                                if (zc.direct) {
 #pragma unroll 4
-                                for (int k = 0; k < NT; ++k) {
-                                    const ulonglong2 a = sj2[2 * k], b = sj2[2 * k + 1];
+                                    for (int k = 32 * g; k < 32 * g + 32; ++k) {
+                                        const ulonglong2 a = sj2[2 * k], b = sj2[2 * k + 1];
 #pragma unroll
-                                    for (int h = 0; h < H; ++h)
-                                        near_pair_x2<false>(X[h], Y[h], Zs[h], a.x, a.y, b.x, invL2, M2, nM2, nL2,
-                                                            mn);
-                                }
-                            } else {
+                                        for (int h = 0; h < H; ++h)
+                                            near_pair_x2<false>(X[h], Y[h], Zs[h], a.x, a.y, b.x, invL2, M2, nM2, nL2,
+                                                                mn);
+                                    }
+                                } else {
 #pragma unroll 4
-                                for (int k = 0; k < NT; ++k) {
-                                    const ulonglong2 a = sj2[2 * k], b = sj2[2 * k + 1];
+                                    for (int k = 32 * g; k < 32 * g + 32; ++k) {
+                                        const ulonglong2 a = sj2[2 * k], b = sj2[2 * k + 1];
 #pragma unroll
-                                    for (int h = 0; h < H; ++h)
-                                        near_pair_x2<true>(X[h], Y[h], Z[h], a.x, a.y, b.x, invL2, M2, nM2, nL2, mn);
+                                        for (int h = 0; h < H; ++h)
+                                            near_pair_x2<true>(X[h], Y[h], Z[h], a.x, a.y, b.x, invL2, M2, nM2, nL2,
+                                                               mn);
+                                    }
                                 }
                             }
                         }
@@ -786,15 +801,15 @@ __global__ void __launch_bounds__(NT, ((V == 4 || V == 6) && P == PDQ_MIXED) ? 6
                         }
                     }
                     if constexpr (CT)
-                        flag_tile<P, NT, U, kFlags>(A, mn < thr * thr, j0, nflag, s_flag, base, end, zeta, s_ct);
+                        flag_tile<P, NT, U, V, kFlags>(A, mn < thr * thr, j0, nflag, s_flag, base, end, zeta, s_ct);
                     else
                         __syncthreads();
                 }
-                if constexpr (CT) flush_flags<P, NT, U>(A, nflag, s_flag, base, end, zeta, s_ct);
+                if constexpr (CT) flush_flags<P, NT, U, V>(A, nflag, s_flag, base, end, zeta, s_ct);
                 if constexpr (V == 6) {       // the Coulomb sums of the Newton-pair kernel
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        const int64_t g = base + u * NT + tid;
+                        const int64_t g = base + tile_slot<NT, U, V>(u);
                         if (g < end) { const float4 a = A.acc4[g]; ax[u] = a.x; ay[u] = a.y; az[u] = a.z; }
                     }
                 } else if constexpr (V != 1) {
@@ -813,7 +828,7 @@ __global__ void __launch_bounds__(NT, ((V == 4 || V == 6) && P == PDQ_MIXED) ? 6
                     double lo = INFINITY, hi = -INFINITY;
 #pragma unroll
                     for (int u = 0; u < U; ++u)
-                        if (base + u * NT + tid < end) { lo = fmin(lo, (double)zi[u]); hi = fmax(hi, (double)zi[u]); }
+                        if (base + tile_slot<NT, U, V>(u) < end) { lo = fmin(lo, (double)zi[u]); hi = fmax(hi, (double)zi[u]); }
                     for (int d = 16; d > 0; d >>= 1) {
                         lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, d));
                         hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, d));
@@ -853,7 +868,7 @@ __global__ void __launch_bounds__(NT, ((V == 4 || V == 6) && P == PDQ_MIXED) ? 6
                             for (int u = 0; u < U; ++u)
                                 coulomb_pair_track(xi[u], yi[u], zi[u], p, L, invL, c2, ax[u], ay[u], az[u], mnh);
                         }
-                        flag_tile<P, NT, U, kFlags>(A, mnh <= __double2hiint(thr * thr), j0, nflag, s_flag, base, end,
+                        flag_tile<P, NT, U, V, kFlags>(A, mnh <= __double2hiint(thr * thr), j0, nflag, s_flag, base, end,
                                                     zeta, s_ct);
                     } else {
                         // as the MIXED path: a tile pair inside one period window takes a uniform
@@ -905,7 +920,7 @@ __global__ void __launch_bounds__(NT, ((V == 4 || V == 6) && P == PDQ_MIXED) ? 6
                         __syncthreads();
                     }
                 }
-                if constexpr (CT) flush_flags<P, NT, U>(A, nflag, s_flag, base, end, zeta, s_ct);
+                if constexpr (CT) flush_flags<P, NT, U, V>(A, nflag, s_flag, base, end, zeta, s_ct);
             }
         }
         if constexpr (P == PDQ_FP64 && V != 5) {
@@ -914,7 +929,7 @@ __global__ void __launch_bounds__(NT, ((V == 4 || V == 6) && P == PDQ_MIXED) ? 6
                 const int64_t cap = A.cap;
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const int64_t g = base + u * NT + tid;
+                    const int64_t g = base + tile_slot<NT, U, V>(u);
                     if (g < end) {
                         part[(jc * 3 + 0) * cap + g] = ax[u];
                         part[(jc * 3 + 1) * cap + g] = ay[u];
@@ -929,7 +944,7 @@ __global__ void __launch_bounds__(NT, ((V == 4 || V == 6) && P == PDQ_MIXED) ? 6
                 __threadfence();
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const int64_t g = base + u * NT + tid;
+                    const int64_t g = base + tile_slot<NT, U, V>(u);
                     if (g < end) {
                         double sx = 0.0, sy = 0.0, sz = 0.0;
 #pragma unroll 4
@@ -947,7 +962,7 @@ __global__ void __launch_bounds__(NT, ((V == 4 || V == 6) && P == PDQ_MIXED) ? 6
         const pdq_sample_params sp = A.params[s];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int64_t g = base + u * NT + tid;
+            const int64_t g = base + tile_slot<NT, U, V>(u);
             int cls = -1;
             bool was_alive = false, dep = false;
             if (g < end) {
