@@ -1,6 +1,6 @@
 // pdq_mfmc.cu -- multi-fidelity Monte Carlo allocation and Sobol' estimators
-// (Sec. 3 of the paper): FP64 pick-freeze sums on the device, estimator
-// assembly on the host.
+// (Sec. 3 of the paper): FP64 pick-freeze sums and estimators on the device,
+// percentiles on the host.
 //
 // Model i's evaluations are laid out as y_i[g][col][c]: group g (a shared
 // sample sequence, nested across models), column 0 = f(x), 1 = f(x'),
@@ -33,42 +33,43 @@ struct SumArgs {
     const double* y[8];     // per model, device [n_i][d+2][C]
     int64_t m[8];           // nested counts
     int32_t k, d, C;
+    int32_t outs;           // outputs per cluster, at most kSumOutputs
     uint2 key;
     double* sums;           // [1+B][k][2][C][4+2d]
 };
 
-// One cluster of kSumCtas CTAs per (block of outputs, model, replicate): thread (t, c) of the cluster takes
+// One cluster of CTAs per (block of outputs, model, replicate): thread (t, c) of the cluster takes
 // the group positions t, t + T, ... of output c, so that a warp's reads of a group are runs of the table
 // (one output per CTA read a 32-byte sector for each 8-byte value, and drew every position's index again
 // for each output).  The sums up to m_{i-1} (prefix 0) are taken on the way to m_i.  Each CTA adds its
-// threads' sums in thread order, the first CTA of the cluster adds the CTAs' in rank order: the
+// threads' sums in a fixed tree, the first CTA of the cluster adds the CTAs' in rank order: the
 // result does not depend on the schedule.  Bound by the FP64 pipe, 13 operations per position and
 // output at d = 3; D: the number of inputs (0: any, from A.d), so that the accumulators stay in registers.
 // A study of 834 and 16,570 groups, 10 outputs, 200 replicates: 1.04 ms; 1.39 ms before.
-constexpr int kSumCtas = 4, kSumThreads = 256, kSumOutputs = 32;
+constexpr int kSumThreads = 256, kSumOutputs = 32;
 
 template <int D>
-__global__ void __cluster_dims__(kSumCtas, 1, 1) __launch_bounds__(kSumThreads) k_mfmc_sums(const SumArgs A) {
+__global__ void __launch_bounds__(kSumThreads) k_mfmc_sums(const SumArgs A) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
-    constexpr int kMaxD = D ? D : kMaxInputs;
-    __shared__ double red[kSumThreads];
-    __shared__ double part[4 + 2 * kMaxD][kSumOutputs];
+    constexpr int kMaxD = D ? D : kMaxInputs, kSums = 4 + 2 * kMaxD;
+    __shared__ double red[8][kSumThreads];
+    __shared__ double part[kSums][kSumOutputs];
     const int d = D ? D : A.d, C = A.C, ncol = d + 2, nq = 4 + 2 * d;
-    const int rank = (int)cluster.block_rank(), c0 = (int)(blockIdx.x / kSumCtas) * kSumOutputs;
+    const int ctas = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), c0 = (int)(blockIdx.x / ctas) * A.outs;
     const int i = blockIdx.y, b = blockIdx.z;         // model; 0 = the sample itself, >= 1 bootstrap
-    const int nc = C - c0 < kSumOutputs ? C - c0 : kSumOutputs, T = kSumThreads / nc;
+    const int nc = C - c0 < A.outs ? C - c0 : A.outs, T = kSumThreads / nc;
     const int tid = threadIdx.x, cc = tid % nc, tt = tid / nc;
     const bool active = tt < T;                       // the threads past T whole rows of outputs idle
     const double* __restrict__ y = A.y[i];
-    double acc[4 + 2 * kMaxD];
+    double acc[kSums];
 #pragma unroll
-    for (int q = 0; q < 4 + 2 * kMaxD; ++q) acc[q] = 0.0;
+    for (int q = 0; q < kSums; ++q) acc[q] = 0.0;
     int64_t t = (int64_t)rank * T + tt;
     for (int p = i > 0 ? 0 : 1; p < 2; ++p) {
         const int64_t m = p ? A.m[i] : A.m[i - 1];
         if (active) {
-            for (; t < m; t += (int64_t)kSumCtas * T) {
+            for (; t < m; t += (int64_t)ctas * T) {
                 int64_t g = t;
                 if (b > 0) {
                     // block-wise resampling: position t in [m_{l-1}, m_l) draws from the same block,
@@ -93,17 +94,25 @@ __global__ void __cluster_dims__(kSumCtas, 1, 1) __launch_bounds__(kSumThreads) 
                 }
             }
         }
+        // the rows of threads fold in a fixed tree, 8 sums at a time (a chain of T FP64 adds by one thread
+        // per output took 20 us a sum at one output)
 #pragma unroll
-        for (int q = 0; q < 4 + 2 * kMaxD; ++q) {
-            const int j = (q - 4) % kMaxD;            // input of a product sum
-            if (q >= 4 && j >= d) continue;
-            red[tid] = acc[q];
+        for (int q0 = 0; q0 < kSums; q0 += 8) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (q0 + e < kSums) red[e][tid] = acc[q0 + e];
             __syncthreads();
-            if (tid < nc) {
-                double v = 0.0;
-                for (int r = 0; r < T; ++r) v += red[r * nc + tid];
-                part[q][tid] = v;
+            for (int n = T; n > 1;) {
+                const int half = (n + 1) / 2, fold = (n - half) * nc;
+                for (int u = tid; u < 8 * fold; u += kSumThreads) {
+                    const int e = u / fold, r = u - e * fold;
+                    red[e][r] += red[e][half * nc + r];
+                }
+                __syncthreads();
+                n = half;
             }
+            for (int u = tid; u < 8 * nc; u += kSumThreads)
+                if (q0 + u / nc < kSums) part[q0 + u / nc][u % nc] = red[u / nc][u % nc];
             __syncthreads();
         }
         cluster.sync();
@@ -113,7 +122,7 @@ __global__ void __cluster_dims__(kSumCtas, 1, 1) __launch_bounds__(kSumThreads) 
                 const int c = u / nq, q = u % nq;
                 const int qs = q < 4 + d ? q : 4 + kMaxD + (q - 4 - d);
                 double v = 0.0;
-                for (int r = 0; r < kSumCtas; ++r) v += cluster.map_shared_rank(&part[0][0], r)[qs * kSumOutputs + c];
+                for (int r = 0; r < ctas; ++r) v += cluster.map_shared_rank(&part[0][0], r)[qs * kSumOutputs + c];
                 out[(int64_t)c * nq + q] = v;
             }
         }
@@ -121,56 +130,80 @@ __global__ void __cluster_dims__(kSumCtas, 1, 1) __launch_bounds__(kSumThreads) 
     }
 }
 
-static void launch_sums(const SumArgs& A, int n_boot, cudaStream_t s) {
-    const dim3 grid((unsigned)((A.C + kSumOutputs - 1) / kSumOutputs * kSumCtas), (unsigned)A.k, (unsigned)(1 + n_boot));
+template <int D>
+static int launch_sums_d(const SumArgs& A, int ctas, int n_boot, cudaStream_t s) {
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)((A.C + A.outs - 1) / A.outs * ctas), (unsigned)A.k, (unsigned)(1 + n_boot));
+    cfg.blockDim = dim3(kSumThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    memset(&attr, 0, sizeof(attr));
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)ctas;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    PDQ_CUDA(cudaLaunchKernelEx(&cfg, k_mfmc_sums<D>, A));
+    return PDQ_OK;
+}
+
+// A cluster takes all outputs (up to 32) with one CTA; while the clusters of a model are too few to give every SM
+// 8 CTAs, and a thread keeps 12 positions of the longest model, the cluster grows to 8 CTAs and then
+// takes fewer outputs, at the price of partly used sectors.  No replicates, 40,000 groups, 10 outputs: 0.10 ms
+// (0.45 ms with 4 CTAs for all outputs, 0.30 ms with a CTA per output).
+static int launch_sums(SumArgs A, int n_boot, int sms, cudaStream_t s) {
+    int ctas = 1;
+    A.outs = A.C < kSumOutputs ? A.C : kSumOutputs;
+    const auto few = [&] { return (int64_t)((A.C + A.outs - 1) / A.outs) * (1 + n_boot) * ctas < 8 * (int64_t)sms; };
+    const auto keeps = [&](int outs, int n) { return A.m[A.k - 1] >= (int64_t)12 * n * (kSumThreads / outs); };
+    while (ctas < 8 && few() && keeps(A.outs, 2 * ctas)) ctas *= 2;
+    while (A.outs > 1 && few() && keeps((A.outs + 1) / 2, ctas)) A.outs = (A.outs + 1) / 2;
     switch (A.d) {
-        case 1: k_mfmc_sums<1><<<grid, kSumThreads, 0, s>>>(A); break;
-        case 2: k_mfmc_sums<2><<<grid, kSumThreads, 0, s>>>(A); break;
-        case 3: k_mfmc_sums<3><<<grid, kSumThreads, 0, s>>>(A); break;
-        case 4: k_mfmc_sums<4><<<grid, kSumThreads, 0, s>>>(A); break;
-        default: k_mfmc_sums<0><<<grid, kSumThreads, 0, s>>>(A);
+        case 1: return launch_sums_d<1>(A, ctas, n_boot, s);
+        case 2: return launch_sums_d<2>(A, ctas, n_boot, s);
+        case 3: return launch_sums_d<3>(A, ctas, n_boot, s);
+        case 4: return launch_sums_d<4>(A, ctas, n_boot, s);
+        default: return launch_sums_d<0>(A, ctas, n_boot, s);
     }
 }
 
-// Host assembly of one replicate: mean, variance, main and total indices per output.
-struct Estimates {
-    std::vector<double> mean, var, smain, stot;   // [C], [C], [d][C], [d][C]
+struct AssembleArgs {
+    double alpha[8];
+    int64_t m[8];
+    int32_t k, d, C, reps;
+    double* sums;
 };
-
-static void assemble(const double* sums, int k, int d, int C, const int64_t* m, const double* alpha, Estimates* e) {
-    const int nq = 4 + 2 * d;
-    e->mean.assign(C, 0.0); e->var.assign(C, 0.0);
-    e->smain.assign((size_t)d * C, 0.0); e->stot.assign((size_t)d * C, 0.0);
-    for (int c = 0; c < C; ++c) {
-        std::vector<double> Vj(d, 0.0), Tj(d, 0.0);
-        double mean = 0.0, var = 0.0;
-        for (int i = 0; i < k; ++i) {
-            for (int p = 1; p >= (i > 0 ? 0 : 1); --p) {
-                const double mm = (double)(p ? m[i] : m[i - 1]);
-                const double* s = sums + (((int64_t)i * 2 + p) * C + c) * nq;
-                const double E = s[0] / mm, Ep = s[2] / mm;
-                const double V = (s[1] - mm * E * E) / (mm - 1.0), Vp = (s[3] - mm * Ep * Ep) / (mm - 1.0);
-                // term sign/weight: model 1 enters once; model i >= 2 as alpha_i (y_{m_i} - y_{m_{i-1}})
-                const double wgt = i == 0 ? 1.0 : (p ? alpha[i] : -alpha[i]);
-                mean += wgt * E;
-                var += wgt * V;
-                for (int j = 0; j < d; ++j) {
-                    // Owen's main-effect estimator and Jansen's total-effect estimator (Sec. 3.3)
-                    const double vj = 2.0 * mm / (2.0 * mm - 1.0) *
-                                      (s[4 + j] / mm - 0.25 * (E + Ep) * (E + Ep) + (V + Vp) / (4.0 * mm));
-                    const double tj = s[4 + d + j] / (2.0 * mm);
-                    Vj[j] += wgt * vj;
-                    Tj[j] += wgt * tj;
-                }
-            }
-        }
-        e->mean[c] = mean;
-        e->var[c] = var;
-        for (int j = 0; j < d; ++j) {
-            e->smain[(size_t)j * C + c] = Vj[j] / var;
-            e->stot[(size_t)j * C + c] = Tj[j] / var;
+// Mean, variance and the indices of input j of one (replicate, output) from its sums, into the slot of model 0's
+// prefix 0, which has none: [2 + 2d] doubles (mean, var, s_main [d], s_total [d]).
+__host__ __device__ inline void assemble(const AssembleArgs& A, double* rep, int c, int j) {
+    const int nq = 4 + 2 * A.d;
+    double mean = 0.0, var = 0.0, Vj = 0.0, Tj = 0.0;
+    for (int i = 0; i < A.k; ++i) {
+        for (int p = 1; p >= (i > 0 ? 0 : 1); --p) {
+            const double mm = (double)(p ? A.m[i] : A.m[i - 1]);
+            const double* s = rep + (((int64_t)i * 2 + p) * A.C + c) * nq;
+            const double E = s[0] / mm, Ep = s[2] / mm;
+            const double V = (s[1] - mm * E * E) / (mm - 1.0), Vp = (s[3] - mm * Ep * Ep) / (mm - 1.0);
+            // term sign/weight: model 1 enters once; model i >= 2 as alpha_i (y_{m_i} - y_{m_{i-1}})
+            const double wgt = i == 0 ? 1.0 : (p ? A.alpha[i] : -A.alpha[i]);
+            mean += wgt * E;
+            var += wgt * V;
+            // Owen's main-effect estimator and Jansen's total-effect estimator (Sec. 3.3)
+            Vj += wgt * (2.0 * mm / (2.0 * mm - 1.0) *
+                         (s[4 + j] / mm - 0.25 * (E + Ep) * (E + Ep) + (V + Vp) / (4.0 * mm)));
+            Tj += wgt * (s[4 + A.d + j] / (2.0 * mm));
         }
     }
+    double* out = rep + (int64_t)c * nq;
+    if (j == 0) { out[0] = mean; out[1] = var; }
+    out[2 + j] = Vj / var;
+    out[2 + A.d + j] = Tj / var;
+}
+// One thread per (replicate, output, input).
+__global__ void k_mfmc_assemble(const AssembleArgs A) {
+    const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, b = u / ((int64_t)A.C * A.d);
+    if (b < A.reps) assemble(A, A.sums + b * A.k * 2 * A.C * (4 + 2 * A.d), (int)(u / A.d % A.C), (int)(u % A.d));
 }
 
 }  // namespace pdq
@@ -252,30 +285,55 @@ extern "C" int pdq_mfmc_sobol(int32_t k, const double* const* y, const int64_t* 
     A.key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
     A.sums = (double*)workspace;
     cudaStream_t s = (cudaStream_t)stream;
-    launch_sums(A, n_boot, s);
-    PDQ_CUDA(cudaGetLastError());
-    std::vector<double> h(need / sizeof(double));
-    PDQ_CUDA(cudaMemcpyAsync(h.data(), workspace, need, cudaMemcpyDeviceToHost, s));
-    PDQ_CUDA(cudaStreamSynchronize(s));
-    const size_t per_rep = (size_t)k * 2 * C * (4 + 2 * d);
-    Estimates e;
-    assemble(h.data(), k, d, C, m, alpha, &e);
-    for (int c = 0; c < C; ++c) { mean[c] = e.mean[c]; var[c] = e.var[c]; }
-    for (size_t q = 0; q < (size_t)d * C; ++q) { s_main[q] = e.smain[q]; s_total[q] = e.stot[q]; }
+    int dev = 0, sms = 1;
+    PDQ_CUDA(cudaGetDevice(&dev));
+    PDQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    rc = launch_sums(A, n_boot, sms, s);
+    if (rc) return rc;
+    AssembleArgs B;
+    memset(&B, 0, sizeof(B));
+    for (int i = 0; i < k; ++i) { B.alpha[i] = alpha[i]; B.m[i] = m[i]; }
+    B.k = k; B.d = d; B.C = C; B.reps = 1 + n_boot; B.sums = A.sums;
+    // Each replicate's estimates are the first C rows of its sums.  A few are put together on the host, which
+    // takes less than a kernel's launch.
+    const size_t nq = 4 + 2 * (size_t)d, row = (size_t)C * nq, per_rep = (size_t)k * 2 * row;
+    std::vector<double> h;
+    if (n_boot == 0) {
+        h.resize(per_rep);
+        PDQ_CUDA(cudaMemcpyAsync(h.data(), workspace, per_rep * sizeof(double), cudaMemcpyDeviceToHost, s));
+        PDQ_CUDA(cudaStreamSynchronize(s));
+        for (int c = 0; c < C; ++c)
+            for (int j = 0; j < d; ++j) assemble(B, h.data(), c, j);
+    } else {
+        h.resize(row * (size_t)(1 + n_boot));
+        k_mfmc_assemble<<<(unsigned)(((int64_t)B.reps * C * d + 63) / 64), 64, 0, s>>>(B);
+        PDQ_CUDA(cudaGetLastError());
+        PDQ_CUDA(cudaMemcpy2DAsync(h.data(), row * sizeof(double), workspace, per_rep * sizeof(double),
+                                   row * sizeof(double), (size_t)(1 + n_boot), cudaMemcpyDeviceToHost, s));
+        PDQ_CUDA(cudaStreamSynchronize(s));
+    }
+    for (int c = 0; c < C; ++c) {
+        const double* e = h.data() + (size_t)c * nq;
+        mean[c] = e[0];
+        var[c] = e[1];
+        for (int j = 0; j < d; ++j) { s_main[(size_t)j * C + c] = e[2 + j]; s_total[(size_t)j * C + c] = e[2 + d + j]; }
+    }
     if (n_boot > 0) {
-        // percentile interval: sorted replicate values at ranks round(0.025 (B-1)) and round(0.975 (B-1))
-        std::vector<std::vector<double>> bm((size_t)d * C), bt((size_t)d * C);
-        for (int b = 1; b <= n_boot; ++b) {
-            Estimates eb;
-            assemble(h.data() + per_rep * b, k, d, C, m, alpha, &eb);
-            for (size_t q = 0; q < (size_t)d * C; ++q) { bm[q].push_back(eb.smain[q]); bt[q].push_back(eb.stot[q]); }
-        }
+        // percentile interval: the replicate values of ranks round(0.025 (B-1)) and round(0.975 (B-1))
         const int lo = (int)lround(0.025 * (n_boot - 1)), hi = (int)lround(0.975 * (n_boot - 1));
-        for (size_t q = 0; q < (size_t)d * C; ++q) {
-            std::sort(bm[q].begin(), bm[q].end());
-            std::sort(bt[q].begin(), bt[q].end());
-            s_main_ci[2 * q] = bm[q][lo]; s_main_ci[2 * q + 1] = bm[q][hi];
-            s_total_ci[2 * q] = bt[q][lo]; s_total_ci[2 * q + 1] = bt[q][hi];
+        std::vector<double> v(n_boot);
+        const auto less = [](double a, double b) { return a < b || (b != b && a == a); };      // NaN last
+        for (int which = 0; which < 2; ++which) {
+            for (int j = 0; j < d; ++j) {
+                for (int c = 0; c < C; ++c) {
+                    for (int b = 0; b < n_boot; ++b) v[b] = h[row * (size_t)(1 + b) + (size_t)c * nq + 2 + which * d + j];
+                    double* ci = (which ? s_total_ci : s_main_ci) + 2 * ((size_t)j * C + c);
+                    std::nth_element(v.begin(), v.begin() + lo, v.end(), less);
+                    ci[0] = v[lo];
+                    std::nth_element(v.begin() + lo, v.begin() + hi, v.end(), less);
+                    ci[1] = v[hi];
+                }
+            }
         }
     }
     return PDQ_OK;
