@@ -422,11 +422,11 @@ __device__ __forceinline__ void pp_pair(const PPConst& K, const float4* T, const
 // evaluated with all lanes busy; the lanes' partial sums (about a dozen pairs each) are reduced in a
 // fixed order.
 // Bound by instruction issue (screening ~1,500 candidates and ~410 pairs of ~190 instructions per
-// particle).  One million particles, mesh 256^3: 6.8 ms (7.5 ms with the cell index recomputed in FP64 by
-// every lane); 42.4 ms in FP64 with the Hermite table in
+// particle).  One million particles, mesh 256^3: 5.9 ms (6.8 ms at 3 CTAs and 80 registers, 7.5 ms with the cell
+// index recomputed in FP64 by every lane); 42.4 ms in FP64 with the Hermite table in
 // global memory (FP64 pipe 87 % busy), 13.6 ms in float-float over the 27 cells of width r_cut.
 constexpr int kPPWarps = 8;
-__global__ void __launch_bounds__(32 * kPPWarps) k_p3m_pp(const P3MGeom G, const P3MPart S, const int* start,
+__global__ void __launch_bounds__(32 * kPPWarps, 4) k_p3m_pp(const P3MGeom G, const P3MPart S, const int* start,
                                                           int64_t ncells, const int* list,
                                                           const float4* __restrict__ sorted, int64_t stride,
                                                           double* sums) {
