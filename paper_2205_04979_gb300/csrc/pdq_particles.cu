@@ -1260,10 +1260,11 @@ __global__ void __launch_bounds__(NT) k_pairs_sym64(const StepArgs A) {
 // grows and that no longer holds.  The item table is k_pairs_sym64's (tiles of 2 NT particles, JS
 // chunks of the sample's j range); each CTA adds its item's sums to A.acc64 by atomics.
 // Bound by the FP32 FMA pipe (~135 operations per ordered pair, packed for two i).  100,000 particles,
-// 64 threads: 56 ms per step, 192 ms in k_pairs_sym64 (FP64 pipe 90 % busy); error of the sums against
+// 64 threads: 55.5 ms per step, 192 ms in k_pairs_sym64 (FP64 pipe 90 % busy); error of the sums against
 // extended precision, in units of 2^-53 of their 2-norm: 3.8 (6.3 before), at 8,192 particles 5.8 (5.7).
 // Three-float accumulators that are flushed once per j-tile instead of once per group left 7 and 14 units, without
-// the second word of the sums 24 and 38.
+// the second word of the sums 24 and 38.  Splitting the groups near in z by the pairs' distances instead (FP64
+// within one mean spacing) took 47 ms, but left 8.4 units at 100,000 particles.
 template <int NT>
 __global__ void __launch_bounds__(NT, 384 / NT) k_pairs_split64(const StepArgs A) {
     constexpr int W = NT / 32;
@@ -1362,7 +1363,7 @@ __global__ void __launch_bounds__(NT, 384 / NT) k_pairs_split64(const StepArgs A
                     const float sg = (float)(shift * invL);
                     const f2 zh = f2_sub(H[2], f2_dup(sg * Lh)), zm = f2_sub(M[2], f2_dup(sg * Lm));
                     const f2 zl = f2_sub(T[2], f2_dup(sg * Ll));
-#pragma unroll 1
+#pragma unroll 2
                     for (int k = 32 * g; k < 32 * g + ng; ++k) {
                         const ulonglong2 f0 = s_f[0][k], f1 = s_f[1][k], f2_ = s_f[2][k], f3 = s_f[3][k];
                         const ulonglong2 f4 = s_f[4][k], f5 = s_f[5][k];
