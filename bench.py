@@ -92,8 +92,15 @@ def dist_env():
     return int(os.environ.get("RANK", 0)), int(os.environ.get("WORLD_SIZE", 1)), int(os.environ.get("LOCAL_RANK", 0))
 
 
-def pipe_peak(mixed, newton):
+# FP64 Newton-pair runs sum the far pairs of samples of this many particles and more in float-float
+# (k_pairs_split64): ~135 FP32 operations per ordered pair for the 12 flops it counts
+SPLIT_MIN_PARTICLES, SPLIT_OPS_PER_PAIR = 8192, 135
+
+
+def pipe_peak(mixed, newton, split=False):
     """(peak TFLOP/s, note, instruction-mix peak or None) of the pair kernel's pipe, measured.
+
+    split: FP64 sums whose pairs run in float-float on the FP32 pipe.
 
     FP32: the packed FFMA2 rate (fma.rn.f32x2, 4 flops per lane per instruction), the pipe's
     highest flop rate.  FP64: the DFMA rate.  The Newton-pair kernels issue 16 pipe operations
@@ -107,7 +114,7 @@ def pipe_peak(mixed, newton):
                            % PEAKS_FILE)
     k = rec["kernels"]
     clk = rec["clocks"].get("sm_mhz")
-    if mixed:
+    if mixed or split:
         peak = k["ffma2"]["flops_per_s"] / 1e12
         note = ("measured FP32 FFMA2 (packed f32x2) peak, %.2f TFLOP/s at %.0f MHz on %d SMs" %
                 (peak, clk, rec["sms"]))
@@ -117,7 +124,10 @@ def pipe_peak(mixed, newton):
         note = "measured FP64 DFMA peak, %.3f TFLOP/s at %.0f MHz on %d SMs" % (peak, clk, rec["sms"])
         ops = k["dfma"]["lane_ops_per_s"]
     mix = None
-    if newton:
+    if split:
+        mix = {"peak": ops * 12 / SPLIT_OPS_PER_PAIR / 1e12,
+               "note": "the measured pipe operation rate x 12 flops / %d operations (float-float pair)" % SPLIT_OPS_PER_PAIR}
+    elif newton:
         mix = {"peak": ops * NEWTON_FLOPS_PER_LANE_OP / 1e12,
                "note": "the measured pipe operation rate x 24 flops / 16 operations (Newton-pair mix)"}
     return peak, note, mix
@@ -448,8 +458,15 @@ def run_ours(args):
         # min(compact_every, 10) steps, 10 without compaction; both precisions
         ci = min(cfg.compact_every, 10) if cfg.compact_every > 0 else 10
         n_rebin = sum(1 for k in range(args.steps - 1) if (s0 + k + 1) % ci == 0)
-        # sort, build_items, the step kernel(s) per step (Newton pairs: pair sums + update), re-bin + items
+        # sort, build_items, the step kernel(s) per step (Newton pairs, and FP64 tile pairs of up to 2,048
+        # particles: pair sums + update; FP64 Newton pairs sum large samples in a kernel of their own),
+        # re-bin + items
         per_step = 2 if cfg.variant == 3 and (not args.contact or prec == pdq.MIXED) else 1
+        if prec == pdq.FP64 and not args.contact:
+            if cfg.variant == 3 and int(np.sum(counts)) >= SPLIT_MIN_PARTICLES:
+                per_step = 3
+            elif cfg.variant == 0 and cfg.block == 32 and 32 < int(np.sum(counts)) <= 2048:
+                per_step = 2
         launches = 1 + 1 + per_step * args.steps + 2 * n_rebin
 
         # e2e: state in pinned host memory; every step uploads the state, steps it and downloads the
@@ -500,7 +517,8 @@ def run_ours(args):
         return
     newton = cfg.variant == 3 and (not args.contact or prec == pdq.MIXED)
     flops_per_pair = NEWTON_FLOPS_PER_PAIR if newton else FLOPS_PER_PAIR
-    peak_tflops, peak_note, mix = pipe_peak(prec == pdq.MIXED, newton)
+    split = newton and prec == pdq.FP64 and int(np.max(counts)) >= SPLIT_MIN_PARTICLES
+    peak_tflops, peak_note, mix = pipe_peak(prec == pdq.MIXED, newton, split)
     achieved = flops_per_pair * pairs / (ms / 1e3) / 1e12
     if mix is not None:
         mix["frac"] = achieved / mix["peak"]
@@ -534,7 +552,9 @@ def run_ours(args):
                                 "taking them (near pairs, contact forces, update)" if args.contact else
                                 "k_pairs_sym (Newton-pair Coulomb sums), then the given-sums k_step update"
                                 if prec == pdq.MIXED else
-                                "k_pairs_sym64 (FP64 Newton-pair Coulomb sums), then the given-sums k_step update")
+                                "%s, then the given-sums k_step update" % (
+                                    "k_pairs_split64 (FP64 Coulomb sums, far pairs in float-float)" if split else
+                                    "k_pairs_sym64 (FP64 Newton-pair Coulomb sums)"))
                                if newton else "k_step (all-pairs Coulomb + local step)",
                      "note": "%s; %d flops per ordered pair; time per step from CUDA events over the timed "
                              "region%s" % (peak_note, flops_per_pair,
@@ -955,7 +975,7 @@ def run_p3m(args):
                                   "%dx%dx%d, alpha=%.4f, r_cut=%.2f" % (n, w["dt"], M, 360.0 / M, Nz, plan.nx,
                                                                       plan.nx, Nz, plan.alpha, plan.r_cut)},
            "all_pairs_fp64_ms_per_step": ref_ms, "clocks": clocks,
-           "gpu_launches": int(args.steps * 16)}
+           "gpu_launches": int(args.steps * 13)}
     print(json.dumps(out), flush=True)
 
 
@@ -963,15 +983,15 @@ def run_p3m(args):
 # c = V^2/2 + dw + dPhi (7), root -2c/(a + sqrt(a^2 + 2c)) (7, sqrt and the division counted as
 # one each), cell means and exponential fitting vm, a', expm1, G = em/vm, E (6), Q += P G, P *= E (3)
 LF_FLOPS_PER_CELL = 23
-# FP64-pipe lane instructions per (item, cell) as executed (ncu instruction counters on a launch of
-# 16,384 samples x 10 classes: the square root, divisions and expm1 expand to seeds plus Newton or
+# FP64-pipe lane operations per (item, cell) as executed (ncu on a launch of 16,384 samples x 10
+# classes, pipe 82.4 % busy: the square root, divisions and expm1 expand to seeds plus correction or
 # polynomial steps), and the DRAM bytes (read + write) of a 65,536-sample launch, scaled by samples
-LF_FP64_OPS_PER_CELL = 61.41
+LF_FP64_OPS_PER_CELL = 46.4
 LF_DRAM_BYTES_PER_SAMPLE = 2.172e6 / 65536
-# the FP32 march: (what bounds it, thread instructions per (item, cell) as executed (ncu, same capture
-# size), the measured rate it is compared with): every instruction takes an issue slot, and the issue
+# the FP32 march: (what bounds it, thread instructions per (item, cell) as executed (ncu, 65,536
+# samples; a packed instruction serves two items), the measured rate it is compared with): every instruction takes an issue slot, and the issue
 # limit of 4 warp instructions per clock per SM equals the measured scalar FFMA lane rate
-LF_F32_PIPE = ("instruction issue", 56.48, "ffma")
+LF_F32_PIPE = ("instruction issue", 28.58, "ffma")
 
 
 def lf_cpu_baseline(w, params, seconds):
@@ -1070,7 +1090,7 @@ def run_lf(args):
     cells = w["n_y"] - 1
     sec, sec64 = ms / args.steps / 1e3, ms64 / args.steps / 1e3
     rel = np.abs(vd / vd64 - 1)
-    roof = {"bound": "alu", "kernel": "k_lf_vdep<float>", "unit": "TFLOP/s", "traffic": LF_DRAM_BYTES_PER_SAMPLE * S,
+    roof = {"bound": "alu", "kernel": "k_lf_vdep32", "unit": "TFLOP/s", "traffic": LF_DRAM_BYTES_PER_SAMPLE * S,
             "achieved": LF_FLOPS_PER_CELL * cells * items / sec / 1e12,
             "peak": k["ffma2"]["flops_per_s"] / 1e12 if k else None,
             "note": "%d operations per (item, cell) of the scheme, sqrt, expm1 and divisions counted as one each "
@@ -1097,13 +1117,13 @@ def run_lf(args):
         "e2e": {"value": items * args.steps / (ms_e2e / 1e3), "unit": "evaluations/s",
                 "h2d_bytes_per_step": int(S * 32), "d2h_bytes_per_step": int(S * C * 8)},
         "fp64": {"value": items * args.steps / (ms64 / 1e3), "ms_per_step": ms64 / args.steps, "clocks": clocks64,
-                 "roofline": {"bound": "alu", "kernel": "k_lf_vdep<double>", "unit": "Gop/s",
+                 "roofline": {"bound": "alu", "kernel": "k_lf_vdep64", "unit": "Gop/s",
                               "achieved": LF_FP64_OPS_PER_CELL * cells * items / sec64 / 1e9,
                               "peak": k["dfma"]["lane_ops_per_s"] / 1e9 if k else None,
                               "frac": (LF_FP64_OPS_PER_CELL * cells * items / sec64 / k["dfma"]["lane_ops_per_s"]
                                        if k else None),
                               "note": "%.2f FP64-pipe lane operations per (item, cell) as executed (ncu "
-                                      "instruction counters), against the measured DFMA lane-operation rate"
+                                      "pipe counters), against the measured DFMA lane-operation rate"
                                       % LF_FP64_OPS_PER_CELL}},
         "mixed_vs_fp64": {"max_rel": float(rel.max()), "median_rel": float(np.median(rel)), "items": int(items)},
         "us_per_sample_all_classes": ms / args.steps / S * 1e3,

@@ -264,7 +264,10 @@ int pdq_step_workspace_size(const pdq_state* state, const pdq_step_cfg* cfg, siz
  *   exponential integrator with u, f, a frozen over the step;
  *   wall contact when R - r - d/2 <= 0: STICK removes the particle,
  *   REBOUND applies CoR_n of Sec. 4.3 (sticking when it is 0).
- * FP64 runs everything in double; MIXED keeps x, y, the wall gap, the vdW
+ * FP64 runs everything in double, except that pair variant 3 sums the far
+ * pairs of samples of 8,192 particles and more in pairs of floats (each pair
+ * to 2^-46, the sums no further from the exact ones than double's); MIXED
+ * keeps x, y, the wall gap, the vdW
  * term and the tallies in double and runs the pair sum, interpolation, drag
  * and velocities in float.  `workspace` (>= pdq_step_workspace_size bytes,
  * device, 256-byte aligned) holds the work queue.  The particles of each
@@ -496,8 +499,9 @@ int pdq_mfmc_workspace_size(int32_t k, int32_t d, int32_t C, int32_t n_boot, siz
  * (m_0 = 0) to m_{l-1} + ((philox(t, b, 0, 2).x * (m_l - m_{l-1})) >> 32)
  * (Philox4x32-10, key = seed); model i reads positions t < m_i, so it never
  * reads beyond its own m_i groups.
- * FP64 sums on the device (one deterministic CTA reduction per model,
- * prefix, output and replicate), assembly on the host.  Host outputs: mean[C],
+ * FP64 sums on the device (fixed reduction trees per model, prefix, output
+ * and replicate: deterministic) and every replicate's estimates; the
+ * percentiles are selected on the host.  Host outputs: mean[C],
  * var[C], s_main[d][C], s_total[d][C], s_main_ci / s_total_ci [d][C][2]
  * (may be NULL when n_boot = 0).  Synchronises `stream`.
  * Errors: INVALID_ARG, WORKSPACE, CUDA.                                      */
@@ -567,8 +571,9 @@ int pdq_lf_fluid_variance(const pdq_field* field, double* var, pdq_stream_t stre
  * zeta used), var device [n_r] any v_f'^2 profile at `field`'s radial nodes
  * (normally pdq_lf_fluid_variance's), vdep device [S][C] (row = sample, the
  * deposition velocity over the centreline particle density; caller-owned).
- * One thread per item, 5 (n_y - 1) doubles (PDQ_MIXED: floats) of shared
- * memory per CTA of 256 samples.  Enqueued on `stream`; no allocation, no synchronisation.
+ * PDQ_FP64: one thread per item, CTAs of 256 threads with 5 (n_y - 1) doubles
+ * of shared memory; PDQ_MIXED: one thread per two samples of a class, CTAs of
+ * 512 threads with 5 (n_y - 1) pairs of floats.  Enqueued on `stream`; no allocation, no synchronisation.
  * Errors: INVALID_ARG (sizes, desc out of range, field radius != phys
  * Re_tau, NULL pointers), CUDA.                                              */
 int pdq_lf_vdep(const pdq_field* field, const pdq_phys* phys, const pdq_lf_desc* lf, const double* var,
