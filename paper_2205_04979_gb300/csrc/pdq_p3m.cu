@@ -366,9 +366,11 @@ __global__ void k_lf_table(double alpha, double umax, float4* tab) {
 
 // The particle-independent floats of the pair arithmetic.
 struct PPConst {
-    float Lh, Lm, Ll, invL;      // the period, split like a coordinate
+    float Lh, Lm, Ll;            // the period, split like a coordinate
     float rch, rcl, dch, dcl;    // r_cut^2 and d_c^2
     float kh, kl;                // table intervals per unit r^2
+    float L, invL, rc2;          // of the screen: the period and (r_cut + 1e-3)^2 + 1e-3
+    float wxy, R;                // cell width across, pipe radius
 };
 
 // One short-range pair: q_j (d / max(r, d_c)^3 - K_L(d)) when r < r_cut, in float-float (~145 FP32
@@ -422,12 +424,13 @@ __device__ __forceinline__ void pp_pair(const PPConst& K, const float4* T, const
 // evaluated with all lanes busy; the lanes' partial sums (about a dozen pairs each) are reduced in a
 // fixed order.
 // Bound by instruction issue (screening ~1,500 candidates and ~410 pairs of ~190 instructions per
-// particle).  One million particles, mesh 256^3: 5.9 ms (6.8 ms at 3 CTAs and 80 registers, 7.5 ms with the cell
+// particle).  One million particles, mesh 256^3: 5.4 ms (5.9 ms with PPConst worked out per thread: its FP64 was
+// repeated where registers ran short, pipe 53 % busy, now 8 %; 6.8 ms at 3 CTAs and 80 registers, 7.5 ms with the cell
 // index recomputed in FP64 by every lane); 42.4 ms in FP64 with the Hermite table in
 // global memory (FP64 pipe 87 % busy), 13.6 ms in float-float over the 27 cells of width r_cut.
 constexpr int kPPWarps = 8;
-__global__ void __launch_bounds__(32 * kPPWarps, 4) k_p3m_pp(const P3MGeom G, const P3MPart S, const int* start,
-                                                          int64_t ncells, const int* list,
+__global__ void __launch_bounds__(32 * kPPWarps, 4) k_p3m_pp(const P3MGeom G, const PPConst K, const P3MPart S,
+                                                          const int* start, int64_t ncells, const int* list,
                                                           const float4* __restrict__ sorted, int64_t stride,
                                                           double* sums) {
     __shared__ float4 T[2 * kTab];
@@ -437,20 +440,10 @@ __global__ void __launch_bounds__(32 * kPPWarps, 4) k_p3m_pp(const P3MGeom G, co
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int* qw = queue[w];
     const int n_live = start[ncells];
-    const float rcf = (float)G.rc + 1e-3f, rc2f = rcf * rcf + 1e-3f, Lf = (float)G.L, invLf = 1.0f / Lf;
-    PPConst K;
-    {
-        // (the floor keeps d_c^-3 inside FP32's range; it is 1e-10 wall units)
-        const double rc2 = G.rc * G.rc, dc2 = fmax(G.contact * G.contact, 1e-20), kk = kTab / rc2;
-        split3(G.grid, G.L, K.Lh, K.Lm, K.Ll);
-        K.invL = invLf;
-        K.rch = (float)rc2; K.rcl = (float)(rc2 - (double)K.rch);
-        K.dch = (float)dc2; K.dcl = (float)(dc2 - (double)K.dch);
-        K.kh = (float)kk; K.kl = (float)(kk - (double)K.kh);
-    }
+    const float rc2f = K.rc2, Lf = K.L, invLf = K.invL;
     const unsigned lt = (1u << lane) - 1u;
     const float4 *sh = sorted, *sm = sorted + stride, *sl = sorted + 2 * stride;
-    const float wxy = (float)(2.0 * G.R / G.ncx), Rf = (float)G.R;
+    const float wxy = K.wxy, Rf = K.R;
     for (int t = blockIdx.x * kPPWarps + w; t < n_live; t += gridDim.x * kPPWarps) {
         const float4 ih = sh[t], im = sm[t], il = sl[t];
         // column lane of the 5 x 5 around i: its runs [b0, e0) and, across the period, [b1, e1)
@@ -552,6 +545,21 @@ P3MGeom geom_of(const pdq_p3m* P, double contact) {
     G.lf_tab = P->lf_tab;
     G.grid = split_grid(std::max(P->R, P->L));
     return G;
+}
+
+PPConst pp_const_of(const P3MGeom& G) {
+    // (the floor keeps d_c^-3 inside FP32's range; it is 1e-10 wall units)
+    const double rc2 = G.rc * G.rc, dc2 = std::max(G.contact * G.contact, 1e-20), kk = kTab / rc2;
+    const float rcf = (float)G.rc + 1e-3f;
+    PPConst K;
+    split3(G.grid, G.L, K.Lh, K.Lm, K.Ll);
+    K.rch = (float)rc2; K.rcl = (float)(rc2 - (double)K.rch);
+    K.dch = (float)dc2; K.dcl = (float)(dc2 - (double)K.dch);
+    K.kh = (float)kk; K.kl = (float)(kk - (double)K.kh);
+    K.L = (float)G.L; K.invL = 1.0f / K.L;
+    K.rc2 = rcf * rcf + 1e-3f;
+    K.wxy = (float)(2.0 * G.R / G.ncx); K.R = (float)G.R;
+    return K;
 }
 
 void free_plan(pdq_p3m* P) {
@@ -676,6 +684,7 @@ extern "C" int pdq_p3m_coulomb(pdq_p3m* P, const pdq_phys* phys, const pdq_state
     if (st->n_classes < 1 || st->n_classes > PDQ_MAX_CLASSES) return PDQ_ERR_INVALID_ARG;
     int rc = PDQ_OK;
     const P3MGeom G = geom_of(P, contact_distance(phys, st));
+    const PPConst K = pp_const_of(G);
     std::vector<int64_t> off(st->n_samples + 1);
     std::vector<int32_t> cnt(st->n_samples);
     PDQ_CUDA(cudaMemcpyAsync(off.data(), st->offset, off.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
@@ -720,7 +729,7 @@ extern "C" int pdq_p3m_coulomb(pdq_p3m* P, const pdq_phys* phys, const pdq_state
         k_cell_sort<<<grid_of(P->ncells, 128), 128, 0, s>>>(P->cell_start, P->ncells, P->cell_list);
         k_cell_gather<<<gp, 256, 0, s>>>(G, S, P->cell_start, P->ncells, P->cell_list, P->sorted, P->max_n);
         k_p3m_pp<<<(unsigned)std::min<int64_t>(grid_of(S.n, kPPWarps), 16 * 152), 32 * kPPWarps, 0, s>>>(
-            G, S, P->cell_start, P->ncells, P->cell_list, P->sorted, P->max_n, sums);
+            G, K, S, P->cell_start, P->ncells, P->cell_list, P->sorted, P->max_n, sums);
     }
     PDQ_CUDA(cudaGetLastError());
     return PDQ_OK;

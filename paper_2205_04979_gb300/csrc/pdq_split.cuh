@@ -36,11 +36,12 @@ inline SplitGrid split_grid(double extent) {
     return SplitGrid{6755399441055744.0 * g, 6755399441055744.0 * g * 1.1920928955078125e-07};
 }
 // hi + mid + lo = x; off the grid's range (|x| > top) the parts still sum to x.
-__device__ __forceinline__ void split3(const SplitGrid& G, double x, float& hi, float& mid, float& lo) {
-    hi = (float)__dadd_rn(__dadd_rn(x, G.magic_hi), -G.magic_hi);
-    const double r = __dsub_rn(x, (double)hi);
-    mid = (float)__dadd_rn(__dadd_rn(r, G.magic_mid), -G.magic_mid);
-    lo = (float)__dsub_rn(r, (double)mid);
+__host__ __device__ __forceinline__ void split3(const SplitGrid& G, double x, float& hi, float& mid, float& lo) {
+    // sums only, so no contraction can change them
+    hi = (float)((x + G.magic_hi) - G.magic_hi);
+    const double r = x - (double)hi;
+    mid = (float)((r + G.magic_mid) - G.magic_mid);
+    lo = (float)(r - (double)mid);
 }
 
 // Separation (D, E) of two split coordinates.  The hi parts' difference is 0 or at least g, the mid
