@@ -151,14 +151,21 @@ static int launch_sums_d(const SumArgs& A, int ctas, int n_boot, cudaStream_t s)
 // A cluster takes all outputs (up to 32) with one CTA; while the clusters of a model are too few to give every SM
 // 8 CTAs, and a thread keeps 12 positions of the longest model, the cluster grows to 8 CTAs and then
 // takes fewer outputs, at the price of partly used sectors.  No replicates, 40,000 groups, 10 outputs: 0.10 ms
-// (0.45 ms with 4 CTAs for all outputs, 0.30 ms with a CTA per output).
+// (0.45 ms with 4 CTAs for all outputs, 0.30 ms with a CTA per output).  While SMs are idle an output more or less
+// costs a CTA nothing, so there a thread keeps only 2 positions: the few CTAs' FP64 pipes are the bound
+// (no replicates, 600 groups, 3 inputs, 10 outputs: 66 to 72 us a call; 79 us without this, 71 us with a CTA per
+// output).
 static int launch_sums(SumArgs A, int n_boot, int sms, cudaStream_t s) {
     int ctas = 1;
     A.outs = A.C < kSumOutputs ? A.C : kSumOutputs;
     const auto few = [&] { return (int64_t)((A.C + A.outs - 1) / A.outs) * (1 + n_boot) * ctas < 8 * (int64_t)sms; };
-    const auto keeps = [&](int outs, int n) { return A.m[A.k - 1] >= (int64_t)12 * n * (kSumThreads / outs); };
-    while (ctas < 8 && few() && keeps(A.outs, 2 * ctas)) ctas *= 2;
-    while (A.outs > 1 && few() && keeps((A.outs + 1) / 2, ctas)) A.outs = (A.outs + 1) / 2;
+    const auto keeps = [&](int outs, int n, int positions) {
+        return A.m[A.k - 1] >= (int64_t)positions * n * (kSumThreads / outs);
+    };
+    const auto idle = [&] { return (int64_t)((A.C + A.outs - 1) / A.outs) * (1 + n_boot) * ctas * A.k < sms; };
+    while (ctas < 8 && few() && keeps(A.outs, 2 * ctas, 12)) ctas *= 2;
+    while (A.outs > 1 && few() && keeps((A.outs + 1) / 2, ctas, 12)) A.outs = (A.outs + 1) / 2;
+    while (A.outs > 1 && idle() && keeps((A.outs + 1) / 2, ctas, 2)) A.outs = (A.outs + 1) / 2;
     switch (A.d) {
         case 1: return launch_sums_d<1>(A, ctas, n_boot, s);
         case 2: return launch_sums_d<2>(A, ctas, n_boot, s);
