@@ -246,7 +246,8 @@ typedef struct pdq_tally {
 
 /* Workspace bytes pdq_step_particles needs for this state and configuration
  * (the work-item table; MIXED: the z-binning sort's scratch; pair variant 3:
- * 16 B (MIXED) or 24 B (PDQ_FP64) x capacity of sums; PDQ_FP64 with few
+ * 16 B (MIXED) or 24 B (PDQ_FP64) x capacity of sums, and for PDQ_FP64 from
+ * 32,768 slots on 80 B per sample for the far pairs' choices; PDQ_FP64 with few
  * i-tiles, one-sided: per-chunk partial pair sums, 24 B x particles x chunks,
  * chunks <= 64, chosen from the capacity, the tile and the device's SM
  * count).                                                                    */
@@ -264,10 +265,16 @@ int pdq_step_workspace_size(const pdq_state* state, const pdq_step_cfg* cfg, siz
  *   exponential integrator with u, f, a frozen over the step;
  *   wall contact when R - r - d/2 <= 0: STICK removes the particle,
  *   REBOUND applies CoR_n of Sec. 4.3 (sticking when it is 0).
- * FP64 runs everything in double, except that pair variant 3 sums the far
- * pairs of samples of 8,192 particles and more in pairs of floats (each pair
- * to 2^-46, the sums no further from the exact ones than double's); MIXED
- * keeps x, y, the wall gap, the vdW
+ * FP64 runs everything in double, except that pair variant 3 may sum the far
+ * pairs of samples of 32,768 particles and more in pairs of floats (~2^-47.6
+ * each).  It does so for a sample and step where 128 of its particles show
+ * those terms to be small against the sums; on the clouds measured (32,768 to
+ * 150,000 particles) a particle's sum is then off by 2.5 to 5 x 2^-53 of it in
+ * the median, as in double (3 to 5).  Charges of both signs in equal parts, a
+ * few that outweigh the rest and particles bunched along z stay in double, and
+ * so does any sample when the workspace is smaller than
+ * pdq_step_workspace_size (the room for the choices is left out first).  Pair
+ * variant 0 is double throughout.  MIXED keeps x, y, the wall gap, the vdW
  * term and the tallies in double and runs the pair sum, interpolation, drag
  * and velocities in float.  `workspace` (>= pdq_step_workspace_size bytes,
  * device, 256-byte aligned) holds the work queue.  The particles of each

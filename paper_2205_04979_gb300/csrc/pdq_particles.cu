@@ -175,6 +175,16 @@ __device__ __forceinline__ void coulomb_pair_x2s(f2 xi, f2 yi, f2 zi, f2 xj, f2 
     az[0] = __fmaf_rn(s0, z0, az[0]); az[1] = __fmaf_rn(s1, z1, az[1]);
 }
 
+// FP64 pair variant 3, per sample and step: what the probes found, and whether and from which z
+// distance on k_pairs_split64 sums the sample's pairs in float-float (0: not at all).
+constexpr int kSplitTries = 4;
+struct SplitChoice {
+    double far;
+    unsigned long long near[kSplitTries];
+    int half[kSplitTries], tail[kSplitTries];
+    int bad, done;
+};
+
 struct StepArgs {
     StepConst K;
     const void* pos_in; const void* vel_in; const double2* xy_in;
@@ -197,6 +207,8 @@ struct StepArgs {
     // MIXED pair variant 3: particles per thread of k_pairs_sym and CTAs per tile (newton_cut)
     int newton_u, newton_parts;
     SplitGrid grid;      // FP64 pair variant 3: of the split coordinates (k_pairs_split64)
+    SplitChoice* split;  // [n_samples], or NULL: every pair in FP64
+    int n_samples;
     // host only: upper bound on the work items of a launch (the persistent grid is capped by it,
     // so that few items spread one per CTA over the SMs instead of piling onto the first CTAs)
     int64_t max_items;
@@ -1030,9 +1042,99 @@ __global__ void __launch_bounds__(NT, (U == 12 ? 3 : U == 8 ? 4 : 5) * (128 / NT
                             gridDim.y);
 }
 
-// Samples of at least this many particles take k_pairs_split64 instead of k_pairs_sym64 (pair variant
-// 3 in FP64).
-constexpr int kSplitMin = 8192;
+// Which samples take k_pairs_split64 instead of k_pairs_sym64 (pair variant 3 in FP64).  Its far pairs carry
+// ~2^-47.6 each (float-float: some 20 roundings of 2^-49), double's 2^-52, so the sums stay as exact as
+// double's only where the far terms are small against the sum.  Measured on clouds of 8,192 to 100,000 particles
+// (one charge, lognormal, 3 to 10 classes, both signs, a few huge charges, bunches, a lattice; 512 particles
+// each against double-double), the median error of a particle's sum in units of 2^-53 of it is
+// sqrt(2^2 + (85 rho)^2) within 10 %, rho = sqrt(sum over far pairs of f^2) / |sum f|.  k_pairs_sym64's is 2.4 at
+// 8,192 and 2.6 at 16,384 particles, 3.4 from 32,768 on (its chunks lengthen) and 4.5 at 100,000.  So:
+//   - samples of kSplitMin particles and more;
+//   - rho <= 0.029 (n / 32768)^(1/4) for half of kProbes particles spread over the sample, three times that
+//     for nine tenths of them, by the nearest of kSplitTries limits of far that satisfies both; charges of
+//     both signs in equal parts or a few that outweigh the rest have rho 0.3 to 1 and stay in FP64;
+//   - near pairs, which k_pairs_split64 evaluates from both sides, at most a quarter (100,000 particles bunched
+//     along z, near share ~0.5: 210 ms per step against k_pairs_sym64's 193);
+//   - coordinates on the split grid, sums inside FP32's range.
+constexpr int kSplitMin = 32768, kProbes = 128;
+
+// Probe blockIdx.x of the samples blockIdx.y, blockIdx.y + gridDim.y, ...: its sum and its far terms (FP32 does),
+// tallied per sample; the last probe of a sample decides.  kProbes CTAs read the sample's positions from L2 once
+// each: ~0.04 ms at 100,000 particles.
+__global__ void __launch_bounds__(256) k_split_choose(const StepArgs A) {
+    __shared__ float s_red[8][4 + 2 * kSplitTries];
+    const StepConst& K = A.K;
+    const double4_32a* __restrict__ pos_in = (const double4_32a*)A.pos_in;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const float L = (float)K.L, invL = (float)K.invL, c2 = (float)K.contact2, top = A.grid.top;
+    for (int s = blockIdx.y; s < A.n_samples; s += gridDim.y) {
+        const int n = A.count[s];
+        if (n < kSplitMin) continue;
+        const int64_t o = A.offset[s];
+        const int i = (int)((2 * blockIdx.x + 1) * (int64_t)n / (2 * kProbes));
+        const double4_32a pi = pos_in[o + i];
+        const float xi = (float)pi.x, yi = (float)pi.y, zi = (float)pi.z;
+        const double spacing = cbrt(kPi * K.R * K.R * K.L / (double)n), dcz = sqrt(K.contact2) + 1e-9;
+        auto limit = [&](int m) {
+            const double mult = m == 0 ? 2.0 : m == 1 ? 3.0 : m == 2 ? 4.5 : 6.0;
+            return fmax(dcz, mult * spacing);
+        };
+        float far[kSplitTries], v[4 + 2 * kSplitTries];      // sum x, y, z; off the grid; far f^2; near count
+#pragma unroll
+        for (int m = 0; m < kSplitTries; ++m) far[m] = (float)limit(m);
+#pragma unroll
+        for (int k = 0; k < 4 + 2 * kSplitTries; ++k) v[k] = 0.f;
+#pragma unroll 4
+        for (int j = tid; j < n; j += 256) {
+            const double4_32a p = pos_in[o + j];
+            const float x = (float)p.x, y = (float)p.y, z = (float)p.z;
+            if (!(fmaxf(fabsf(x), fmaxf(fabsf(y), fabsf(z))) <= top)) v[3] = 1.f;
+            const float dx = xi - x, dy = yi - y;
+            float dz = zi - z;
+            dz -= L * rintf(dz * invL);
+            const float r2 = fmaxf(dx * dx + dy * dy + dz * dz, c2), ri = rsqrtf(r2);
+            const float w = j == i ? 0.f : (float)p.w * ri * ri * ri, f2 = w * w * r2;
+            v[0] += w * dx; v[1] += w * dy; v[2] += w * dz;
+#pragma unroll
+            for (int m = 0; m < kSplitTries; ++m) {
+                if (fabsf(dz) > far[m]) v[4 + m] += f2;
+                else v[4 + kSplitTries + m] += 1.f;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4 + 2 * kSplitTries; ++k) {
+            for (int d = 16; d > 0; d >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], d);
+            if (lane == 0) s_red[warp][k] = v[k];
+        }
+        __syncthreads();
+        if (tid == 0) {
+            for (int k = 0; k < 4 + 2 * kSplitTries; ++k)
+                for (int w = 1; w < 8; ++w) s_red[0][k] += s_red[w][k];
+            const float* t = s_red[0];
+            const float s2 = t[0] * t[0] + t[1] * t[1] + t[2] * t[2];
+            const float rho = 0.029f * sqrtf(sqrtf((float)n / 32768.f)), lim = rho * rho * s2;
+            SplitChoice& C = A.split[s];
+            if (t[3] > 0.f) atomicOr(&C.bad, 1);
+            for (int m = 0; m < kSplitTries; ++m) {
+                atomicAdd(&C.near[m], (unsigned long long)t[4 + kSplitTries + m]);
+                if (!(s2 > 1e-24f && s2 < 1e24f)) continue;      // f^2 of the far pairs may leave FP32's range
+                if (t[4 + m] <= lim) atomicAdd(&C.half[m], 1);
+                if (t[4 + m] <= 9.f * lim) atomicAdd(&C.tail[m], 1);
+            }
+            __threadfence();
+            if (atomicAdd(&C.done, 1) == kProbes - 1) {
+                __threadfence();
+                double choice = 0.0;
+                for (int m = kSplitTries - 1; m >= 0; --m)
+                    if (atomicAdd(&C.half[m], 0) >= kProbes / 2 && atomicAdd(&C.tail[m], 0) >= kProbes * 9 / 10 &&
+                        atomicAdd(&C.near[m], 0ull) <= (unsigned long long)n * (kProbes / 4) && !atomicOr(&C.bad, 0))
+                        choice = limit(m);
+                C.far = choice;
+            }
+        }
+        __syncthreads();
+    }
+}
 
 // FP64 Newton pair: coulomb_pair_x2_sym for one i-particle in double (minimum image by the
 // 1.5 * 2^52 rounding constant, as the one-sided FP64 pair).
@@ -1088,7 +1190,7 @@ __global__ void __launch_bounds__(NT) k_pairs_sym64(const StepArgs A) {
         const int2 it = A.items[item];
         const int64_t o = A.offset[it.x];
         const int64_t end = o + A.count[it.x];
-        if (end - o >= kSplitMin) {      // k_pairs_split64's
+        if (A.split && end - o >= kSplitMin && A.split[it.x].far > 0.0) {      // k_pairs_split64's
             __syncthreads();
             continue;
         }
@@ -1252,19 +1354,19 @@ __global__ void __launch_bounds__(NT) k_pairs_sym64(const StepArgs A) {
     }
 }
 
-// FP64 Coulomb sums of large samples, one-sided, with the far pairs on the FP32 pipe: a j group whose
-// z distance from the warp's i-particles exceeds twice the sample's mean spacing is summed in float-float
-// (pdq_split.cuh, ~2^-46 per pair, three-float accumulators), the near groups in FP64.  A far pair's
-// term is small against the sum, so its rounding is too: over samples of 8,192 to 100,000 particles
-// the sums are no further from the exact ones than k_pairs_sym64's.  Below kSplitMin the near share
-// grows and that no longer holds.  The item table is k_pairs_sym64's (tiles of 2 NT particles, JS
-// chunks of the sample's j range); each CTA adds its item's sums to A.acc64 by atomics.
-// Bound by the FP32 FMA pipe (~135 operations per ordered pair, packed for two i).  100,000 particles,
-// 64 threads: 55.5 ms per step, 192 ms in k_pairs_sym64 (FP64 pipe 90 % busy); error of the sums against
-// extended precision, in units of 2^-53 of their 2-norm: 3.8 (6.3 before), at 8,192 particles 5.8 (5.7).
-// Three-float accumulators that are flushed once per j-tile instead of once per group left 7 and 14 units, without
-// the second word of the sums 24 and 38.  Splitting the groups near in z by the pairs' distances instead (FP64
-// within one mean spacing) took 47 ms, but left 8.4 units at 100,000 particles.
+// FP64 Coulomb sums of the samples that k_split_choose picked, one-sided, with the far pairs on the FP32 pipe: a j
+// group whose z distance from the warp's i-particles exceeds the chosen limit is summed in float-float
+// (pdq_split.cuh, ~2^-47.6 per pair, three-float accumulators), the near groups in FP64.  The item table is
+// k_pairs_sym64's (tiles of 2 NT particles, JS chunks of the sample's j range); each CTA adds its item's sums to
+// A.acc64 by atomics.
+// Bound by the FP32 FMA pipe (~135 operations per ordered pair, packed for two i).  100,000 particles, 64 threads: 54 ms
+// per step for one class (far from 2 mean spacings on), 58 ms for 10 classes with lognormal charges (from 3), 192 ms
+// in k_pairs_sym64; 32,768: 8.0 to 12.4 ms against 21.7.  Median error of a particle's sum in units of 2^-53 of
+// it, over clouds of one sign: 2.7 to 4.2 at 100,000 (k_pairs_sym64 4.2 to 5.2), 2.6 to 4.6 at 65,536 (3.7 to
+// 4.5), 2.7 to 3.3 at 32,768 (3.2 to 3.8); clouds of both signs take k_pairs_sym64.
+// Three-float accumulators that are flushed once per j-tile instead of once per group left 7 and 14 units (8,192 and
+// 100,000 particles), without the second word of the sums 24 and 38.  Splitting the groups near in z by the pairs'
+// distances instead (FP64 within one mean spacing) took 47 ms, but left 8.4 units at 100,000 particles.
 template <int NT>
 __global__ void __launch_bounds__(NT, 384 / NT) k_pairs_split64(const StepArgs A) {
     constexpr int W = NT / 32;
@@ -1278,14 +1380,14 @@ __global__ void __launch_bounds__(NT, 384 / NT) k_pairs_split64(const StepArgs A
     const int2 it = A.items[item];
     const int64_t o = A.offset[it.x], end = o + A.count[it.x], n = end - o;
     if (n < kSplitMin) return;
+    const double far = A.split[it.x].far;
+    if (!(far > 0.0)) return;
     const int JS = A.jsplit, tile = it.y / JS, jc = it.y - tile * JS;
     const int64_t base = o + (int64_t)tile * (2 * NT), ch = ((n + JS - 1) / JS + NT - 1) / NT * NT;
     const int64_t jb = o + jc * ch, je = jb + ch < end ? jb + ch : end;
     if (jb >= je) return;
     const double4_32a* __restrict__ pos_in = (const double4_32a*)A.pos_in;
     const double L = K.L, invL = K.invL, c2 = K.contact2, halfL = 0.5 * L;
-    const double dcz = sqrt(c2) + 1e-9;        // contact distance + rounding margin
-    const double far = fmax(dcz, 2.0 * cbrt(kPi * K.R * K.R * L / (double)n));
     // this lane's two i-particles, a contiguous run of 64 per warp
     double xi[2], yi[2], zi[2], sum[3][2];
     double ilo = INFINITY, ihi = -INFINITY;
@@ -1898,9 +2000,13 @@ static int launch_newton64(const StepArgs& A, cudaStream_t s) {
     const int64_t full = (int64_t)sm_count() * per_sm;
     PDQ_CUDA(cudaMemsetAsync(A.acc64, 0, 3 * sizeof(double) * (size_t)(A.cap > 0 ? A.cap : 1), s));
     if (A.K.forces & PDQ_F_COULOMB) {    // the sums enter the update only with the Coulomb force on
+        if (A.split) {
+            PDQ_CUDA(cudaMemsetAsync(A.split, 0, sizeof(SplitChoice) * (size_t)A.n_samples, s));
+            k_split_choose<<<dim3(kProbes, (unsigned)std::min<int64_t>(A.n_samples, A.cap / kSplitMin)), 256, 0, s>>>(A);
+        }
         k_pairs_sym64<NT, 2><<<(unsigned)std::max<int64_t>(1, std::min(full, A.max_items > 0 ? A.max_items : full)),
                                NT, 0, s>>>(A);
-        if (A.cap >= kSplitMin)
+        if (A.split)
             k_pairs_split64<NT><<<(unsigned)std::max<int64_t>(1, A.max_items), NT, 0, s>>>(A);
     }
     StepArgs B = A;
@@ -2034,10 +2140,12 @@ static int newton_chunks(const pdq_state* st, int TI, bool coarse) {
 
 // Workspace: items | order | tag scratch of the z-binning sort;
 // FP64 with JS > 1 (one-sided): tile counters | partial sums [JS][3][capacity];
-// pair variant 3: the sums, float4 [capacity] (MIXED) or double [capacity][3] (FP64).
+// pair variant 3: the sums, float4 [capacity] (MIXED) or double [capacity][3] (FP64), and the choices of
+// k_split_choose where a sample can be large enough (*split_off; 0 where not, and with `coarse`).
 static void workspace_layout(const pdq_state* st, int TI, size_t* items_bytes, size_t* total,
                              size_t* cnt_off = nullptr, size_t* part_off = nullptr, bool contact = false,
-                             size_t* acc_off = nullptr, bool newton = false, bool coarse = false) {
+                             size_t* acc_off = nullptr, bool newton = false, bool coarse = false,
+                             size_t* split_off = nullptr) {
     const int JS = newton ? newton_chunks(st, TI, coarse) : j_split(st, TI, contact, coarse);
     const int64_t max_tiles = st->capacity / TI + st->n_samples + 1;
     *items_bytes = align256(sizeof(int2) * (size_t)max_tiles * JS);
@@ -2047,6 +2155,9 @@ static void workspace_layout(const pdq_state* st, int TI, size_t* items_bytes, s
         if (acc_off) *acc_off = *total;
         const size_t per = st->precision == PDQ_FP64 ? 3 * sizeof(double) : sizeof(float4);
         *total += align256(per * (size_t)(st->capacity > 0 ? st->capacity : 1));
+        const bool split = st->precision == PDQ_FP64 && st->capacity >= kSplitMin && !coarse;
+        if (split_off) *split_off = split ? *total : 0;
+        if (split) *total += align256(sizeof(SplitChoice) * (size_t)st->n_samples);
     }
     if (JS > 1 && !newton) {
         if (cnt_off) *cnt_off = *total;
@@ -2207,8 +2318,8 @@ int step_impl(const pdq_field* field, const pdq_phys* phys, pdq_state* st, const
     if (NT != 64 && NT != 128 && NT != 256 && !(NT == 32 && st->precision == PDQ_FP64)) return PDQ_ERR_INVALID_ARG;
     const bool newton = !ext && newton_pairs(st, cfg);
     if (newton && NT != 64 && NT != 128) return PDQ_ERR_INVALID_ARG;   // its update step runs 2 NT threads
-    size_t items_bytes, need, cnt_off = 0, part_off = 0, acc_off = 0;
-    workspace_layout(st, NT * U, &items_bytes, &need, &cnt_off, &part_off, contact, &acc_off, newton);
+    size_t items_bytes, need, cnt_off = 0, part_off = 0, acc_off = 0, split_off = 0;
+    workspace_layout(st, NT * U, &items_bytes, &need, &cnt_off, &part_off, contact, &acc_off, newton, false, &split_off);
     if (newton && st->precision == PDQ_MIXED) {
         cut = mixed_cut(st, cfg);
         // a workspace that only fits the item table of whole, wide tiles takes those
@@ -2222,7 +2333,8 @@ int step_impl(const pdq_field* field, const pdq_phys* phys, pdq_state* st, const
     bool coarse = false;
     if (!ext && st->precision == PDQ_FP64 && workspace_bytes < need) {      // likewise for fewer chunks
         coarse = true;
-        workspace_layout(st, NT * U, &items_bytes, &need, &cnt_off, &part_off, contact, &acc_off, newton, coarse);
+        workspace_layout(st, NT * U, &items_bytes, &need, &cnt_off, &part_off, contact, &acc_off, newton, coarse,
+                         &split_off);
     }
     if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255)) return PDQ_ERR_WORKSPACE;
     const int JS = newton ? newton_chunks(st, NT * U, coarse) : j_split(st, NT * U, contact || ext, coarse);
@@ -2254,6 +2366,8 @@ int step_impl(const pdq_field* field, const pdq_phys* phys, pdq_state* st, const
     A.ext = ext;
     if (newton && st->precision == PDQ_MIXED) A.acc4 = (float4*)((char*)workspace + acc_off);
     if (newton && st->precision == PDQ_FP64) A.acc64 = (double*)((char*)workspace + acc_off);
+    if (split_off) A.split = (SplitChoice*)((char*)workspace + split_off);
+    A.n_samples = st->n_samples;
     A.max_items = (st->capacity / (NT * U) + st->n_samples + 1) * JS;
     if (JS > 1 && !newton) {
         A.tile_cnt = (int*)((char*)workspace + cnt_off);

@@ -5,7 +5,7 @@
 //
 // A coordinate is cut into three floats on fixed grids, hi + mid + lo (all 53 bits), so the
 // differences of the hi and of the mid parts are exact; a separation is then a float-float (D, E)
-// and everything after it carries ~47 bits.
+// and everything after it carries ~47 bits (a pair's term is off by 2^-47.6 of it, rms).
 #pragma once
 
 #include "pdq_device.cuh"
@@ -27,13 +27,14 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // rounds a double to a multiple of g.  g = 2^-23 times a power of two above every coordinate.
 struct SplitGrid {
     double magic_hi, magic_mid;
+    float top, g;
 };
 inline SplitGrid split_grid(double extent) {
     double top = 1.0;
     while (top < extent) top *= 2.0;
     while (top > 2.0 * extent) top *= 0.5;
     const double g = top * 1.1920928955078125e-07;                    // 2^-23
-    return SplitGrid{6755399441055744.0 * g, 6755399441055744.0 * g * 1.1920928955078125e-07};
+    return SplitGrid{6755399441055744.0 * g, 6755399441055744.0 * g * 1.1920928955078125e-07, (float)top, (float)g};
 }
 // hi + mid + lo = x; off the grid's range (|x| > top) the parts still sum to x.
 __host__ __device__ __forceinline__ void split3(const SplitGrid& G, double x, float& hi, float& mid, float& lo) {

@@ -281,6 +281,54 @@ def test_fp64_newton_pairs_large_samples(pdq, fields, counts, block):
     assert np.sqrt(float(err / ref)) <= 24 * 2.0 ** -53
 
 
+@pytest.mark.parametrize("n,cloud", [(32768, "uniform"), (40000, "classes"), (32768, "signs"), (40000, "few"),
+                                     (32768, "bunched")])
+def test_fp64_newton_pairs_hard_clouds(pdq, fields, n, cloud):
+    # the Coulomb sums of large FP64 samples whose far pairs outweigh the near ones: charges of both signs, 10
+    # charges 10^4 times the others; 10 classes of charges 1..1000; half the particles in a slab 10 wide.  Sums from
+    # a step of that force from rest, against extended precision on 32 particles.  Bar of the median error: FP64
+    # chains of n / 64 <= 625 adds round to 0.29 sqrt(625) = 7.2 units of 2^-53, far pairs where they may carry
+    # 2^-47 leave 3 at their limit; 12 units.  The choice stands at the end of the workspace: float-float from a
+    # distance for the first two, none for the others.
+    rng = np.random.default_rng(n)
+    r, th = 178.0 * np.sqrt(rng.random(n)), 2 * np.pi * rng.random(n)
+    X = np.stack([r * np.cos(th), r * np.sin(th), 720.0 * rng.random(n)], 1)
+    q = np.full(n, 37.0)
+    if cloud == "classes":
+        q = np.geomspace(1.0, 1000.0, 10)[np.arange(n) % 10]
+    elif cloud == "signs":
+        q *= np.where(rng.random(n) < 0.5, -1.0, 1.0)
+    elif cloud == "few":
+        q[rng.choice(n, 10, replace=False)] *= 1e4
+    elif cloud == "bunched":
+        X[: n // 2, 2] = 360.0 + 10.0 * rng.random(n // 2)
+    phys, st = pdq.phys_default(), pdq.State(pdq.FP64, [n], [10.0])
+    prm = pdq.params_tensor(PRM3[:1])
+    pdq.seed_particles(fields[0], phys, st, prm, 1)
+    st.pos[0][:, :3], st.pos[0][:, 3] = torch.tensor(X, device="cuda"), torch.tensor(q, device="cuda")
+    cfg = pdq.step_cfg(1e-6, forces=pdq.F_COULOMB, gravity=(0, 0, 0), block=64, variant=3)
+    ws = pdq.workspace(st, cfg)
+    pdq.step_particles(fields[0], phys, st, prm, cfg, 1, pdq.Tally(1, 1), ws)
+    v = np.zeros((n, 3))
+    v[st.tag.cpu().numpy()[:, 0]] = st.current()[1].cpu().numpy()[:, :3]
+    ld = np.longdouble
+    X, q = X.astype(ld), q.astype(ld)
+    dc2 = ld(oracle.class_table([10.0])[0, 1]) ** 2
+    idx = rng.choice(n, 32, replace=False)
+    want = []
+    for i in idx:
+        d = X[i] - X
+        d[:, 2] -= 720 * np.rint(d[:, 2] / 720)
+        r2 = np.maximum((d * d).sum(1), dc2)
+        want.append(q[i] * (q[:, None] * d / (r2 * np.sqrt(r2))[:, None]).sum(0))
+    want = np.array(want)
+    k = (want * v[idx]).sum() / (want * want).sum()           # the class's coefficient, with its rounding
+    err = np.sqrt(((v[idx] / k - want) ** 2).sum(1) / (want * want).sum(1))
+    assert float(np.median(err)) <= 12 * 2.0 ** -53
+    far = float(ws[-256:-248].view(torch.float64))
+    assert far > 0 if cloud in ("uniform", "classes") else far == 0
+
+
 @pytest.mark.parametrize("counts", [[1], [31], [32, 0, 33], [700, 5, 129], [2048], [2049]])
 def test_fp64_tile_pairs_of_small_samples(pdq, fields, counts):
     # 32 threads and up to 2,048 particles: sums by pairs of 32-particle tiles (one tile, a partial one, an even
