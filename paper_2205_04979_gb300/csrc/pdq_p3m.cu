@@ -14,8 +14,8 @@
 //          component -> inverse FFT -> TSC interpolation; then a cell list
 //          (cells >= r_cut/2 x r_cut/4, stable per-cell order, particles copied in
 //          cell order) and the direct short-range sum with the minimum image along z.
-// FP64 on the mesh (cuFFT does the transforms), float-float for the short-range pairs
-// (pdq_split.cuh).  One sample at a time.
+// FP64 on the mesh (cuFFT does the transforms) and for the short-range pairs of the inner half of r_cut; the outer
+// ones, where K_S is below a sixth of 1/r^3, in float-float (pdq_split.cuh).  One sample at a time.
 #include <cufft.h>
 #include <math.h>
 
@@ -46,9 +46,9 @@ struct pdq_p3m {
     int* cell_start;            // [ncells + 1]
     int* cell_fill;             // [ncells]
     int* cell_list;             // [max_n]
-    float4* sorted;             // [3][max_n] live particles in cell order, split: x, y, z hi and q hi; mid and q lo;
-                                // lo and the cell's index
-    float4* lf_tab;             // [2][kTab] K_L factor by quartics on kTab intervals of u = (alpha r)^2 < (alpha r_cut)^2
+    double4_32a* sorted64;      // [max_n] live particles in cell order: x, y, z, q
+    float4* sorted;             // [3][max_n] the same, split: x, y, z hi and q hi; mid and q lo; lo and the cell's index
+    float4* ks_tab;             // short-range factor: near_tab and far_tab, kTabWords
     double* sums;               // [sums_cap][3], for the step driver
     int64_t sums_cap;
 };
@@ -59,14 +59,20 @@ namespace {
 struct P3MGeom {
     double R, L, h, hz, x0, alpha, rc, contact;
     int Mx, Nx, Nz, n_img, ncx, ncz;
-    const float4* lf_tab;
+    const float4* ks_tab;
     SplitGrid grid;             // of the split coordinates
 };
 
-// The short-range pairs read the long-range factor from quartics in u = (alpha r)^2, one per interval
-// of a table (through 5 Chebyshev nodes each: relative interpolation error ~2e-15 at alpha r_cut = 3.3),
-// instead of erf and exp.  1,024 intervals of 32 B fit shared memory beside the pair queues.
-constexpr int kTab = 1024;
+// The short-range pairs read K_S's factor 1/r^3 - K_L from polynomials in r^2, in place of the reciprocal square root, K_L
+// and their difference; both tables fit shared memory beside the queues.
+// Inner pairs, r < r_n: sextics in FP64 on kOct octaves of 64 intervals each that end at the first power of two from
+// r_n^2 on.  Through 7 Chebyshev nodes (h/(4 r^2))^7 <= 2^-56 of a power law remains; where the factor falls off
+// faster it is small against 1/r^3, which is what its error matters against.  Closer pairs (below r_n/16, or
+// inside the contact distance) take pp_close.
+// Outer pairs, r_n = r_cut/2 <= r: quintics on kFar intervals, in float-float down to t^2; t^3 carries 7e-7 of the value,
+// so its float leaves 2^-45 of K_S, 2^-48 of 1/r^3.
+constexpr int kOct = 8, kNear = 64 * kOct, kFar = 512;
+constexpr int kTabWords = 7 * kNear / 2 + 2 * kFar + kFar / 2;      // in float4
 
 struct P3MPart {                // the particles of one sample, current half of the state
     const void* pos;
@@ -306,18 +312,21 @@ __global__ void k_cell_sort(const int* start, int64_t ncells, int* list) {
     }
 }
 
-// Live particles copied in cell order, their coordinates and charge split into floats.
+// Live particles copied in cell order, in FP64 and split into floats.  A particle whose coordinates lie off the split
+// grid, or whose charge leaves FP32's range, gets a split charge that is none, and its pairs all run in FP64.
 __global__ void k_cell_gather(const P3MGeom G, const P3MPart S, const int* start, int64_t ncells, const int* list,
-                              float4* sorted, int64_t stride) {
+                              double4_32a* s64, float4* sorted, int64_t stride) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= start[ncells]) return;
     double x, y, z, q;
     load_particle(S, S.o + list[t], x, y, z, q);
+    s64[t] = make_double4_32a(x, y, z, q);
     float4 h, m, l;
     split3(G.grid, x, h.x, m.x, l.x);
     split3(G.grid, y, h.y, m.y, l.y);
     split3(G.grid, z, h.z, m.z, l.z);
-    h.w = (float)q;
+    const bool fits = fmax(fabs(x), fmax(fabs(y), fabs(z))) <= (double)G.grid.top && (q == 0.0 || (fabs(q) > 1e-15 && fabs(q) < 1e20));
+    h.w = fits ? (float)q : NAN;
     m.w = (float)(q - (double)h.w);
     l.w = __int_as_float(cell_of(G, x, y, z));
     sorted[t] = h;
@@ -325,87 +334,144 @@ __global__ void k_cell_gather(const P3MGeom G, const P3MPart S, const int* start
     sorted[2 * stride + t] = l;
 }
 
-// K_L factor at u = (alpha r)^2: c alpha^3 sum_m (-1)^m 2 u^m / (m! (2m + 3)) below u = 1 (where the
-// closed form cancels), the closed form above.
-__device__ __forceinline__ double long_factor_u(double u, double alpha) {
-    const double c = 1.1283791670955126, a3 = alpha * alpha * alpha;
-    if (u < 1.0) {
-        double s = 0.0, t = 1.0;                    // t = (-u)^m / m!
-        for (int m = 0; m < 24; ++m) {
-            s += 2.0 * t / (2 * m + 3);
-            t *= -u / (m + 1);
-        }
-        return c * a3 * s;
+// One thread per interval: the polynomial in t = r^2 - (the interval's lower edge) through N Chebyshev nodes, by divided
+// differences over the interval's width h (a power of two, or any), expanded to powers.
+template <int N>
+__device__ void ks_poly(double alpha, double lower, double h, double p[N]) {
+    double x[N], f[N];
+    for (int i = 0; i < N; ++i) {
+        x[i] = 0.5 - 0.5 * cos(kPi * (2 * i + 1) / (2.0 * N));
+        const double r2 = lower + h * x[i], r = sqrt(r2);
+        f[i] = erfc(alpha * r) / (r2 * r) + 1.1283791670955126 * alpha * exp(-alpha * alpha * r2) / r2;
     }
-    const double x = sqrt(u);
-    return a3 * (erf(x) / (u * x) - c * exp(-u) / u);
-}
-
-// One thread per interval: the quartic in t = position inside the interval (0..1) through the five
-// Chebyshev nodes, by divided differences expanded to powers; the two leading coefficients as
-// float-floats.
-__global__ void k_lf_table(double alpha, double umax, float4* tab) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= kTab) return;
-    double x[5], f[5];
-    for (int i = 0; i < 5; ++i) {
-        x[i] = 0.5 - 0.5 * cos(kPi * (2 * i + 1) / 10.0);
-        f[i] = long_factor_u(umax * (k + x[i]) / kTab, alpha);
-    }
-    for (int j = 1; j < 5; ++j)
-        for (int i = 4; i >= j; --i) f[i] = (f[i] - f[i - 1]) / (x[i] - x[i - j]);
-    double p[5] = {f[4], 0.0, 0.0, 0.0, 0.0};
-    for (int i = 3; i >= 0; --i) {                  // p <- p (t - x_i) + f_i
-        for (int j = 4; j > 0; --j) p[j] = p[j - 1] - x[i] * p[j];
+    for (int j = 1; j < N; ++j)
+        for (int i = N - 1; i >= j; --i) f[i] = (f[i] - f[i - 1]) / (x[i] - x[i - j]);
+    p[0] = f[N - 1];
+    for (int j = 1; j < N; ++j) p[j] = 0.0;
+    for (int i = N - 2; i >= 0; --i) {              // p <- p (t - x_i) + f_i
+        for (int j = N - 1; j > 0; --j) p[j] = p[j - 1] - x[i] * p[j];
         p[0] = f[i] - x[i] * p[0];
     }
-    const float c0 = (float)p[0], c1 = (float)p[1];
-    tab[k] = make_float4(c0, (float)(p[0] - (double)c0), c1, (float)(p[1] - (double)c1));
-    tab[kTab + k] = make_float4((float)p[2], (float)p[3], (float)p[4], 0.f);
+    double scale = 1.0;
+    for (int j = 0; j < N; ++j, scale /= h) p[j] *= scale;
+}
+__global__ void k_ks_table(double alpha, int e0, double far0, double h_far, float4* tab) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < kNear) {
+        double p[7];
+        const double octave = ldexp(1.0, e0 + k / 64), h = octave / 64.0;
+        ks_poly<7>(alpha, octave + h * (k % 64), h, p);
+        for (int j = 0; j < 7; ++j) ((double*)tab)[j * kNear + k] = p[j];
+    }
+    if (k < kFar) {
+        double p[6];
+        const float lower = (float)(far0 + h_far * k);
+        ks_poly<6>(alpha, (double)lower, h_far, p);
+        float c[6], l[3];
+        for (int j = 0; j < 6; ++j) {
+            c[j] = (float)p[j];
+            if (j < 3) l[j] = (float)(p[j] - (double)c[j]);
+        }
+        float4* far = tab + 7 * kNear / 2;
+        far[k] = make_float4(c[0], l[0], c[1], l[1]);
+        far[kFar + k] = make_float4(c[2], l[2], c[3], c[4]);
+        ((float2*)(far + 2 * kFar))[k] = make_float2(c[5], lower);
+    }
 }
 
-// The particle-independent floats of the pair arithmetic.
+// The particle-independent numbers of the short-range pairs.  Comparisons of positive doubles are made on their
+// bits, beside the FP64 pipe.
 struct PPConst {
-    float Lh, Lm, Ll;            // the period, split like a coordinate
-    float rch, rcl, dch, dcl;    // r_cut^2 and d_c^2
-    float kh, kl;                // table intervals per unit r^2
-    float L, invL, rc2;          // of the screen: the period and (r_cut + 1e-3)^2 + 1e-3
-    float wxy, R;                // cell width across, pipe radius
+    double L, invL, alpha, dc2;
+    long long half_bits, cut_bits;               // L/2, r_cut^2
+    long long low_bits, end_bits;                // the near table's range, from d_c^2 at the least
+    int base;                                    // its first edge's upper word without the last 14 bits
+    float Lh, Lm, Ll;                            // the period, split like a coordinate
+    float rch, rcl;                              // r_cut^2
+    float far0, kf, far_min;                     // the far table's start, intervals per unit r^2; from d_c^2 at the least
+    float Lf, invLf, rc2, rn2;                   // of the screen: the period, the widened r_cut^2, and r_n^2
+    float wxy, R;                                // cell width across, pipe radius
 };
 
-// One short-range pair: q_j (d / max(r, d_c)^3 - K_L(d)) when r < r_cut, in float-float (~145 FP32
-// operations); added to the float-float sums s, c.
-__device__ __forceinline__ void pp_pair(const PPConst& K, const float4* T, const float4 ih, const float4 im,
-                                        const float4 il, const float4 jh, const float4 jm, const float4 jl, float s[3],
-                                        float c[3]) {
+// 1 / max(r, d_c)^3 - K_L factor at the close pairs: K_L by c alpha^3 sum_m (-1)^m 2 u^m / (m! (2m + 3)), u = (alpha r)^2, to
+// m = 17 below u = 1 (where the closed form cancels; the next term is 2^-57), by the closed form above.
+__device__ __forceinline__ double pp_close(const PPConst& K, double r2) {
+    const double c = 1.1283791670955126, u = K.alpha * K.alpha * r2, a3 = K.alpha * K.alpha * K.alpha;
+    double kl;
+    if (u < 1.0) {
+        constexpr double inv_fact[18] = {
+            1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720, 1.0 / 5040, 1.0 / 40320, 1.0 / 362880,
+            1.0 / 3628800, 1.0 / 39916800, 1.0 / 479001600, 1.0 / 6227020800.0, 1.0 / 87178291200.0,
+            1.0 / 1307674368000.0, 1.0 / 20922789888000.0, 1.0 / 355687428096000.0};
+        double s = 0.0;
+#pragma unroll
+        for (int m = 17; m >= 0; --m) s = __fma_rn(s, -u, 2.0 * inv_fact[m] / (2 * m + 3));
+        kl = c * a3 * s;
+    } else {
+        const double x = sqrt(u);
+        kl = a3 * (erf(x) / (u * x) - c * exp(-u) / u);
+    }
+    return inv_cube64(fmax(r2, K.dc2)) - kl;
+}
+
+// One short-range pair: q_j (d / max(r, d_c)^3 - K_L(d)) when r < r_cut, in FP64 (17 operations).
+__device__ __forceinline__ void pp_pair(const PPConst& K, const double* T, const double4_32a& pi, const double4_32a& pj,
+                                        double& sx, double& sy, double& sz) {
+    const double dx = pi.x - pj.x, dy = pi.y - pj.y;
+    double dz = pi.z - pj.z;
+    if ((__double_as_longlong(dz) & 0x7fffffffffffffffll) > K.half_bits)      // few pairs: nearest image
+        dz = __fma_rn(-K.L, rint(dz * K.invL), dz);
+    const double r2 = __fma_rn(dx, dx, __fma_rn(dy, dy, dz * dz));
+    const long long bits = __double_as_longlong(r2);
+    if ((unsigned long long)bits >= (unsigned long long)K.cut_bits) return;      // NaN too, of either sign
+    double f;
+    if (bits >= K.low_bits && bits < K.end_bits) {
+        const int hi = (int)(bits >> 32);
+        const double* p = T + ((hi >> 14) - K.base);
+        const double t = r2 - __hiloint2double(hi & ~0x3fff, 0);
+        f = p[6 * kNear];
+#pragma unroll
+        for (int j = 5; j >= 0; --j) f = __fma_rn(f, t, p[j * kNear]);
+    } else f = pp_close(K, r2);
+    f *= pj.w;
+    sx = __fma_rn(f, dx, sx);
+    sy = __fma_rn(f, dy, sy);
+    sz = __fma_rn(f, dz, sz);
+}
+
+// The same for r >= r_n in float-float (~110 FP32 operations), added to the float-float sums s, c; false (and
+// nothing added) when the pair is not one for it.
+__device__ __forceinline__ bool pp_far(const PPConst& K, const float4* T, const float4 ih, const float4 im,
+                                       const float4 il, const float4 jh, const float4 jm, const float4 jl, float s[3],
+                                       float c[3]) {
     float D[3], E[3], R, r;
     split_diff(ih.x, im.x, il.x, jh.x, jm.x, jl.x, D[0], E[0]);
     split_diff(ih.y, im.y, il.y, jh.y, jm.y, jl.y, D[1], E[1]);
-    const float dz = __fsub_rn(ih.z, jh.z), n = rintf(dz * K.invL);        // nearest image, n in {-1, 0, 1}
+    const float dz = __fsub_rn(ih.z, jh.z), n = rintf(dz * K.invLf);       // nearest image, n in {-1, 0, 1}
     two_sum(__fmaf_rn(-n, K.Lh, dz), __fmaf_rn(-n, K.Lm, __fsub_rn(im.z, jm.z)), D[2], E[2]);
     E[2] = __fadd_rn(E[2], __fmaf_rn(-n, K.Ll, __fsub_rn(il.z, jl.z)));
     split_norm2(D, E, R, r);
-    if (!(__fadd_rn(__fsub_rn(R, K.rch), __fsub_rn(r, K.rcl)) < 0.f)) return;
-    // K_L factor: interval and position inside it, then the quartic with its last steps in float-float
-    float X, Xe;
-    split_mul(R, r, K.kh, K.kl, X, Xe);
-    int k = (int)X;
-    k = k < kTab ? k : kTab - 1;
-    const float th = __fsub_rn(X, (float)k);
-    const float4 t0 = T[k], t1 = T[kTab + k];
-    const float v = __fmaf_rn(th, __fmaf_rn(th, __fmaf_rn(th, t1.z, t1.y), t1.x), t0.w);    // c1 lo and the rest
-    const float m = __fmul_rn(th, t0.z);
-    float kl, ke;
-    fast_two_sum(t0.x, m, kl, ke);
-    ke = __fadd_rn(__fadd_rn(ke, t0.y),
-                   __fmaf_rn(th, v, __fmaf_rn(Xe, t0.z, __fmaf_rn(th, t0.z, -m))));
-    const bool clamp = __fadd_rn(__fsub_rn(R, K.dch), __fsub_rn(r, K.dcl)) < 0.f;
-    float w, we, g, ge;
-    split_inv_cube(clamp ? K.dch : R, clamp ? K.dcl : r, w, we);
-    two_sum(w, -kl, g, ge);
-    ge = __fadd_rn(ge, __fsub_rn(we, ke));
+    if (!(R >= K.far_min) || isnan(__fadd_rn(ih.w, jh.w))) return false;
+    if (!(__fadd_rn(__fsub_rn(R, K.rch), __fsub_rn(r, K.rcl)) < 0.f)) return true;
+    int k = (int)__fmul_rn(__fsub_rn(R, K.far0), K.kf);
+    k = k < kFar ? k : kFar - 1;
+    const float4 t0 = T[k], t1 = T[kFar + k];
+    const float2 t2 = ((const float2*)(T + 2 * kFar))[k];
+    float th, te, kl, ke;
+    fast_two_sum(__fsub_rn(R, t2.y), r, th, te);
+    fast_two_sum(t1.x, __fmul_rn(th, __fmaf_rn(th, __fmaf_rn(th, t2.x, t1.w), t1.z)), kl, ke);
+    ke = __fadd_rn(ke, t1.y);
+    auto horner = [&](float ch, float cl) {        // (kl, ke) <- (ch, cl) + (th, te) (kl, ke), |ch| above the rest
+        const float m = __fmul_rn(th, kl);
+        const float me = __fmaf_rn(th, ke, __fmaf_rn(te, kl, __fmaf_rn(th, kl, -m)));
+        float e;
+        fast_two_sum(ch, m, kl, e);
+        ke = __fadd_rn(e, __fadd_rn(cl, me));
+    };
+    horner(t0.z, t0.w);
+    horner(t0.x, t0.y);
     float f, fe;
-    split_mul(g, ge, jh.w, jm.w, f, fe);
+    split_mul(kl, ke, jh.w, jm.w, f, fe);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         float p, e, u;
@@ -413,39 +479,43 @@ __device__ __forceinline__ void pp_pair(const PPConst& K, const float4* T, const
         two_sum(s[a], p, s[a], u);
         c[a] = __fadd_rn(c[a], __fadd_rn(u, e));
     }
+    return true;
 }
 
 // Short-range part: q_j (d / max(r, d_c)^3 - K_L(d)) over j != i closer than r_cut, added to sums.
 // One warp per particle i (cell order).  Cells are r_cut/2 wide across and r_cut/4 along the pipe
 // and a column's cells follow one another, so the candidates are one run of particles (two across the
 // period) in each of at most 25 columns; lane c looks column c's runs up, all at once.  The lanes then
-// screen 32 candidates at a time on the hi parts (r^2 < (r_cut + 1e-3)^2 + 1e-3), the next 32 in
-// flight, the survivors go to a per-warp queue in shared memory, and every 32 queued pairs are
-// evaluated with all lanes busy; the lanes' partial sums (about a dozen pairs each) are reduced in a
-// fixed order.
-// Bound by instruction issue (screening ~1,500 candidates and ~410 pairs of ~190 instructions per
-// particle).  One million particles, mesh 256^3: 5.4 ms (5.9 ms with PPConst worked out per thread: its FP64 was
-// repeated where registers ran short, pipe 53 % busy, now 8 %; 6.8 ms at 3 CTAs and 80 registers, 7.5 ms with the cell
-// index recomputed in FP64 by every lane); 42.4 ms in FP64 with the Hermite table in
-// global memory (FP64 pipe 87 % busy), 13.6 ms in float-float over the 27 cells of width r_cut.
-constexpr int kPPWarps = 8;
-__global__ void __launch_bounds__(32 * kPPWarps, 4) k_p3m_pp(const P3MGeom G, const PPConst K, const P3MPart S,
+// screen 32 candidates at a time on the hi parts (r_cut widened by the coordinates' rounding), the next 32 in flight.
+// The survivors go to one of two per-warp queues in shared memory, inner or outer, and every 32 queued pairs are
+// evaluated with all lanes busy; the lanes' partial sums are reduced in a fixed order.
+// Bound by instruction issue and the FP64 pipe together (~1,500 candidates, ~50 inner pairs of 17 FP64 operations and
+// ~360 outer ones of ~130 instructions per particle).  One million particles, mesh 256^3: 8.0 ms; all pairs in FP64 by
+// the table 16.5 ms; 42.4 ms in FP64 over the 27 cells of width r_cut with K_L by a cubic table.  Error of the sums
+// against extended precision, 2-norm at 100,000 particles: 1.0e-16 (like charges) and 2.2e-16 (both signs), 4.5e-16
+// and 7.1e-16 with that table; all pairs in float-float with K_L in quartics left 8e-12 and 7e-11, that K_L to 2^-50
+// still 1.6e-15 and 7.6e-15.
+constexpr int kPPWarps = 8, kPPShared = 16 * kTabWords + kPPWarps * 128 * 4;
+__global__ void __launch_bounds__(32 * kPPWarps, 3) k_p3m_pp(const P3MGeom G, const PPConst K, const P3MPart S,
                                                           const int* start, int64_t ncells, const int* list,
+                                                          const double4_32a* __restrict__ s64,
                                                           const float4* __restrict__ sorted, int64_t stride,
                                                           double* sums) {
-    __shared__ float4 T[2 * kTab];
-    __shared__ int queue[kPPWarps][64];
-    for (int k = threadIdx.x; k < 2 * kTab; k += blockDim.x) T[k] = G.lf_tab[k];
+    extern __shared__ float4 pp_smem[];                    // the tables, then the queues
+    for (int k = threadIdx.x; k < kTabWords; k += blockDim.x) pp_smem[k] = G.ks_tab[k];
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int* qw = queue[w];
+    const double* Tn = (const double*)pp_smem;
+    const float4* Tf = pp_smem + 7 * kNear / 2;
+    int* qw = (int*)(pp_smem + kTabWords) + w * 128;       // inner, outer: 64 entries each
     const int n_live = start[ncells];
-    const float rc2f = K.rc2, Lf = K.L, invLf = K.invL;
-    const unsigned lt = (1u << lane) - 1u;
+    const float rc2f = K.rc2, rn2f = K.rn2, Lf = K.Lf, invLf = K.invLf;
     const float4 *sh = sorted, *sm = sorted + stride, *sl = sorted + 2 * stride;
+    const unsigned lt = (1u << lane) - 1u;
     const float wxy = K.wxy, Rf = K.R;
     for (int t = blockIdx.x * kPPWarps + w; t < n_live; t += gridDim.x * kPPWarps) {
         const float4 ih = sh[t], im = sm[t], il = sl[t];
+        const double4_32a pi = s64[t];
         // column lane of the 5 x 5 around i: its runs [b0, e0) and, across the period, [b1, e1)
         int b0 = 0, e0 = 0, b1 = 0, e1 = 0;
         {
@@ -471,9 +541,11 @@ __global__ void __launch_bounds__(32 * kPPWarps, 4) k_p3m_pp(const P3MGeom G, co
                 }
             }
         }
+        double sx = 0.0, sy = 0.0, sz = 0.0;
         float s[3] = {0.f, 0.f, 0.f}, c[3] = {0.f, 0.f, 0.f};
-        int qn = 0;
-        auto pair = [&](int p) { pp_pair(K, T, ih, im, il, sh[p], sm[p], sl[p], s, c); };
+        int qn[2] = {0, 0};
+        auto near = [&](int p) { pp_pair(K, Tn, pi, s64[p], sx, sy, sz); };
+        auto far = [&](int p) { if (!pp_far(K, Tf, ih, im, il, sh[p], sm[p], sl[p], s, c)) near(p); };
         const float4 none = make_float4(1e15f, 0.f, 0.f, 0.f);
 #pragma unroll 1
         for (int half = 0; half < 2; ++half) {
@@ -501,35 +573,41 @@ __global__ void __launch_bounds__(32 * kPPWarps, 4) k_p3m_pp(const P3MGeom G, co
                 const float ex = ih.x - fc.x, ey = ih.y - fc.y;
                 float ez = ih.z - fc.z;
                 ez -= Lf * rintf(ez * invLf);
-                const bool pass = ex * ex + ey * ey + ez * ez < rc2f;
-                const unsigned m = __ballot_sync(0xffffffffu, pass);
-                if (pass) qw[qn + __popc(m & lt)] = pc;
-                qn += __popc(m);
+                const float d2 = ex * ex + ey * ey + ez * ez;
+#pragma unroll
+                for (int o = 0; o < 2; ++o) {
+                    const bool pass = o ? d2 >= rn2f && d2 < rc2f : d2 < rn2f;
+                    const unsigned m = __ballot_sync(0xffffffffu, pass);
+                    if (pass) qw[64 * o + qn[o] + __popc(m & lt)] = pc;
+                    qn[o] += __popc(m);
+                }
                 __syncwarp();
-                if (qn >= 32) {
-                    pair(qw[lane]);
-                    __syncwarp();
-                    if (lane < qn - 32) qw[lane] = qw[32 + lane];
-                    qn -= 32;
-                    __syncwarp();
+#pragma unroll
+                for (int o = 0; o < 2; ++o) {
+                    if (qn[o] >= 32) {
+                        if (o) far(qw[64 + lane]);
+                        else near(qw[lane]);
+                        __syncwarp();
+                        if (lane < qn[o] - 32) qw[64 * o + lane] = qw[64 * o + 32 + lane];
+                        qn[o] -= 32;
+                        __syncwarp();
+                    }
                 }
             }
         }
-        if (lane < qn) pair(qw[lane]);
+        if (lane < qn[0]) near(qw[lane]);
+        if (lane < qn[1]) far(qw[64 + lane]);
         __syncwarp();
-        for (int d = 16; d > 0; d >>= 1) {
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const float os = __shfl_xor_sync(0xffffffffu, s[a], d), oc = __shfl_xor_sync(0xffffffffu, c[a], d);
-                float u;
-                two_sum(s[a], os, s[a], u);
-                c[a] = __fadd_rn(__fadd_rn(c[a], oc), u);
-            }
-        }
-        if (lane < 3) {      // lane a adds component a
-            const float sa = lane == 0 ? s[0] : lane == 1 ? s[1] : s[2], ca = lane == 0 ? c[0] : lane == 1 ? c[1] : c[2];
-            sums[3 * (S.o + list[t]) + lane] += (double)sa + (double)ca;
-        }
+        sx += (double)s[0] + (double)c[0];
+        sy += (double)s[1] + (double)c[1];
+        sz += (double)s[2] + (double)c[2];
+        // half of the components each time the lanes halve (6 adds): x ends in lane 0, y in lane 8, z in lane 16
+        const bool up = lane & 16, up2 = lane & 8;
+        const double a = (up ? sz : sx) + __shfl_xor_sync(0xffffffffu, up ? sx : sz, 16);
+        const double b = (up ? 0.0 : sy) + __shfl_xor_sync(0xffffffffu, up ? sy : 0.0, 16);
+        double v = (up2 ? b : a) + __shfl_xor_sync(0xffffffffu, up2 ? a : b, 8);
+        for (int d = 4; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+        if ((lane & 7) == 0 && lane < 24) sums[3 * (S.o + list[t]) + lane / 8] += v;
     }
 }
 
@@ -542,22 +620,50 @@ P3MGeom geom_of(const pdq_p3m* P, double contact) {
     G.R = P->R; G.L = P->L; G.h = P->h; G.hz = P->hz; G.x0 = P->x0; G.alpha = P->alpha; G.rc = P->rc;
     G.contact = contact; G.Mx = P->Mx; G.Nx = P->Nx; G.Nz = P->Nz; G.n_img = P->n_img;
     G.ncx = P->ncx; G.ncz = P->ncz;
-    G.lf_tab = P->lf_tab;
+    G.ks_tab = P->ks_tab;
     G.grid = split_grid(std::max(P->R, P->L));
     return G;
 }
 
+long long bits_of(double v) {
+    long long b;
+    memcpy(&b, &v, sizeof(b));
+    return b;
+}
+
+// The outer pairs start at r_n: half of r_cut where K_S is small there (alpha r_cut as usual) and its floats keep
+// their range, else none are.
+double near_end(double alpha, double rc) { return alpha * rc >= 3.0 && rc > 1e-3 && rc < 1e4 ? 0.5 * rc : rc; }
+// The near table's first octave is 2^e0, the far table's first edge far0.
+int near_start(double alpha, double rc) {
+    const double rn = near_end(alpha, rc);
+    int e;
+    const double m = frexp(rn * rn, &e);            // r_n^2 = m 2^e, 1/2 <= m < 1
+    return (m > 0.5 ? e : e - 1) - kOct;
+}
+double far_start(double alpha, double rc) {
+    const double rn = near_end(alpha, rc);
+    return (double)(float)(0.98 * rn * rn);
+}
+
 PPConst pp_const_of(const P3MGeom& G) {
-    // (the floor keeps d_c^-3 inside FP32's range; it is 1e-10 wall units)
-    const double rc2 = G.rc * G.rc, dc2 = std::max(G.contact * G.contact, 1e-20), kk = kTab / rc2;
-    const float rcf = (float)G.rc + 1e-3f;
     PPConst K;
+    const int e0 = near_start(G.alpha, G.rc);
+    const double first = ldexp(1.0, e0), rc2 = G.rc * G.rc, rn = near_end(G.alpha, G.rc), far0 = far_start(G.alpha, G.rc);
+    K.L = G.L; K.invL = 1.0 / G.L; K.alpha = G.alpha;
+    K.dc2 = std::max(G.contact * G.contact, 1e-20);       // coincident particles stay finite: 1e-10 wall units
+    K.half_bits = bits_of(0.5 * G.L);
+    K.cut_bits = bits_of(rc2);
+    K.low_bits = bits_of(std::max(K.dc2, first));
+    K.end_bits = bits_of(ldexp(1.0, e0 + kOct));
+    K.base = (int)(bits_of(first) >> 46);
     split3(G.grid, G.L, K.Lh, K.Lm, K.Ll);
     K.rch = (float)rc2; K.rcl = (float)(rc2 - (double)K.rch);
-    K.dch = (float)dc2; K.dcl = (float)(dc2 - (double)K.dch);
-    K.kh = (float)kk; K.kl = (float)(kk - (double)K.kh);
-    K.L = (float)G.L; K.invL = 1.0f / K.L;
+    K.far0 = (float)far0; K.far_min = (float)std::max(far0, K.dc2); K.kf = (float)(kFar / (rc2 - far0));
+    K.Lf = (float)G.L; K.invLf = 1.0f / K.Lf;
+    const float rcf = (float)G.rc + 1e-3f;
     K.rc2 = rcf * rcf + 1e-3f;
+    K.rn2 = rn < G.rc ? (float)(rn * rn) : K.rc2;          // at most rc2: the screen's filler must fail both
     K.wxy = (float)(2.0 * G.R / G.ncx); K.R = (float)G.R;
     return K;
 }
@@ -569,7 +675,7 @@ void free_plan(pdq_p3m* P) {
     if (P->have_inv) cufftDestroy(P->inv);
     cudaFree(P->Gh); cudaFree(P->Q); cudaFree(P->Qh); cudaFree(P->Ah); cudaFree(P->A);
     cudaFree(P->cell_count); cudaFree(P->cell_start); cudaFree(P->cell_fill); cudaFree(P->cell_list);
-    cudaFree(P->sorted); cudaFree(P->lf_tab);
+    cudaFree(P->sorted64); cudaFree(P->sorted); cudaFree(P->ks_tab);
     cudaFree(P->sums);
     delete P;
 }
@@ -623,8 +729,9 @@ extern "C" int pdq_p3m_create(const pdq_field* field, const pdq_p3m_desc* d, int
     alloc((void**)&P->cell_start, (P->ncells + 1) * sizeof(int));
     alloc((void**)&P->cell_fill, P->ncells * sizeof(int));
     alloc((void**)&P->cell_list, P->max_n * sizeof(int));
+    alloc((void**)&P->sorted64, P->max_n * sizeof(double4_32a));
     alloc((void**)&P->sorted, 3 * P->max_n * sizeof(float4));
-    alloc((void**)&P->lf_tab, 2 * kTab * sizeof(float4));
+    alloc((void**)&P->ks_tab, kTabWords * sizeof(float4));
     alloc((void**)&Gr, 3 * P->nreal * sizeof(double));
     // The charges reach only Mx of the Nx planes across (the rest is the zero padding of the open
     // convolution) and the field is read on the same Mx: the (y, z) transforms run on those planes alone,
@@ -646,7 +753,9 @@ extern "C" int pdq_p3m_create(const pdq_field* field, const pdq_p3m_desc* d, int
     if (rc == PDQ_OK) {
         const P3MGeom G = geom_of(P, 0.0);
         k_p3m_kernel<<<grid_of(P->nreal, 256), 256, 0, s>>>(G, Gr, Gr + P->nreal, Gr + 2 * P->nreal);
-        k_lf_table<<<grid_of(kTab, 128), 128, 0, s>>>(P->alpha, P->alpha * P->alpha * P->rc * P->rc, P->lf_tab);
+        const double far0 = far_start(P->alpha, P->rc);
+        k_ks_table<<<grid_of(std::max(kNear, kFar), 128), 128, 0, s>>>(P->alpha, near_start(P->alpha, P->rc), far0,
+                                                                       (P->rc * P->rc - far0) / kFar, P->ks_tab);
         for (int c = 0; c < 3 && rc == PDQ_OK; ++c)
             rc = cufft_status(cufftExecD2Z(whole, Gr + c * P->nreal, P->Gh + c * P->ncplx));
         if (rc == PDQ_OK) k_p3m_deconv<<<grid_of(P->ncplx, 256), 256, 0, s>>>(G, P->Gh, (int64_t)P->ncplx);
@@ -696,6 +805,7 @@ extern "C" int pdq_p3m_coulomb(pdq_p3m* P, const pdq_phys* phys, const pdq_state
     PDQ_CUDA(cufftSetStream(P->fwd, s) == CUFFT_SUCCESS ? cudaSuccess : cudaErrorUnknown);
     PDQ_CUDA(cufftSetStream(P->lines, s) == CUFFT_SUCCESS ? cudaSuccess : cudaErrorUnknown);
     PDQ_CUDA(cufftSetStream(P->inv, s) == CUFFT_SUCCESS ? cudaSuccess : cudaErrorUnknown);
+    PDQ_CUDA(cudaFuncSetAttribute(k_p3m_pp, cudaFuncAttributeMaxDynamicSharedMemorySize, kPPShared));
     const int h = st->cur;
     for (int k = 0; k < st->n_samples; ++k) {
         if (cnt[k] == 0) continue;
@@ -727,9 +837,9 @@ extern "C" int pdq_p3m_coulomb(pdq_p3m* P, const pdq_phys* phys, const pdq_state
         k_cell_scan<<<1, 1024, 0, s>>>(P->cell_count, P->ncells, P->cell_start);
         k_cell_fill<<<gp, 256, 0, s>>>(G, S, P->cell_start, P->cell_fill, P->cell_list);
         k_cell_sort<<<grid_of(P->ncells, 128), 128, 0, s>>>(P->cell_start, P->ncells, P->cell_list);
-        k_cell_gather<<<gp, 256, 0, s>>>(G, S, P->cell_start, P->ncells, P->cell_list, P->sorted, P->max_n);
-        k_p3m_pp<<<(unsigned)std::min<int64_t>(grid_of(S.n, kPPWarps), 16 * 152), 32 * kPPWarps, 0, s>>>(
-            G, K, S, P->cell_start, P->ncells, P->cell_list, P->sorted, P->max_n, sums);
+        k_cell_gather<<<gp, 256, 0, s>>>(G, S, P->cell_start, P->ncells, P->cell_list, P->sorted64, P->sorted, P->max_n);
+        k_p3m_pp<<<(unsigned)std::min<int64_t>(grid_of(S.n, kPPWarps), 16 * 152), 32 * kPPWarps, kPPShared, s>>>(
+            G, K, S, P->cell_start, P->ncells, P->cell_list, P->sorted64, P->sorted, P->max_n, sums);
     }
     PDQ_CUDA(cudaGetLastError());
     return PDQ_OK;

@@ -126,6 +126,31 @@ def test_p3m_sums_mixed_state(pdq, setup):
     assert np.max(np.abs(got - want)) <= 1e-9 * _rms(want)
 
 
+def _two_particle_errors(pdq, plan, d, Gh, a, b):
+    """Error of the GPU's sums relative to the larger one, per sample of two particles a[k], b[k]."""
+    n = len(a)
+    X = np.stack([a, b], 1).reshape(-1, 3)
+    x, y, z = X[:, 0].copy(), X[:, 1].copy(), np.mod(X[:, 2], d.L)
+    q = np.tile([0.7, 0.4], n)
+    st = _state(pdq, 0, [2] * n, (x, y, z, q, np.zeros((2 * n, 3)), np.full(2 * n, 2, np.int32),
+                                  np.tile([0, 1], n).astype(np.int32)))
+    got = plan.coulomb(pdq.phys_default(), st).cpu().numpy()
+    want = _ref_sums(d, Gh, [2] * n, x, y, z, q)
+    return np.abs(got - want).reshape(n, 6).max(1) / np.abs(want).reshape(n, 6).max(1)
+
+
+def test_p3m_short_range_pairs_in_double(pdq, setup):
+    # pairs alone in a sample from alpha r = 0.18 (below it the reference's own closed form cancels) to near r_cut.
+    # Bar: a pair and its table 2^-52, the transforms over 2^18 nodes 18 2^-53 of a mesh field that is up to ~100
+    # times the pair's force near r_cut (self-fields that cancel): 4e-13
+    f, of, grid, plan, d, Gh = setup
+    rng = np.random.default_rng(5)
+    r = np.geomspace(0.18 / plan.alpha, 0.95 * plan.r_cut, 24)
+    u = rng.standard_normal((24, 3))
+    a = np.stack([rng.uniform(-60, 60, 24), rng.uniform(-60, 60, 24), rng.uniform(0, 720, 24)], 1)
+    assert np.max(_two_particle_errors(pdq, plan, d, Gh, a, a + u * (r / np.linalg.norm(u, axis=1))[:, None])) <= 4e-13
+
+
 @pytest.mark.parametrize("seam", [False, True])
 @pytest.mark.parametrize("at", ["contact", "table", "cut"])
 def test_p3m_short_range_pairs_at_their_edges(pdq, setup, at, seam):
