@@ -661,7 +661,9 @@ PPConst pp_const_of(const P3MGeom& G) {
     K.rch = (float)rc2; K.rcl = (float)(rc2 - (double)K.rch);
     K.far0 = (float)far0; K.far_min = (float)std::max(far0, K.dc2); K.kf = (float)(kFar / (rc2 - far0));
     K.Lf = (float)G.L; K.invLf = 1.0f / K.Lf;
-    const float rcf = (float)G.rc + 1e-3f;
+    // a hi part is off by half of the grid's 2^-23 max(R, L) (up to twice that), their differences by as much again in
+    // FP32: the distances of the screen are off by less than (R + L) 2^-21
+    const float rcf = (float)(G.rc + 1e-3 + (G.R + G.L) * 4.76837158203125e-07);
     K.rc2 = rcf * rcf + 1e-3f;
     K.rn2 = rn < G.rc ? (float)(rn * rn) : K.rc2;          // at most rc2: the screen's filler must fail both
     K.wxy = (float)(2.0 * G.R / G.ncx); K.R = (float)G.R;

@@ -151,6 +151,24 @@ def test_p3m_short_range_pairs_in_double(pdq, setup):
     assert np.max(_two_particle_errors(pdq, plan, d, Gh, a, a + u * (r / np.linalg.norm(u, axis=1))[:, None])) <= 4e-13
 
 
+def test_p3m_pairs_just_inside_the_cut_of_a_long_pipe(pdq):
+    # a pipe whose coordinates lie on a grid of g = 8192 2^-23 in FP32: pairs 2e-4 inside r_cut whose coordinates all
+    # round away from each other, by 0.98 g each, still count.  A lost pair changes the sum by K_S(r_cut) r_cut^2 =
+    # 0.07 of the pair's force at alpha r_cut = 1.9; bar as above
+    L, M, Nz, g = 8000.0, 16, 512, 8192.0 * 2.0 ** -23
+    desc = pdq.field_desc(n_r=17, n_th=8, n_z=16)
+    desc.l_plus = L
+    f = pdq.Field(desc, 0)
+    alpha = AH / (2 * 180.0 / M)
+    side = (round(1.9 / alpha / np.sqrt(3) / g) + 0.02) * g
+    rc = np.sqrt(3) * side + 2e-4
+    plan = pdq.P3M(f, M=M, Nz=Nz, alpha=alpha, r_cut=rc, n_img=20, max_particles=2)
+    d = ref.Desc(180.0, L, M, Nz, alpha, rc, n_img=20)
+    m = np.random.default_rng(6).uniform([0, 0, 100], [60, 60, 7900], (16, 3))
+    a = (np.round(m / g) + 0.51) * g
+    assert np.max(_two_particle_errors(pdq, plan, d, ref.influence(d), a, a - side)) <= 1e-9
+
+
 @pytest.mark.parametrize("seam", [False, True])
 @pytest.mark.parametrize("at", ["contact", "table", "cut"])
 def test_p3m_short_range_pairs_at_their_edges(pdq, setup, at, seam):
