@@ -2331,7 +2331,7 @@ int step_impl(const pdq_field* field, const pdq_phys* phys, pdq_state* st, const
         }
     }
     bool coarse = false;
-    if (!ext && st->precision == PDQ_FP64 && workspace_bytes < need) {      // likewise for fewer chunks
+    if (st->precision == PDQ_FP64 && workspace_bytes < need) {      // likewise for fewer chunks (given sums use none)
         coarse = true;
         workspace_layout(st, NT * U, &items_bytes, &need, &cnt_off, &part_off, contact, &acc_off, newton, coarse,
                          &split_off);

@@ -231,3 +231,25 @@ def test_p3m_step_matches_oracle(pdq, setup, block):
     assert np.max(np.abs(gx[live] - rx[live]) / (1 + np.abs(rx[live]))) < 1e-11
     assert np.max(np.abs(gv[live, :3] - rv[live]) / (1 + np.abs(rv[live]))) < 1e-10
     assert np.array_equal(tally.n_alive.cpu().numpy(), tallies[1])
+
+
+def test_p3m_step_takes_a_workspace_without_partial_sums(pdq, setup):
+    # 2,000 FP64 particles at 32 threads: given sums need no partial sums of the tile pairs, so a workspace with the
+    # 17 chunks that a one-sided pair sum of this size is cut into (items, order, tags, counters, sums) is enough
+    f, of, grid, plan, d, Gh = setup
+    counts = [1200, 800]
+    arr = _cloud(counts, 8)
+    prm = pdq.params_tensor(np.array([[0.05, 0.5, 0.5], [0.1, 0.2, 0.3]]))
+    cfg = pdq.step_cfg(0.1, block=32, window_start=0)
+
+    def a256(v):
+        return (v + 255) // 256 * 256
+    tiles, chunks = 2000 // 32 + 2 + 1, 17
+    small = a256(8 * tiles * chunks) + a256(4 * 2) + a256(8 * 2000) + a256(4 * tiles) + a256(24 * chunks * 2000)
+    out = []
+    for ws in (None, torch.empty(small, dtype=torch.uint8, device="cuda")):
+        st = _state(pdq, 0, counts, arr)
+        ws = pdq.workspace(st, cfg) if ws is None else ws
+        pdq.step_particles_p3m(f, pdq.phys_default(), st, prm, cfg, 1, pdq.Tally(2, 3), plan, ws)
+        out.append(st.current()[0].clone())
+    assert torch.allclose(out[0], out[1], rtol=1e-12, atol=1e-12)
