@@ -140,12 +140,24 @@ __device__ __forceinline__ float rsqrt_ftz(float x) {
 }
 __device__ __forceinline__ double rsqrt_ftz(double x) { return rsqrt(x); }
 
-// r2^(-3/2) in FP64 for a normal r2 > 0: the hardware's FP64 estimate y of r2^(-1/2) (~2^-20) and the
-// binomial series of (1 - d)^(-3/2) in d = 1 - r2 y^2, to d^3: 7 FP64 operations, against ~10 for the
-// library's reciprocal square root (with its branch for special values) and the two products.
-__device__ __forceinline__ double inv_cube64(double r2) {
+// The hardware's estimates of x^(-1/2) and 1/x in FP64 for normal x (PTX rsqrt.approx.ftz.f64 and
+// rcp.approx.ftz.f64 work on the upper 20 bits of the mantissa): relative error below 2^-19 (2^-20.0 measured).
+__device__ __forceinline__ double rsqrt_seed(double x) {
     double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return y;
+}
+__device__ __forceinline__ double rcp_seed(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    return r;
+}
+
+// r2^(-3/2) in FP64 for a normal, finite r2 > 0: y = rsqrt_seed(r2) and the binomial series of
+// (1 - d)^(-3/2) in d = 1 - r2 y^2 (below 2^-18), to d^3 (the next term is 2.5 d^4 < 2^-70): 7 FP64 operations,
+// against ~10 for the library's reciprocal square root (with its branch for special values) and the two products.
+__device__ __forceinline__ double inv_cube64(double r2) {
+    const double y = rsqrt_seed(r2);
     const double t = y * y;
     const double d = __fma_rn(-r2, t, 1.0);
     const double c = d * __fma_rn(d, __fma_rn(d, 2.1875, 1.875), 1.5);
