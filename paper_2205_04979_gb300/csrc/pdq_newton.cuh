@@ -61,8 +61,9 @@ __device__ __forceinline__ ZClass zclass(float alo, float ahi, float blo, float 
 }
 
 // How a Newton-pair launch over S samples of `capacity` particles in all is cut, for CTAs of NT threads
-// of which `slots` run at once: U particles per thread and parts per tile.  A tile of a large batch is
-// taken whole with u_max (12) per thread.  When the heaviest item (a sample's first tile, ~NT U N pairs)
+// of which `slots` run at once (counted at u_max: narrower tiles run 4 or 5 CTAs of 128 threads where 12 per thread
+// run 3, but the items per slot were measured with this count): U particles per thread and parts per tile.
+// A tile of a large batch is taken whole with u_max (12) per thread.  When the heaviest item (a sample's first tile, ~NT U N pairs)
 // is not small against the work per slot, S N^2 / 2 / slots, the launch would end on a few CTAs or leave
 // SMs idle: the tile then narrows until its diagonal block, (NT U)^2 / 2 pairs on one CTA, is at most
 // a slot's share, and its later particles are cut into parts so that each slot gets kNewtonItems of the
@@ -104,7 +105,7 @@ inline NewtonCut newton_cut(int64_t capacity, int64_t S, int NT, int64_t slots, 
 //     j-side sums of a tile are added in shared memory and leave with one float4 atomic per j.
 // The earlier particles of the sample reach this tile as the j side of earlier tiles.
 // With CUT the tile's work is cut over `parts` > 1 CTAs: part 0 does the diagonal block, part
-// p >= 1 the p-th of parts - 1 equal runs of j-tiles of the later particles (newton_parts says when).
+// p >= 1 the p-th of parts - 1 equal runs of j-tiles of the later particles (newton_cut says when).
 // load(g) gives particle g as (x, y, z, q).  Padding particles sit far off the axis
 // (x = +-1e15) with zero charge, so they add nothing.  All threads of the CTA take part; the
 // shared arrays are the calling kernel's (one set per kernel instantiation).

@@ -2022,7 +2022,8 @@ static int launch_newton_u(const StepArgs& A, cudaStream_t s) {
     if (A.K.forces & PDQ_F_COULOMB) {    // the sums enter the update only with the Coulomb force on
         const dim3 grid((unsigned)std::max<int64_t>(1, A.max_items), (unsigned)A.newton_parts);
         if (A.newton_parts > 1) k_pairs_sym<NT, U, true><<<grid, NT, 0, s>>>(A);
-        else k_pairs_sym<NT, U, false><<<grid, NT, 0, s>>>(A);
+        else if constexpr (U == (CONTACT ? 8 : 12)) k_pairs_sym<NT, U, false><<<grid, NT, 0, s>>>(A);   // only wide tiles are whole
+        else return PDQ_ERR_INVALID_ARG;
     }
     return launch_step<PDQ_MIXED, 2 * NT, U / 2, CONTACT ? 6 : 5>(A, s);
 }

@@ -250,3 +250,40 @@ def test_signed_charge_seed_parity(pdq, fields):
     ost, _ = oracle.seed(of, ST3, counts, prm, 11, charge_sigma=0.5, p=op)
     q = st.current()[0][:, 3].cpu().numpy()
     assert np.allclose(q, ost.q, rtol=1e-13, atol=0) and np.any(q < 0) and np.any(q > 0)
+
+
+@pytest.mark.parametrize("block", [64, 128])
+def test_mixed_contact_whole_wide_tiles(pdq, fields, block):
+    # Newton pairs at 8 particles per thread and the contact variant at 4 over twice the threads, as in large batches: a
+    # workspace that only fits the item table of whole wide tiles.  Samples of one tile, one tile +-1 and two tiles + 1.
+    # Bar: the oracle's response to one FP32 unit of z, for each of 2 steps, and as much for the pair sums
+    T = 8 * block
+    counts = [T - 1, T, T + 1, 2 * T + 1] * 8
+    n, S = sum(counts), len(counts)
+    f, of, grid = fields
+    arr = _contact_state(counts, 12, z_range=(2.0, 12.0))
+    fl = oracle.F_ALL | oracle.F_CONTACT
+    prm = np.tile(np.array([[0.05, 0.8, 0.5]]), (S, 1))
+    st, ost = _load(pdq, 1, counts, arr)
+    cfg = pdq.step_cfg(DT, forces=fl, block=block, variant=3)
+
+    def a256(v):
+        return (v + 255) // 256 * 256
+    ws = torch.empty(a256(8 * (n // T + S + 1)) + a256(4 * S) + a256(8 * n) + a256(16 * n), dtype=torch.uint8,
+                     device="cuda")
+    assert ws.numel() < pdq.workspace(st, cfg).numel()
+    pdq.step_particles(f, pdq.phys_default(), st, pdq.params_tensor(prm), cfg, 2, pdq.Tally(S, 3), ws)
+    assert pdq.check_state(st) == 0
+    off = np.r_[0, np.cumsum(counts)]
+    out = []
+    for ulp in (False, True):
+        _, o = _load(pdq, 1, counts, arr)
+        if ulp:
+            way = np.where(np.random.default_rng(0).uniform(size=n) < 0.5, -np.inf, np.inf).astype(np.float32)
+            o.z = np.nextafter(o.z.astype(np.float32), way).astype(np.float64)
+        oracle.run(of, grid, oracle.cfg(DT, forces=fl), ST3, off, prm, o, 2)
+        out.append(o)
+    a, b = out
+    sx = max(np.max(np.abs(getattr(a, k) - getattr(b, k)) / (1 + np.abs(getattr(a, k)))) for k in "xyz")
+    sv = max(np.max(np.abs(getattr(a, k) - getattr(b, k)) / (1 + np.abs(getattr(a, k)))) for k in ("vx", "vy", "vz"))
+    _compare(st, a, off, max(2e-5, 4 * sx), max(2e-3, 4 * sv))

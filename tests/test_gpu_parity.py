@@ -612,3 +612,54 @@ def test_mixed_newton_pairs_graph_replay(pdq, fields):
         _compare_by_id(st, ost, off, 2e-6, 2e-5, max_flip=0.005)
     a, b = (r[1].n_alive.cpu().numpy() for r in runs)
     assert np.abs(a - b).max() <= 2           # a deposition decision may flip on last-bit differences
+
+
+def _wide_workspace(counts, block, ilp):
+    """Step workspace with the item table of tiles of `ilp` particles per thread: items, order, tags, float4 sums."""
+    def a256(v):
+        return (v + 255) // 256 * 256
+    n = int(np.sum(counts))
+    size = a256(8 * (n // (block * ilp) + len(counts) + 1)) + a256(4 * len(counts)) + a256(8 * n) + a256(16 * n)
+    return torch.empty(size, dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("block", [64, 128])
+def test_mixed_newton_pairs_whole_wide_tiles(pdq, fields, block):
+    # a workspace that only fits the item table of whole tiles of 12 particles per thread (smaller than what
+    # pdq_step_workspace_size asks for, taken all the same): samples of one tile, one tile +-1 and two tiles + 1
+    T = 12 * block
+    counts = [T - 1, T, T + 1, 2 * T + 1] * (6 if block == 128 else 12)
+    f, of, grid, _ = fields
+    prm = np.tile(PRM3[:1], (len(counts), 1))
+    phys, st, p, ost, off = _setup(pdq, fields, 1, counts, ST3, prm)
+    cfg = pdq.step_cfg(0.1, block=block, variant=3)
+    ws = _wide_workspace(counts, block, 12)
+    assert ws.numel() < pdq.workspace(st, cfg).numel()
+    tally = pdq.Tally(len(counts), 3)
+    pdq.step_particles(f, phys, st, p, cfg, 3, tally, ws)
+    assert pdq.check_state(st) == 0
+    nd, na = oracle.run(of, grid, oracle.cfg(0.1), ST3, off, prm, ost, 3)
+    assert _compare_by_id(st, ost, off, 2e-6, 2e-5, max_flip=0.005) > 0
+    assert np.array_equal(tally.n_alive.cpu().numpy()[:, 0] > 0, na[:, 0] > 0)
+    with pytest.raises(pdq.PdqError):            # one slot of 256 bytes less is refused
+        pdq.step_particles(f, phys, st, p, cfg, 1, tally, ws[:-256])
+
+
+def test_fp64_newton_pairs_in_a_workspace_of_few_chunks(pdq, fields):
+    # FP64 Newton pairs with the item table of the former, fewer chunks (8 i-tiles each) and no room for the far pairs'
+    # choices: the same sums in another order
+    counts = [3000, 517]
+    f, of, grid, _ = fields
+    phys, st, p, ost, off = _setup(pdq, fields, 0, counts, ST3, PRM3[:2])
+    cfg = pdq.step_cfg(0.1, block=64, variant=3)
+
+    def a256(v):
+        return (v + 255) // 256 * 256
+    n, TI = sum(counts), 128
+    chunks = -(-n // (8 * TI))
+    ws = torch.empty(a256(8 * (n // TI + 3) * chunks) + a256(8) + a256(8 * n) + a256(24 * n), dtype=torch.uint8,
+                     device="cuda")
+    assert ws.numel() < pdq.workspace(st, cfg).numel()
+    pdq.step_particles(f, phys, st, p, cfg, 1, pdq.Tally(2, 3), ws)
+    oracle.run(of, grid, oracle.cfg(0.1), ST3, off, PRM3[:2], ost, 1)
+    assert _compare_by_id(st, ost, off, 1e-12, 1e-12) > 0

@@ -152,3 +152,31 @@ def test_fp64_chunked_items_cover_each_pair_once(n, NT):
     assert n_items > 0
     want = np.ones((n, n), np.int64) - np.eye(n, dtype=np.int64)
     assert np.array_equal(count, want)
+
+
+def newton_part_range(n, nd, NT, part, parts):
+    """Later particles [jb, je) of a part, counted from the tile's base, as newton_tile cuts them (part 0: none)."""
+    per = (-(-(n - nd) // NT) + parts - 2) // (parts - 1) * NT
+    if part == 0:
+        return n, n
+    jb = nd + (part - 1) * per
+    return jb, min(jb + per, n)
+
+
+@pytest.mark.parametrize("NT", [64, 128])
+@pytest.mark.parametrize("U", [4, 8, 12])
+def test_parts_cover_the_later_particles_once(NT, U):
+    # every later particle in one part, parts of whole j-tiles but for the sample's last, over sizes around the tile, one
+    # and two j-tiles more, and as many or more parts than j-tiles (parts without particles are skipped)
+    T = NT * U
+    for n in (1, T - 1, T, T + 1, T + NT - 1, T + NT, T + NT + 1, T + 2 * NT + 1, 2 * T + 1, 5 * T - 7):
+        nd = min(n, T)
+        for parts in (2, 3, 7, 1 + n // NT + 1):
+            seen = np.zeros(n, int)
+            for part in range(parts):
+                jb, je = newton_part_range(n, nd, NT, part, parts)
+                if jb >= je:
+                    continue
+                assert (jb - nd) % NT == 0 and ((je - nd) % NT == 0 or je == n)
+                seen[jb:je] += 1
+            assert np.all(seen[nd:] == 1) and np.all(seen[:nd] == 0)
