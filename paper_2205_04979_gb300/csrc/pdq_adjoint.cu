@@ -874,8 +874,9 @@ __device__ __forceinline__ void vjp_pair_x2_sym(f2 xm, f2 ym, f2 zm, f2 nQm, f2 
 // tile's own block one-sided (the j sums of vjp_pair_x2_sym left unused), every
 // later particle of the sample as a Newton pair with 32-j groups walked by skewed lanes.  Sums
 // (x-bar x, y, z, Qp) go to A.acc4 by float4 atomics; k_adj_pairs_finish applies them.
-template <int NT, int U, int MINB>
-__global__ void __launch_bounds__(NT, MINB) k_adj_pairs_sym(const AdjArgs A) {
+// (162 registers for grids of one CTA per SM, as the sums take, left 16 x 2,048 particles at 14.8 ms.)
+template <int NT, int U>
+__global__ void __launch_bounds__(NT, NT == 128 ? 3 : 6) k_adj_pairs_sym(const AdjArgs A) {
     constexpr int W = NT / 32, H = U / 2;
     static_assert(U % 2 == 0 && NT % 32 == 0, "packed pairs over whole warps");
     // staged j: (x,x,y,y), (z,z,Q,Q), (cx,cx,cy,cy), (cz,cz,-,-), each array at a 16-byte stride;
@@ -1391,8 +1392,7 @@ static int adjoint_impl(const pdq_field* field, const pdq_phys* phys, const pdq_
                 if (newton) {
                     PDQ_CUDA(cudaMemsetAsync(A.acc4, 0, acc_bytes, s));
                     k_adj_local<PDQ_MIXED><<<dim3((unsigned)((nmax + 127) / 128), (unsigned)A.S), 128, 0, s>>>(A);
-                    if ((int64_t)grid_vjp.x * grid_vjp.y <= sms) k_adj_pairs_sym<NTN, 4, 1><<<grid_vjp, NTN, 0, s>>>(A);
-                    else k_adj_pairs_sym<NTN, 4, 3><<<grid_vjp, NTN, 0, s>>>(A);
+                    k_adj_pairs_sym<NTN, 4><<<grid_vjp, NTN, 0, s>>>(A);
                     k_adj_pairs_finish<<<dim3((unsigned)((nmax + 255) / 256), (unsigned)A.S), 256, 0, s>>>(A);
                 } else if (mixed) {
                     k_adj_local<PDQ_MIXED><<<dim3((unsigned)((nmax + 127) / 128), (unsigned)A.S), 128, 0, s>>>(A);
