@@ -405,3 +405,47 @@ def test_adjoint_from_state_rejects_zero_charge_scale(pdq):
     cfg = pdq.step_cfg(c["dt"], window_start=c["win"], gravity=c["gravity"])
     with pytest.raises(pdq.PdqError):
         pdq.adjoint_run(field, phys, state, pdq.params_tensor(P), cfg, 10, 5, c["eps"])
+
+
+@pytest.mark.parametrize("store", [False, True])
+def test_mixed_adjoint_of_many_samples_close_to_fp64(pdq, store):
+    # more CTAs of the pair sums and of their VJP than the GPU has SMs (the kernels compiled for several per SM): 200 ragged
+    # samples, some empty or of one particle, against the FP64 adjoint; the MIXED bars of this file
+    rng = np.random.default_rng(0)
+    counts = [0, 1, 513, 1537] + [int(n) for n in rng.integers(100, 700, 196)]
+    prm = pdq.params_tensor(np.array([0.05, 0.5, 0.5]) * (0.5 + rng.random((200, 3))))
+    field, phys = pdq.Field(pdq.field_desc(**GRID), 0), pdq.phys_default()
+    cfg = pdq.step_cfg(TILE["dt"], window_start=TILE["win"], gravity=TILE["gravity"])
+    out = []
+    for precision in (0, 1):
+        batch = pdq.Batch(precision, counts, TILE["st"])
+        J, pbar = pdq.adjoint_run_seeded(field, phys, batch, prm, cfg, TILE["steps"], 5, 0.5, SEED,
+                                         gbar=_onehot_sc(200, 2), store_sums=store)
+        out.append((J.cpu().numpy(), np.transpose(pbar.cpu().numpy(), (1, 0, 2))))
+    (J0, g0), (J1, g1) = out
+    assert np.allclose(J1, J0, rtol=3e-3, atol=1e-6 * np.max(J0))
+    _check_grad(g1, g0, 3e-2, (0,))
+    assert np.all(J1[0] == 0) and np.all(g1[0] == 0)
+
+
+@pytest.mark.parametrize("store", [False, True])
+@pytest.mark.parametrize("steps,K", [(12, 12), (12, 5), (12, 6), (12, 1), (7, 20)])
+def test_mixed_reverse_takes_the_last_segment_it_finds(pdq, steps, K, store):
+    # as the FP64 test above, with MIXED's atomic Newton sums, kept or not, and two cotangents a call: reverse calls right
+    # after the forward sweep, after a reverse call and after a combined call in the same workspace; bar of the kept sums
+    field, phys = pdq.Field(pdq.field_desc(**GRID), 0), pdq.phys_default()
+    cfg = pdq.step_cfg(TILE["dt"], window_start=TILE["win"], gravity=TILE["gravity"])
+    prm = pdq.params_tensor(TILE_PARAMS)
+    batch = pdq.Batch(1, TILE_COUNTS, TILE["st"])
+    g = _onehot_sc(5, 2)
+
+    def combined(K, ws=None):
+        return pdq.adjoint_run_seeded(field, phys, batch, prm, cfg, steps, K, 0.5, SEED, gbar=g, ws=ws,
+                                      store_sums=ws is None and store)[1].cpu().numpy()
+    want = combined(3)
+    ws = pdq.adjoint_workspace(batch.b, steps, K, store_sums=store)
+    pdq.adjoint_run_seeded(field, phys, batch, prm, cfg, steps, K, 0.5, SEED, ws=ws)
+    got = [pdq.adjoint_reverse(field, phys, batch.b, prm, cfg, steps, K, 0.5, g, ws).cpu().numpy() for _ in range(2)]
+    got += [combined(K, ws), pdq.adjoint_reverse(field, phys, batch.b, prm, cfg, steps, K, 0.5, g, ws).cpu().numpy()]
+    for a in got:
+        assert np.max(np.abs(a - want)) <= 1e-3 * np.max(np.abs(want))
