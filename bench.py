@@ -92,9 +92,9 @@ def dist_env():
     return int(os.environ.get("RANK", 0)), int(os.environ.get("WORLD_SIZE", 1)), int(os.environ.get("LOCAL_RANK", 0))
 
 
-# FP64 Newton-pair runs sum the far pairs of samples of this many particles and more in float-float
-# (k_pairs_split64): ~135 FP32 operations per ordered pair for the 12 flops it counts
-SPLIT_MIN_PARTICLES, SPLIT_OPS_PER_PAIR = 8192, 135
+# FP64 Newton-pair runs sum the far pairs of large samples in float-float (k_pairs_split64): ~135 FP32
+# operations per ordered pair for the 12 flops it counts
+SPLIT_OPS_PER_PAIR = 135
 
 
 def pipe_peak(mixed, newton, split=False):
@@ -458,15 +458,8 @@ def run_ours(args):
         # min(compact_every, 10) steps, 10 without compaction; both precisions
         ci = min(cfg.compact_every, 10) if cfg.compact_every > 0 else 10
         n_rebin = sum(1 for k in range(args.steps - 1) if (s0 + k + 1) % ci == 0)
-        # sort, build_items, the step kernel(s) per step (Newton pairs, and FP64 tile pairs of up to 2,048
-        # particles: pair sums + update; FP64 Newton pairs sum large samples in a kernel of their own),
-        # re-bin + items
-        per_step = 2 if cfg.variant == 3 and (not args.contact or prec == pdq.MIXED) else 1
-        if prec == pdq.FP64 and not args.contact:
-            if cfg.variant == 3 and int(np.sum(counts)) >= SPLIT_MIN_PARTICLES:
-                per_step = 3
-            elif cfg.variant == 0 and cfg.block == 32 and 32 < int(np.sum(counts)) <= 2048:
-                per_step = 2
+        # sort, build_items, the step kernels per step, re-bin + items
+        per_step, far_split = pdq.step_kernels(state, cfg)
         launches = 1 + 1 + per_step * args.steps + 2 * n_rebin
 
         # e2e: state in pinned host memory; every step uploads the state, steps it and downloads the
@@ -517,7 +510,7 @@ def run_ours(args):
         return
     newton = cfg.variant == 3 and (not args.contact or prec == pdq.MIXED)
     flops_per_pair = NEWTON_FLOPS_PER_PAIR if newton else FLOPS_PER_PAIR
-    split = newton and prec == pdq.FP64 and int(np.max(counts)) >= SPLIT_MIN_PARTICLES
+    split = far_split
     peak_tflops, peak_note, mix = pipe_peak(prec == pdq.MIXED, newton, split)
     achieved = flops_per_pair * pairs / (ms / 1e3) / 1e12
     if mix is not None:

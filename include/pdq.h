@@ -253,6 +253,13 @@ typedef struct pdq_tally {
  * count).                                                                    */
 int pdq_step_workspace_size(const pdq_state* state, const pdq_step_cfg* cfg, size_t* bytes);
 
+/* Kernels that one step of pdq_step_particles launches for this state and
+ * configuration with a workspace of pdq_step_workspace_size (the z-binnings
+ * and work lists of a call come on top), and whether FP64 far pairs may run in
+ * pairs of floats (far_split may be NULL).  Host-only.
+ * Errors: INVALID_ARG.                                                       */
+int pdq_step_kernels(const pdq_state* state, const pdq_step_cfg* cfg, int32_t* per_step, int32_t* far_split);
+
 /* Advance all samples n_steps steps (App. A.2).  One step of particle i:
  *   a_i = sum_{j != i, same sample} k q_i q_j (x_i - x_j) / (m_i max(|x_i - x_j|, d_c)^3)
  *         (Eq. coulomb; minimum image in z; d_c = phys->contact_scale x the largest

@@ -2034,6 +2034,9 @@ static int launch_newton(const StepArgs& A, bool contact, cudaStream_t s) {
     return A.newton_u == 8 ? launch_newton_u<NT, 8, false>(A, s) : launch_newton_u<NT, 4, false>(A, s);
 }
 
+// FP64 one-sided runs summed by tile pairs (k_pairs_tiles64): 32 threads and a chunk for every tile.
+static bool tile_pairs(int NT, int JS, int64_t cap) { return NT == 32 && JS > 1 && (int64_t)JS * 32 >= cap; }
+
 // variant: MIXED pair math, 0 = all packed f32x2, 1 = packed with scalar accumulation,
 // 2 = as 0 with 8 particles per thread, 3 = Newton pairs (A.acc4 set: k_pairs_sym, then the
 // given-sums step, or with contact the contact variant that takes the sums).
@@ -2077,7 +2080,7 @@ static int dispatch_step(int prec, int NT, int variant, bool contact, const Step
         return PDQ_ERR_INVALID_ARG;
     }
     if (prec == PDQ_FP64) {
-        if (NT == 32 && A.jsplit > 1 && (int64_t)A.jsplit * 32 >= A.cap) {
+        if (tile_pairs(NT, A.jsplit, A.cap)) {
             if (A.K.forces & PDQ_F_COULOMB) k_pairs_tiles64<<<dim3((unsigned)(A.max_items / A.jsplit), (unsigned)(A.jsplit / 2 + 1)), 32 * kTileWarps, 0, s>>>(A);
             k_update_tiles64<<<(unsigned)(A.max_items / A.jsplit * (32 / kTilePart)), 32, 0, s>>>(A);
             return PDQ_OK;
@@ -2112,7 +2115,9 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 static int j_split(const pdq_state* st, int TI, bool contact = false, bool coarse = false) {
     if (st->precision != PDQ_FP64 || contact) return 1;
     const int64_t cap = st->capacity > 0 ? st->capacity : 1;
-    // up to 2,048 particles at 32 threads: one tile per chunk, summed by tile pairs (k_pairs_tiles64)
+    // up to 2,048 particles at 32 threads: one tile per chunk, summed by tile pairs (k_pairs_tiles64).  2,048 in all, since
+    // the partial sums hold a row of `capacity` per chunk and chunks end at 64 (3 MB there; by the largest sample's
+    // tiles several samples would fit, but the host knows no sample's size)
     if (TI == 32 && cap <= 2048 && !coarse) return (int)((cap + 31) / 32);
     const int64_t tile_warps = (cap + TI - 1) / TI * ((TI + 31) / 32);
     int64_t js = (1024 + tile_warps - 1) / tile_warps;
@@ -2285,6 +2290,20 @@ extern "C" int pdq_step_workspace_size(const pdq_state* st, const pdq_step_cfg* 
     workspace_layout(st, tile_threads(st, cfg) * std::min(tile_ilp(st, cfg), 4), &ib, &tot, nullptr, nullptr,
                      cfg && (cfg->forces & PDQ_F_CONTACT), nullptr, newton_pairs(st, cfg));
     *bytes = tot;
+    return PDQ_OK;
+}
+
+extern "C" int pdq_step_kernels(const pdq_state* st, const pdq_step_cfg* cfg, int32_t* per_step, int32_t* far_split) {
+    if (!cfg || !per_step) return PDQ_ERR_INVALID_ARG;
+    int rc = validate_state(st);
+    if (rc) return rc;
+    const bool coulomb = cfg->forces & PDQ_F_COULOMB, contact = cfg->forces & PDQ_F_CONTACT;
+    const bool f64 = st->precision == PDQ_FP64, newton = newton_pairs(st, cfg);
+    const bool split = newton && f64 && coulomb && st->capacity >= kSplitMin;
+    const int NT = tile_threads(st, cfg);
+    const bool tiles = f64 && !newton && !contact && tile_pairs(NT, j_split(st, NT), st->capacity);
+    *per_step = 1 + (coulomb && (newton || tiles)) + (split ? 2 : 0);
+    if (far_split) *far_split = split;
     return PDQ_OK;
 }
 

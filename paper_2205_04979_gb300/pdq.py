@@ -98,6 +98,8 @@ def lib():
                                                          C.POINTER(StateStruct), P]),
             "pdq_step_workspace_size": (C.c_int, [C.POINTER(StateStruct), C.POINTER(StepCfg),
                                                   C.POINTER(C.c_size_t)]),
+            "pdq_step_kernels": (C.c_int, [C.POINTER(StateStruct), C.POINTER(StepCfg), C.POINTER(C.c_int32),
+                                           C.POINTER(C.c_int32)]),
             "pdq_step_particles": (C.c_int, [P, C.POINTER(Phys), C.POINTER(StateStruct), P, C.POINTER(StepCfg),
                                              C.c_int64, C.POINTER(TallyStruct), P, C.c_size_t, P]),
             "pdq_step_particles_noalloc": (C.c_int, [P, C.POINTER(Phys), C.POINTER(StateStruct), P,
@@ -371,6 +373,13 @@ def workspace(state, cfg):
     n = C.c_size_t()
     _check(lib().pdq_step_workspace_size(C.byref(state.st), C.byref(cfg), C.byref(n)), "step_workspace_size")
     return torch.empty(max(int(n.value), 256), dtype=torch.uint8, device="cuda")
+
+
+def step_kernels(state, cfg):
+    """(kernels one step launches, whether FP64 far pairs may run in float-float) for this state and cfg."""
+    n, split = C.c_int32(), C.c_int32()
+    _check(lib().pdq_step_kernels(C.byref(state.st), C.byref(cfg), C.byref(n), C.byref(split)), "step_kernels")
+    return n.value, bool(split.value)
 
 
 def step_particles(field, phys, state, params_dev, cfg, n_steps, tally, ws, stream=None):

@@ -209,3 +209,25 @@ def test_low_fidelity_defaults_and_arguments_rejected_on_host(pdq):
     assert L.pdq_lf_fluid_variance(None, None, None) == -1
     assert L.pdq_lf_vdep(None, C.byref(p), C.byref(d), None, 1, C.cast(st, C.c_void_p), 1, None, None, None) == -1
     assert L.pdq_lf_vdep(None, C.byref(p), None, None, 1, C.cast(st, C.c_void_p), 0, None, None, None) == -1
+
+
+def test_step_kernels_by_precision_variant_and_size(pdq):
+    # pair sums and update; FP64 Newton pairs from 32,768 slots on: the choice and the float-float kernel too; tile pairs of
+    # 33 to 2,048 FP64 particles at 32 threads; the pair kernels only with the Coulomb force
+    s = _fake_mixed_state(pdq, 50000)
+
+    def count(precision, capacity, **kw):
+        s.precision, s.capacity = precision, capacity
+        n, split = C.c_int32(), C.c_int32()
+        assert pdq.lib().pdq_step_kernels(C.byref(s), C.byref(pdq.step_cfg(0.1, **kw)), C.byref(n), C.byref(split)) == 0
+        return n.value, split.value
+    for v in (0, 1, 2):
+        assert count(1, 50000, variant=v) == (1, 0)
+    assert count(1, 50000, variant=3) == (2, 0)
+    assert count(1, 50000, variant=3, forces=pdq.F_ALL | pdq.F_CONTACT) == (2, 0)
+    assert count(0, 32767, variant=3, block=64) == (2, 0) and count(0, 32768, variant=3, block=64) == (4, 1)
+    assert count(0, 32768, variant=3, block=64, forces=pdq.F_DRAG) == (1, 0)
+    assert count(0, 50000, variant=3, forces=pdq.F_ALL | pdq.F_CONTACT) == (1, 0)
+    assert [count(0, n, block=32)[0] for n in (32, 33, 2048, 2049)] == [1, 2, 2, 1]
+    assert count(0, 1000, block=64) == (1, 0) and count(0, 1000, block=32, forces=pdq.F_DRAG) == (1, 0)
+    assert pdq.lib().pdq_step_kernels(C.byref(s), None, None, None) == -1
