@@ -977,9 +977,9 @@ def run_p3m(args):
 # one each), cell means and exponential fitting vm, a', expm1, G = em/vm, E (6), Q += P G, P *= E (3)
 LF_FLOPS_PER_CELL = 23
 # FP64-pipe lane operations per (item, cell) as executed (ncu on a launch of 16,384 samples x 10
-# classes, pipe 82.4 % busy: the square root, divisions and expm1 expand to seeds plus correction or
+# classes, pipe 82.7 % busy: the momentum root and (e^x - 1)/x expand to estimates plus correction or
 # polynomial steps), and the DRAM bytes (read + write) of a 65,536-sample launch, scaled by samples
-LF_FP64_OPS_PER_CELL = 46.4
+LF_FP64_OPS_PER_CELL = 42.0
 LF_DRAM_BYTES_PER_SAMPLE = 2.172e6 / 65536
 # the FP32 march: (what bounds it, thread instructions per (item, cell) as executed (ncu, 65,536
 # samples; a packed instruction serves two items), the measured rate it is compared with): every instruction takes an issue slot, and the issue

@@ -231,7 +231,9 @@ typedef struct pdq_step_cfg {
                           /*   (Eq. coulomb is odd in x_i - x_j), summed through atomics     */
                           /*   (float for MIXED, double for PDQ_FP64; not bit-reproducible   */
                           /*   from run to run), then the local update; block 64 or 128      */
-                          /*   only.  MIXED contact runs take the Coulomb sums this way and  */
+                          /*   only.  PDQ_FP64 samples whose far pairs run in floats (see      */
+                          /*   pdq_step_particles) are summed from each side on its own.      */
+                          /*    MIXED contact runs take the Coulomb sums this way and  */
                           /*   keep the contact forces one-sided; PDQ_FP64 contact runs      */
                           /*   ignore it.  For PDQ_FP64 the only other value read is 0       */
 } pdq_step_cfg;
@@ -345,6 +347,10 @@ int pdq_step_particles_noalloc(const pdq_field* field, const pdq_phys* phys, pdq
  * reordered and compacted, as pdq_step_particles does at the start of a call).
  * Results are cached per (precision, log2 capacity, log2 samples, forces);
  * a cached entry costs no device work.  Synchronises `stream`.
+ * The choice decides whether results repeat bit for bit: pair variants 0, 1
+ * and 2 add in a fixed order, variant 3 (the fastest from a few thousand
+ * MIXED particles on, and for large FP64 samples) by atomics in any order.  A
+ * caller that needs the same bits on every run sets block and variant itself.
  * Errors: INVALID_ARG, WORKSPACE, CUDA.                                      */
 int pdq_autotune_workspace_size(const pdq_state* state, size_t* bytes);
 int pdq_autotune(const pdq_field* field, const pdq_phys* phys, pdq_state* state, const pdq_sample_params* params,
@@ -613,9 +619,11 @@ int pdq_lf_vdep(const pdq_field* field, const pdq_phys* phys, const pdq_lf_desc*
  * in pairs of floats, off by 2^-48 of d/r^3: the sums are within 1e-15 of the
  * method's in the median.  With alpha h = 0.5 and r_cut = 3.3/alpha the
  * RMS relative error against the exact periodic sum is ~1.4e-4.
- * A plan owns its device memory (kernel transforms, meshes, cell list; about
- * 40 Nx^2 Nz bytes, plus a [capacity][3] FP64 buffer that
- * pdq_step_particles_p3m allocates the first time it meets a state that large).  Pick M with 2(M + 5) a product of small primes (123,
+ * A plan owns its device memory (kernel transforms and meshes about
+ * 56 Nx^2 Nz bytes, the transforms' work areas, 84 bytes per particle of
+ * max_particles, cell tables of up to 2.4 MB at M = 123; plus a [capacity][3] FP64 buffer that
+ * pdq_step_particles_p3m allocates the first time it meets a state that large).
+ * Pick M with 2(M + 5) a product of small primes (123,
  * 251) for fast transforms.                                                  */
 typedef struct pdq_p3m_desc {
     int32_t M;        /* mesh cells across the diameter, >= 4                          */

@@ -1060,7 +1060,7 @@ constexpr int kSplitMin = 32768, kProbes = 128;
 
 // Probe blockIdx.x of the samples blockIdx.y, blockIdx.y + gridDim.y, ...: its sum and its far terms (FP32 does),
 // tallied per sample; the last probe of a sample decides.  kProbes CTAs read the sample's positions from L2 once
-// each: ~0.04 ms at 100,000 particles.
+// each: 0.09 ms at 32,768 particles, 0.26 ms at 100,000 (1.1 and 0.4 % of the step).
 __global__ void __launch_bounds__(256) k_split_choose(const StepArgs A) {
     __shared__ float s_red[8][4 + 2 * kSplitTries];
     const StepConst& K = A.K;
