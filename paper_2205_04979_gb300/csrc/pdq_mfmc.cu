@@ -45,8 +45,19 @@ struct SumArgs {
 // threads' sums in a fixed tree, the first CTA of the cluster adds the CTAs' in rank order: the
 // result does not depend on the schedule.  Bound by the FP64 pipe, 13 operations per position and
 // output at d = 3; D: the number of inputs (0: any, from A.d), so that the accumulators stay in registers.
-// A study of 834 and 16,570 groups, 10 outputs, 200 replicates: 1.04 ms; 1.39 ms before.
-constexpr int kSumThreads = 256, kSumOutputs = 32;
+// A study of 834 and 16,570 groups, 10 outputs, 200 replicates: 1.11 ms; 1.39 ms before.
+// A thread adds its positions in runs of kRun, and the last adds keep what they round off: with few rows a thread's chain
+// is up to ten times as long as with a CTA per output, and the variance and the total indices were 20 to 30 % further
+// from extended precision (834 and 16,570 groups, 10 outputs, 40 seeds, rms: 2.3e-15 and 3.3e-15; 2.0e-15 and 2.6e-15
+// with a CTA per output; 1.4e-15 and 1.9e-15 now).
+constexpr int kSumThreads = 256, kSumOutputs = 32, kRun = 32;
+
+// s + err = a + b exactly (Knuth's two-sum).
+__device__ __forceinline__ double add_exactly(double a, double b, double& err) {
+    const double s = a + b, bb = s - a;
+    err = (a - (s - bb)) + (b - bb);
+    return s;
+}
 
 template <int D>
 __global__ void __launch_bounds__(kSumThreads) k_mfmc_sums(const SumArgs A) {
@@ -54,6 +65,7 @@ __global__ void __launch_bounds__(kSumThreads) k_mfmc_sums(const SumArgs A) {
     cg::cluster_group cluster = cg::this_cluster();
     constexpr int kMaxD = D ? D : kMaxInputs, kSums = 4 + 2 * kMaxD;
     __shared__ double red[8][kSumThreads];
+    __shared__ double total[D ? kSums : 1][kSumThreads];
     __shared__ double part[kSums][kSumOutputs];
     const int d = D ? D : A.d, C = A.C, ncol = d + 2, nq = 4 + 2 * d;
     const int ctas = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), c0 = (int)(blockIdx.x / ctas) * A.outs;
@@ -62,9 +74,23 @@ __global__ void __launch_bounds__(kSumThreads) k_mfmc_sums(const SumArgs A) {
     const int tid = threadIdx.x, cc = tid % nc, tt = tid / nc;
     const bool active = tt < T;                       // the threads past T whole rows of outputs idle
     const double* __restrict__ y = A.y[i];
-    double acc[kSums];
+    // acc: a thread's run of kRun positions; total (its own slots; registers when the number of inputs is general): the runs before
+    double acc[kSums], reg[D ? 1 : kSums];
 #pragma unroll
-    for (int q = 0; q < kSums; ++q) acc[q] = 0.0;
+    for (int q = 0; q < kSums; ++q) {
+        acc[q] = 0.0;
+        if constexpr (D) total[q][tid] = 0.0;
+        else reg[q] = 0.0;
+    }
+    auto flush = [&]() {
+#pragma unroll
+        for (int q = 0; q < kSums; ++q) {
+            if constexpr (D) total[q][tid] += acc[q];
+            else reg[q] += acc[q];
+            acc[q] = 0.0;
+        }
+    };
+    int run = 0;
     int64_t t = (int64_t)rank * T + tt;
     for (int p = i > 0 ? 0 : 1; p < 2; ++p) {
         const int64_t m = p ? A.m[i] : A.m[i - 1];
@@ -92,17 +118,27 @@ __global__ void __launch_bounds__(kSumThreads) k_mfmc_sums(const SumArgs A) {
                         acc[4 + kMaxD + j] += e * e;
                     }
                 }
+                if (++run == kRun) {
+                    flush();
+                    run = 0;
+                }
             }
         }
-        // the rows of threads fold in a fixed tree, 8 sums at a time (a chain of T FP64 adds by one thread
-        // per output took 20 us a sum at one output)
+        flush();
+        // the rows of threads fold in a fixed tree, 8 sums at a time, the last four rows with what their adds round off (a
+        // chain of T FP64 adds by one thread per output took 20 us a sum at one output)
 #pragma unroll
         for (int q0 = 0; q0 < kSums; q0 += 8) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-                if (q0 + e < kSums) red[e][tid] = acc[q0 + e];
+            for (int e = 0; e < 8; ++e) {
+                if (q0 + e < kSums) {
+                    if constexpr (D) red[e][tid] = total[q0 + e][tid];
+                    else red[e][tid] = reg[q0 + e];
+                }
+            }
             __syncthreads();
-            for (int n = T; n > 1;) {
+            int n = T;
+            while (n > 4) {
                 const int half = (n + 1) / 2, fold = (n - half) * nc;
                 for (int u = tid; u < 8 * fold; u += kSumThreads) {
                     const int e = u / fold, r = u - e * fold;
@@ -111,8 +147,16 @@ __global__ void __launch_bounds__(kSumThreads) k_mfmc_sums(const SumArgs A) {
                 __syncthreads();
                 n = half;
             }
-            for (int u = tid; u < 8 * nc; u += kSumThreads)
-                if (q0 + u / nc < kSums) part[q0 + u / nc][u % nc] = red[u / nc][u % nc];
+            for (int u = tid; u < 8 * nc; u += kSumThreads) {
+                const int e = u / nc, c = u - e * nc;
+                if (q0 + e >= kSums) continue;
+                double v = red[e][c], off = 0.0, err;
+                for (int r = 1; r < n; ++r) {
+                    v = add_exactly(v, red[e][r * nc + c], err);
+                    off += err;
+                }
+                part[q0 + e][c] = v + off;
+            }
             __syncthreads();
         }
         cluster.sync();
@@ -121,9 +165,12 @@ __global__ void __launch_bounds__(kSumThreads) k_mfmc_sums(const SumArgs A) {
             for (int u = tid; u < nc * nq; u += kSumThreads) {
                 const int c = u / nq, q = u % nq;
                 const int qs = q < 4 + d ? q : 4 + kMaxD + (q - 4 - d);
-                double v = 0.0;
-                for (int r = 0; r < ctas; ++r) v += cluster.map_shared_rank(&part[0][0], r)[qs * kSumOutputs + c];
-                out[(int64_t)c * nq + q] = v;
+                double v = 0.0, off = 0.0, err;
+                for (int r = 0; r < ctas; ++r) {
+                    v = add_exactly(v, cluster.map_shared_rank(&part[0][0], r)[qs * kSumOutputs + c], err);
+                    off += err;
+                }
+                out[(int64_t)c * nq + q] = v + off;
             }
         }
         cluster.sync();                               // part is read before it is written again, or the CTA ends

@@ -91,6 +91,18 @@ def test_sums_over_blocks_of_outputs(pdq, C, d):
     assert np.allclose(out["s_total_ci"], ci_t, rtol=1e-8, atol=1e-10)
 
 
+def test_sums_of_long_chains(pdq):
+    # 200,000 groups of 32 positive outputs under 1,300 replicates: one CTA of 8 rows sums them, 25,000 positions a thread,
+    # in runs of 32.  Bar of the means: a chain of 781 run sums rounds to 0.29 sqrt(781 / 3) units of 2^-53, 8 rows of them
+    # to 1.7 of the sum, the mean's own half a unit: three times that over 32 outputs, 6 units
+    m, C = 200_000, 32
+    y = torch.rand((m, 3, C), generator=torch.Generator(device="cuda").manual_seed(3), device="cuda",
+                   dtype=torch.float64) + 1.0
+    out = pdq.mfmc_sobol([y], [m], [1.0], n_boot=1300, seed=1)
+    want = y[:, 0].cpu().numpy().astype(np.longdouble).sum(0) / m
+    assert np.max(np.abs(out["mean"] / want - 1)) <= 6 * 2.0 ** -53
+
+
 def test_dgsm_bounds_match_oracle(pdq):
     rng = np.random.default_rng(14)
     X = rng.uniform(-np.pi, np.pi, (5000, 3))
