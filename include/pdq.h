@@ -231,11 +231,11 @@ typedef struct pdq_step_cfg {
                           /*   (Eq. coulomb is odd in x_i - x_j), summed through atomics     */
                           /*   (float for MIXED, double for PDQ_FP64; not bit-reproducible   */
                           /*   from run to run), then the local update; block 64 or 128      */
-                          /*   only.  PDQ_FP64 samples whose far pairs run in floats (see      */
-                          /*   pdq_step_particles) are summed from each side on its own.      */
-                          /*    MIXED contact runs take the Coulomb sums this way and  */
-                          /*   keep the contact forces one-sided; PDQ_FP64 contact runs      */
-                          /*   ignore it.  For PDQ_FP64 the only other value read is 0       */
+                          /*   only.  PDQ_FP64 samples whose far pairs run in floats (see    */
+                          /*   pdq_step_particles) are summed from each side on its own.     */
+                          /*   MIXED contact runs take the Coulomb sums this way and keep    */
+                          /*   the contact forces one-sided; PDQ_FP64 contact runs ignore    */
+                          /*   it.  For PDQ_FP64 the only other value read is 0              */
 } pdq_step_cfg;
 
 /* Caller-owned tallies, device int64 [S][C], accumulated across calls:
@@ -621,9 +621,9 @@ int pdq_lf_vdep(const pdq_field* field, const pdq_phys* phys, const pdq_lf_desc*
  * RMS relative error against the exact periodic sum is ~1.4e-4.
  * A plan owns its device memory (kernel transforms and meshes about
  * 56 Nx^2 Nz bytes, the transforms' work areas, 84 bytes per particle of
- * max_particles, cell tables of up to 2.4 MB at M = 123; plus a [capacity][3] FP64 buffer that
- * pdq_step_particles_p3m allocates the first time it meets a state that large).
- * Pick M with 2(M + 5) a product of small primes (123,
+ * max_particles, cell tables of 2.4 MB at M = 123, and a [capacity][3] FP64
+ * buffer that pdq_step_particles_p3m allocates the first time it meets a
+ * state that large).  Pick M with 2(M + 5) a product of small primes (123,
  * 251) for fast transforms.                                                  */
 typedef struct pdq_p3m_desc {
     int32_t M;        /* mesh cells across the diameter, >= 4                          */
