@@ -34,6 +34,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
+
 #include "pdq_device.cuh"
 #include "pdq_lf_math.cuh"
 
@@ -365,6 +367,10 @@ static int launch_lf(void (*kernel)(LfArgs), int threads, int per, size_t elem, 
     const int64_t nblk = (A.S + per - 1) / per;
     int64_t gx = (int64_t)(sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1) / A.C;
     if (gx < 1) gx = 1;
+    // one CTA per SM while its warps take all the runs: a second one builds a table of its own on the same FP64 pipe
+    // (FP32, 2,048 nodes, 2,500 samples of 10 classes: 396 us, 494 us with two; one march per class and SM 377 us)
+    const int64_t one = std::max<int64_t>(1, sms / A.C);
+    if (nblk <= one * (threads / 32)) gx = std::min(gx, one);
     if (gx > nblk) gx = nblk;
     const dim3 grid((unsigned)gx, (unsigned)A.C);
     kernel<<<grid, threads, smem, (cudaStream_t)stream>>>(A);
