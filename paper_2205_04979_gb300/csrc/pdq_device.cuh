@@ -153,18 +153,6 @@ __device__ __forceinline__ double rcp_seed(double x) {
     return r;
 }
 
-// r2^(-3/2) in FP64 for a normal, finite r2 > 0: y = rsqrt_seed(r2) and the binomial series of
-// (1 - d)^(-3/2) in d = 1 - r2 y^2 (below 2^-18), to d^3 (the next term is 2.5 d^4 < 2^-70): 7 FP64 operations,
-// against ~10 for the library's reciprocal square root (with its branch for special values) and the two products.
-__device__ __forceinline__ double inv_cube64(double r2) {
-    const double y = rsqrt_seed(r2);
-    const double t = y * y;
-    const double d = __fma_rn(-r2, t, 1.0);
-    const double c = d * __fma_rn(d, __fma_rn(d, 2.1875, 1.875), 1.5);
-    const double y3 = y * t;
-    return __fma_rn(y3, c, y3);
-}
-
 __device__ __forceinline__ void coulomb_pair(float xi, float yi, float zi, const float4 pj, float L, float invL,
                                              float c2, float& ax, float& ay, float& az) {
     const float dx = xi - pj.x, dy = yi - pj.y;
@@ -185,7 +173,8 @@ __device__ __forceinline__ void coulomb_pair(double xi, double yi, double zi, co
     const double t = __dadd_rn(__fma_rn(dz, invL, 6755399441055744.0), -6755399441055744.0);
     dz = __fma_rn(-L, t, dz);
     const double r2 = fmax(__fma_rn(dx, dx, __fma_rn(dy, dy, dz * dz)), c2);
-    const double s = pj.w * inv_cube64(r2);
+    const double ri = rsqrt(r2);
+    const double s = pj.w * ri * (ri * ri);
     ax = __fma_rn(s, dx, ax);
     ay = __fma_rn(s, dy, ay);
     az = __fma_rn(s, dz, az);

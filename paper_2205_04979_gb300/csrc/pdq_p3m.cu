@@ -411,7 +411,8 @@ __device__ __forceinline__ double pp_close(const PPConst& K, double r2) {
         const double x = sqrt(u);
         kl = a3 * (erf(x) / (u * x) - c * exp(-u) / u);
     }
-    return inv_cube64(fmax(r2, K.dc2)) - kl;
+    const double ic = rsqrt(fmax(r2, K.dc2));             // 1 / max(r, d_c)
+    return ic * (ic * ic) - kl;
 }
 
 // One short-range pair: q_j (d / max(r, d_c)^3 - K_L(d)) when r < r_cut, in FP64 (17 operations).

@@ -536,7 +536,8 @@ __device__ __forceinline__ void coulomb_pair_direct64(double xi, double yi, doub
     const double dx = xi - pj.x, dy = yi - pj.y, dz = zi - pj.z;
     double r2 = __fma_rn(dx, dx, __fma_rn(dy, dy, dz * dz));
     if constexpr (CLAMP) r2 = fmax(r2, c2);
-    const double s = pj.w * inv_cube64(r2);
+    const double ri = rsqrt(r2);
+    const double s = pj.w * ri * (ri * ri);
     ax = __fma_rn(s, dx, ax);
     ay = __fma_rn(s, dy, ay);
     az = __fma_rn(s, dz, az);
@@ -555,7 +556,8 @@ __device__ __forceinline__ void coulomb_pair_track(double xi, double yi, double 
     const double r2u = __fma_rn(dx, dx, __fma_rn(dy, dy, dz * dz));
     mnh = min(mnh, __double2hiint(r2u));
     const double r2 = fmax(r2u, c2);
-    const double s = pj.w * inv_cube64(r2);
+    const double ri = rsqrt(r2);
+    const double s = pj.w * ri * (ri * ri);
     ax = __fma_rn(s, dx, ax);
     ay = __fma_rn(s, dy, ay);
     az = __fma_rn(s, dz, az);
@@ -1150,7 +1152,8 @@ __device__ __forceinline__ void coulomb_pair_sym64(double xi, double yi, double 
     }
     double r2 = __fma_rn(dx, dx, __fma_rn(dy, dy, dz * dz));
     if constexpr (CLAMP) r2 = fmax(r2, c2);
-    const double ri3 = inv_cube64(r2);
+    const double ri = rsqrt(r2);
+    const double ri3 = ri * (ri * ri);
     const double si = zqj.y * ri3, sj = nqi * ri3;
     ax = __fma_rn(si, dx, ax);
     ay = __fma_rn(si, dy, ay);

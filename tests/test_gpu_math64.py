@@ -30,7 +30,7 @@ def _both(lib, x, a):
     """out[k, 0] ours and out[k, 1] CUDA's, k as in math64_check.cu."""
     n = len(x)
     xs, av = torch.tensor(x, device="cuda"), torch.tensor(a, device="cuda")
-    out = torch.empty((6, 2, n), dtype=torch.float64, device="cuda")
+    out = torch.empty((5, 2, n), dtype=torch.float64, device="cuda")
     p = ctypes.c_void_p
     assert lib.check_math(p(xs.data_ptr()), p(av.data_ptr()), n, p(out.data_ptr())) == 0
     torch.cuda.synchronize()
@@ -41,15 +41,13 @@ def _units(o, k):
     return float(np.max(np.abs(o[k, 0] / o[k, 1] - 1))) * 2.0 ** 53
 
 
-def test_estimates_and_inverse_cube(lib):
+def test_estimates(lib):
     # arguments over 2^-80 .. 2^80, the mantissas at random and at both ends of the 20 bits that the estimates see
     rng = np.random.default_rng(1)
     m = np.r_[1 + rng.random(200000), 1 + np.arange(4096) / 4096, np.nextafter(1 + np.arange(1, 4097) / 4096, 0)]
     x = m * 2.0 ** rng.integers(-80, 81, m.size)
     o = _both(lib, x, np.ones_like(x))
     assert _units(o, 0) <= 2.0 ** (53 - 19) and _units(o, 1) <= 2.0 ** (53 - 19)
-    # ours: t half a unit, y3 and the result one each; CUDA's root, product and quotient one each
-    assert _units(o, 2) <= 6
 
 
 def test_root_of_the_momentum_equation(lib):
@@ -57,7 +55,7 @@ def test_root_of_the_momentum_equation(lib):
     # u/2 + a, 1 of the result, 2^-55 truncation; the closed form: half of a^2 + 2c's, 1 each of root, sum and quotient
     rng = np.random.default_rng(2)
     a, c = 10.0 ** rng.uniform(-8, 4, 400000), 10.0 ** rng.uniform(-20, 6, 400000)
-    assert _units(_both(lib, c, a), 3) <= 6
+    assert _units(_both(lib, c, a), 2) <= 6
 
 
 def test_exponential_quotient(lib):
@@ -68,4 +66,4 @@ def test_exponential_quotient(lib):
     x = np.r_[10.0 ** rng.uniform(-12, np.log10(40), 400000), rng.uniform(0.01, 0.6, 100000), ends,
               np.nextafter(ends, 0), np.nextafter(ends, 1)]
     o = _both(lib, x, np.ones_like(x))
-    assert _units(o, 4) <= 7 and _units(o, 5) <= 4
+    assert _units(o, 3) <= 7 and _units(o, 4) <= 4
