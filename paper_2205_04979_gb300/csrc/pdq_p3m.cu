@@ -66,7 +66,7 @@ struct P3MGeom {
 // The short-range pairs read K_S's factor 1/r^3 - K_L from polynomials in r^2, in place of the reciprocal square root, K_L
 // and their difference; both tables fit shared memory beside the queues.
 // Inner pairs, r < r_n: sextics in FP64 on kOct octaves of 64 intervals each that end at the first power of two from
-// r_n^2 on.  Through 7 Chebyshev nodes (h/(4 r^2))^7 <= 2^-56 of a power law remains; where the factor falls off
+// r_n^2 on.  Through 7 Chebyshev nodes 6.3 (h/(4 r^2))^7 <= 2^-53 of r^-3 remains; where the factor falls off
 // faster it is small against 1/r^3, which is what its error matters against.  Closer pairs (below r_n/16, or
 // inside the contact distance) take pp_close.
 // Outer pairs, r_n = r_cut/2 <= r: quintics on kFar intervals, in float-float down to t^2; t^3 carries 7e-7 of the value,
@@ -394,7 +394,7 @@ struct PPConst {
 };
 
 // 1 / max(r, d_c)^3 - K_L factor at the close pairs: K_L by c alpha^3 sum_m (-1)^m 2 u^m / (m! (2m + 3)), u = (alpha r)^2, to
-// m = 17 below u = 1 (where the closed form cancels; the next term is 2^-57), by the closed form above.
+// m = 17 below u = 1 (where the closed form cancels; the next term is below 2^-56), by the closed form above.
 __device__ __forceinline__ double pp_close(const PPConst& K, double r2) {
     const double c = 1.1283791670955126, u = K.alpha * K.alpha * r2, a3 = K.alpha * K.alpha * K.alpha;
     double kl;
